@@ -418,7 +418,7 @@ int pack_ensemble(const mlt_node* nodes, int n_trees, int depth, int F, std::vec
         else
           inherit[j] = 0.0f;
         if (j < inner) {
-          thr_of[j] = split ? nd.value : 0.0f;
+          thr_of[j] = split ? std::nextafterf(nd.value, -INFINITY) : 0.0f;  // prev(t)
           meta_of[j] = split ? (static_cast<uint32_t>(nd.feature) | (nd.default_left ? kMetaDefaultLeft : 0u)) : 0u;
         }
       }

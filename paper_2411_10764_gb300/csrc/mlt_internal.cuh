@@ -31,8 +31,9 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 // ---------------------------------------------------------------------------
 // Full table (depth D <= kMaxFullDepth): every tree is stored as a complete
 // binary tree of depth D, `tree_bytes` apart (a multiple of 16).  A node has
-// a threshold (float), a feature index (< kMaxF) and a NaN-goes-left flag;
-// its heap index is j (children 2j+1, 2j+2).  Each level is laid out for the
+// the float just below its threshold (prev(t): x >= t is the sign of
+// prev(t) - x), a feature index (< kMaxF) and a NaN-goes-left flag; its heap
+// index is j (children 2j+1, 2j+2).  Each level is laid out for the
 // way a warp reads it (FullLayout below):
 //   levels [0, top)  : 8-byte records {threshold, meta} with meta = feature
 //                      | flag << 31 -- few distinct nodes, mostly broadcast

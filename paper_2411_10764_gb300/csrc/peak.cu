@@ -33,8 +33,8 @@ __global__ void __launch_bounds__(kFullMaxTile)
   const unsigned char* xcol = reinterpret_cast<const unsigned char*>(xs) + static_cast<uint32_t>(tid) * 4u;
   float acc = 0.0f;
   for (int r = 0; r < rounds; ++r)
-    acc = nan ? walk_chunk<D, G, true, 1>(tbuf, 0, resident, a.tree_bytes, xcol, row_bytes, acc, 0u)
-              : walk_chunk<D, G, false, 1>(tbuf, 0, resident, a.tree_bytes, xcol, row_bytes, acc, 0u);
+    acc = nan ? walk_chunk<D, G, true, 1>(tbuf, 0, resident, xcol, row_bytes, acc, 0u)
+              : walk_chunk<D, G, false, 1>(tbuf, 0, resident, xcol, row_bytes, acc, 0u);
   if (tid < rows_here) out[tile0 + tid] = acc;
 }
 

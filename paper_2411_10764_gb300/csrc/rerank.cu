@@ -27,7 +27,8 @@ __device__ __forceinline__ uint32_t go_right_nan(float x, uint32_t thr_bits, uin
   return right;
 }
 
-// One tree of a full table, read from global memory (FullLayout).
+// One tree of a full table, read from global memory (FullLayout; its
+// thresholds are stored as prev(t), so x >= t reads x > prev(t)).
 __device__ float leaf_full(const unsigned char* tree, int D, const float* x) {
   const FullLayout L = full_layout(D);
   uint32_t j = 0;
@@ -43,7 +44,8 @@ __device__ float leaf_full(const unsigned char* tree, int D, const float* x) {
       thr = __ldg(reinterpret_cast<const uint32_t*>(tree + L.off_thr) + (j - L.n_top));
     }
     const float xv = __ldg(x + (meta & ~kMetaDefaultLeft));
-    j = 2u * j + 1u + go_right_nan(xv, thr, meta);
+    const bool right = xv != xv ? !(meta & kMetaDefaultLeft) : xv > __uint_as_float(thr);
+    j = 2u * j + 1u + (right ? 1u : 0u);
   }
   return __ldg(reinterpret_cast<const float*>(tree + L.off_leaf) + (j - L.n_inner));
 }

@@ -245,8 +245,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_screen_small(const __grid_con
     const uint32_t row_bytes = static_cast<uint32_t>(TC) * 4u;
     const unsigned char* xcol = reinterpret_cast<const unsigned char*>(xs) + static_cast<uint32_t>(c) * 4u;
     const uint32_t la = smem_u32(park) + static_cast<uint32_t>(c) * 4u;
-    accv = nan ? walk_chunk<D, G, true, Q>(vt, q, s.v_trees, s.tree_bytes, xcol, row_bytes, 0.0f, la)
-               : walk_chunk<D, G, false, Q>(vt, q, s.v_trees, s.tree_bytes, xcol, row_bytes, 0.0f, la);
+    accv = nan ? walk_chunk<D, G, true, Q>(vt, q, s.v_trees, xcol, row_bytes, 0.0f, la)
+               : walk_chunk<D, G, false, Q>(vt, q, s.v_trees, xcol, row_bytes, 0.0f, la);
     if (Q > 1) {
       __syncthreads();
       if (q == 0)
@@ -255,8 +255,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_screen_small(const __grid_con
     }
     failed = !__syncthreads_and(mbar_wait_bounded(smem_u32(&bars[2]), 0u));
     if (!failed) {
-      accp = nan ? walk_chunk<D, G, true, Q>(pt, q, s.p_trees, s.tree_bytes, xcol, row_bytes, 0.0f, la)
-                 : walk_chunk<D, G, false, Q>(pt, q, s.p_trees, s.tree_bytes, xcol, row_bytes, 0.0f, la);
+      accp = nan ? walk_chunk<D, G, true, Q>(pt, q, s.p_trees, xcol, row_bytes, 0.0f, la)
+                 : walk_chunk<D, G, false, Q>(pt, q, s.p_trees, xcol, row_bytes, 0.0f, la);
       if (Q > 1) {
         __syncthreads();
         if (q == 0)
