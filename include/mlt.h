@@ -442,7 +442,9 @@ int mlt_tune_walk(int model_id, int candidates, int splits, int group, int chunk
  * or lanes per candidate), trees in flight per thread, trees per chunk,
  * chunk buffers, CTAs resident per SM, table kind (0 full, 1 compact,
  * 2 half, 3 split).  Batches that mlt_screen screens in one launch
- * (mlt_tune_fused_small) do not use this shape.  Host-only. */
+ * (mlt_tune_fused_small) do not use this shape, nor do large batches of
+ * stored rows that are walked in ordinal form (integers in place of the
+ * thresholds and features, same results).  Host-only. */
 int mlt_walk_shape(int model_id, int64_t n, int p_pass, int32_t *out);
 
 /* Tuning: batches of up to max_n candidates (0 .. 8,192; the default is

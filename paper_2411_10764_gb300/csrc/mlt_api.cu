@@ -22,6 +22,7 @@
 #include <cuda_fp16.h>
 
 #include "mlt_internal.cuh"
+#include "ordinal.cuh"
 #include "peak.cuh"
 
 // Scratch of mlt_screen_noalloc: one fixed array in the module's global
@@ -99,6 +100,9 @@ struct ScratchOwner {
   // rows of compiled-decoder batches, grown with n x F
   float* feat_buf = nullptr;
   long long feat_cap = 0;
+  // candidates' ordinals, grown with n x F up to kOrdMaxBytes
+  unsigned char* ord_buf = nullptr;
+  size_t ord_cap = 0;
   // host-buffer entry point staging
   long long host_cap_n = -1;
   int host_cap_F = 0;
@@ -202,6 +206,33 @@ bool try_feat_buf(long long elems) {
   }
   g_scr.feat_buf = static_cast<float*>(p);
   g_scr.feat_cap = elems;
+  return true;
+}
+
+// The ordinal buffer: at least `bytes` (grown, kept until the feature count
+// changes or a V or P model is freed).  False where it would be larger than
+// kOrdMaxBytes or cannot be had; the walk then reads the fp32 rows.
+constexpr size_t kOrdMaxBytes = 8ull << 30;
+
+void free_ord_buf() {
+  if (g_scr.ord_buf == nullptr) return;
+  cudaDeviceSynchronize();  // queued screens may still read it
+  cudaFree(g_scr.ord_buf);
+  g_scr.ord_buf = nullptr;
+  g_scr.ord_cap = 0;
+}
+
+bool try_ord_buf(size_t bytes) {
+  if (bytes <= g_scr.ord_cap) return true;
+  if (bytes > kOrdMaxBytes) return false;
+  free_ord_buf();
+  void* p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();  // clear the allocation failure
+    return false;
+  }
+  g_scr.ord_buf = static_cast<unsigned char*>(p);
+  g_scr.ord_cap = bytes;
   return true;
 }
 
@@ -478,11 +509,93 @@ int pack_ensemble(const mlt_node* nodes, int n_trees, int depth, int F, std::vec
   return MLT_OK;
 }
 
+// Ordinal walk of a pass over stored rows: the rule of sizes.  Making the
+// ordinals costs about 17 shared-memory cycles per warp and feature (10
+// search steps), and a visit of the ordinal walk about 1.5 cycles less than
+// the fp32 walk's, so a candidate's visits must outweigh its features; below
+// kOrdMinN candidates the extra launch costs more than the walk saves.
+constexpr long long kOrdMinN = 16384;
+constexpr int kOrdMinVisits = 16;  // per feature
+
+bool ord_wanted(const DeviceModel& m, const ShapeOverride& ov, long long n) {
+  if (m.ord.table == nullptr || n < kOrdMinN) return false;
+  if (ov.threads || ov.chunk_trees || ov.nbuf || ov.lanes || ov.group) return false;  // a fixed shape of the fp32 walk
+  return static_cast<long long>(m.n_trees) * m.depth >= static_cast<long long>(kOrdMinVisits) * g_F;
+}
+
+// Bytes of the ordinals of n candidates, and of their missing-value flags.
+size_t ord_bytes(long long n) { return static_cast<size_t>((n + 31) / 32) * ((g_F + 1) / 2) * 128; }
+size_t ord_flag_bytes(long long n) { return align16(static_cast<size_t>((n + 31) / 32) * ((g_F + 7) / 8)); }
+
+// One walk pass (V over all candidates or P over the survivors).
+struct Pass {
+  ScreenShape shape;
+  bool ord = false;  // the ordinal walk (shape is then plan_ord's)
+};
+
+// Plans of both passes over n candidates.  stored: the rows are in memory and
+// the ordinal buffer may be allocated.
+void plan_passes(const DeviceModel& V, const DeviceModel& P, long long n, bool stored, Pass* pv, Pass* pp) {
+  const DeviceModel* m[2] = {&V, &P};
+  Pass* p[2] = {pv, pp};
+  // the P pass walks the survivors; plan it for about half the batch
+  const long long n_eff[2] = {n, (n + 1) / 2};
+  size_t bytes = 0;
+  for (int i = 0; i < 2; ++i) {
+    p[i]->ord = stored && ord_wanted(*m[i], g_shape[i], n);
+    if (p[i]->ord) p[i]->shape = plan_ord(g_F, m[i]->ord, m[i]->depth, n_eff[i], sm_count(), smem_optin());
+    p[i]->ord = p[i]->ord && p[i]->shape.threads > 0;
+    if (p[i]->ord) bytes = std::max(bytes, ord_bytes(n) + ord_flag_bytes(n));
+  }
+  if (bytes > 0 && !try_ord_buf(bytes)) pv->ord = pp->ord = false;
+  for (int i = 0; i < 2; ++i)
+    if (!p[i]->ord) p[i]->shape = plan_for(*m[i], g_F, n_eff[i], g_shape[i], i == 0);
+}
+
+cudaError_t launch_pass(const DeviceModel& m, TraverseArgs a, const Pass& p, const DecodeParams* dec, long long n,
+                        cudaStream_t st, long long* launches) {
+  const ScreenShape& sh = p.shape;
+  const long long tiles = (n + sh.threads - 1) / sh.threads;
+  a.chunk_trees = sh.chunk_trees;
+  a.nbuf = sh.nbuf;
+  if (tiles <= 0) return cudaSuccess;
+  *launches += 1;
+  if (!p.ord) {
+    a.table = m.table;
+    a.n_trees = m.n_trees;
+    a.tree_bytes = m.tree_bytes;
+    a.max_depth = m.depth;
+    a.tail = reinterpret_cast<const uint2*>(m.tail);
+    return dec ? launch_traverse_dec(m, a, *dec, sh, tiles, st) : launch_traverse(m, a, sh, tiles, st);
+  }
+  *launches += 1;
+  OrdArgs o{};
+  o.feats = a.feats;
+  o.F = a.F;
+  o.vec4 = a.vec4;
+  o.n = n;
+  o.rows = a.p_pass ? a.rows : nullptr;
+  o.count = a.p_pass ? &a.state->survivors : nullptr;
+  o.stream = a.stream;
+  o.out = reinterpret_cast<uint32_t*>(g_scr.ord_buf);
+  o.nan_flags = g_scr.ord_buf + ord_bytes(n);
+  o.err = a.err;
+  cudaError_t e = launch_ordinals(m.ord, o, n, sm_count(), st);
+  if (e != cudaSuccess) return e;
+  a.table = m.ord.table;
+  a.n_trees = m.ord.n_trees;
+  a.ord = o.out;
+  a.nan_flags = o.nan_flags;
+  a.nan_groups = (g_F + 7) / 8;
+  return launch_walk_ord(m.depth, a, sh, tiles, st);
+}
+
 // The whole screening sequence on `st` with scratch `s` (caller holds g_mu).
-// `profile_ok`: phase events may be recorded.
+// fixed_scratch: `s` is the fixed array, no phase events are recorded and
+// nothing is allocated.
 int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec, long long n, float thr,
                     int k, float* out_pvalid, float* out_perf, int64_t* out_topk, const Scratch& s,
-                    bool profile_ok) {
+                    bool fixed_scratch) {
   int dev = 0;
   int rc = current_device(&dev);
   if (rc != MLT_OK) return rc;
@@ -504,9 +617,9 @@ int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec
       dec = nullptr;
     }
   }
-  // the P pass walks the survivors; plan it for about half the batch
-  const ScreenShape sv = plan_for(V, g_F, n, g_shape[MLT_MODEL_V], true);
-  const ScreenShape sp = plan_for(P, g_F, (n + 1) / 2, g_shape[MLT_MODEL_P], false);
+  Pass pv, pp;
+  plan_passes(V, P, n, dec == nullptr && !fixed_scratch, &pv, &pp);
+  const ScreenShape &sv = pv.shape, &sp = pp.shape;
   if (sv.threads == 0 || sp.threads == 0) return fail(MLT_EINVAL, "F=%d leaves no room for a shared-memory tile", g_F);
   TraverseArgs a{};
   a.feats = feats;
@@ -529,19 +642,12 @@ int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec
 
   TraverseArgs av = a;
   av.p_pass = 0;
-  av.table = V.table;
-  av.n_trees = V.n_trees;
-  av.tree_bytes = V.tree_bytes;
-  av.chunk_trees = sv.chunk_trees;
-  av.nbuf = sv.nbuf;
-  av.max_depth = V.depth;
-  av.tail = reinterpret_cast<const uint2*>(V.tail);
   // every call starts from a fresh selection state: its tickets decide which
   // CTA scans the tile counts and ranks the keys, so a count left behind by
   // an earlier call (one that stopped part-way) must not carry over
   MLT_CUDA(cudaMemsetAsync(s.state, 0, sizeof(SelectState), st), "reset selection state");
   cudaEvent_t* ev = nullptr;
-  if (g_profile && profile_ok) {
+  if (g_profile && !fixed_scratch) {
     if (g_events_used + kPhases + 1 > g_events.size()) {
       for (int i = 0; i <= kPhases; ++i) {
         cudaEvent_t e;
@@ -585,28 +691,19 @@ int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec
     av.stall_ns = g_stall_ns;
     g_stall_cta = -1;
   }
-  MLT_CUDA(dec ? launch_traverse_dec(V, av, *dec, sv, tiles_v, st) : launch_traverse(V, av, sv, tiles_v, st),
-           "V pass launch");
+  long long launches = 0;
+  MLT_CUDA(launch_pass(V, av, pv, dec, n, st, &launches), "V pass launch");
   if (ev) MLT_CUDA(cudaEventRecord(ev[1], st), "cudaEventRecord");
   MLT_CUDA(launch_compact(s, n, sv.threads, tiles_v, nullptr, st), "compaction launch");
   if (ev) MLT_CUDA(cudaEventRecord(ev[2], st), "cudaEventRecord");
 
   TraverseArgs ap = a;
   ap.p_pass = 1;
-  ap.table = P.table;
-  ap.n_trees = P.n_trees;
-  ap.tree_bytes = P.tree_bytes;
-  ap.chunk_trees = sp.chunk_trees;
-  ap.nbuf = sp.nbuf;
-  ap.max_depth = P.depth;
-  ap.tail = reinterpret_cast<const uint2*>(P.tail);
-  const long long tiles_p = (n + sp.threads - 1) / sp.threads;
-  MLT_CUDA(dec ? launch_traverse_dec(P, ap, *dec, sp, tiles_p, st) : launch_traverse(P, ap, sp, tiles_p, st),
-           "P pass launch");
+  MLT_CUDA(launch_pass(P, ap, pp, dec, n, st, &launches), "P pass launch");
   if (ev) MLT_CUDA(cudaEventRecord(ev[3], st), "cudaEventRecord");
   MLT_CUDA(launch_topk(s, n, k, topk_base, out_topk, sm_count(), nullptr, st), "top-k launch");
   if (ev) MLT_CUDA(cudaEventRecord(ev[4], st), "cudaEventRecord");
-  g_launches += (tiles_v > 0 ? 1 : 0) + (tiles_v > 0 ? 1 : 0) + (tiles_p > 0 ? 1 : 0) + 1;
+  g_launches += launches + (tiles_v > 0 ? 1 : 0) + 1;
   return MLT_OK;
 }
 
@@ -660,8 +757,9 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
   const DeviceModel& V = g_models[MLT_MODEL_V].dm;
   const DeviceModel& P = g_models[MLT_MODEL_P].dm;
   const long long per = std::min(batch, std::max(1LL, n_total));
-  const ScreenShape sv = plan_for(V, g_F, per, g_shape[MLT_MODEL_V], true);
-  const ScreenShape sp = plan_for(P, g_F, (per + 1) / 2, g_shape[MLT_MODEL_P], false);
+  Pass pv, pp;
+  plan_passes(V, P, per, dec0 == nullptr, &pv, &pp);
+  const ScreenShape &sv = pv.shape, &sp = pp.shape;
   if (sv.threads == 0 || sp.threads == 0) return fail(MLT_EINVAL, "F=%d leaves no room for a shared-memory tile", g_F);
   MLT_CUDA(cudaMemsetAsync(s.state, 0, sizeof(SelectState), st), "reset selection state");
   MLT_CUDA(cudaMemsetAsync(ss, 0, sizeof(StreamState), st), "reset stream state");
@@ -697,31 +795,14 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
     }
     TraverseArgs av = ab;
     av.p_pass = 0;
-    av.table = V.table;
-    av.n_trees = V.n_trees;
-    av.tree_bytes = V.tree_bytes;
-    av.chunk_trees = sv.chunk_trees;
-    av.nbuf = sv.nbuf;
-    av.max_depth = V.depth;
-    av.tail = reinterpret_cast<const uint2*>(V.tail);
     const long long tiles_v = (nb + sv.threads - 1) / sv.threads;
-    MLT_CUDA(dec0 ? launch_traverse_dec(V, av, d, sv, tiles_v, st) : launch_traverse(V, av, sv, tiles_v, st),
-             "V pass launch");
+    MLT_CUDA(launch_pass(V, av, pv, dec0 ? &d : nullptr, nb, st, &launches), "V pass launch");
     MLT_CUDA(launch_compact(s, nb, sv.threads, tiles_v, ss, st), "compaction launch");
     TraverseArgs ap = ab;
     ap.p_pass = 1;
-    ap.table = P.table;
-    ap.n_trees = P.n_trees;
-    ap.tree_bytes = P.tree_bytes;
-    ap.chunk_trees = sp.chunk_trees;
-    ap.nbuf = sp.nbuf;
-    ap.max_depth = P.depth;
-    ap.tail = reinterpret_cast<const uint2*>(P.tail);
-    const long long tiles_p = (nb + sp.threads - 1) / sp.threads;
-    MLT_CUDA(dec0 ? launch_traverse_dec(P, ap, d, sp, tiles_p, st) : launch_traverse(P, ap, sp, tiles_p, st),
-             "P pass launch");
+    MLT_CUDA(launch_pass(P, ap, pp, dec0 ? &d : nullptr, nb, st, &launches), "P pass launch");
     MLT_CUDA(launch_accumulate(ss, s.state, nb, tgt, st), "accumulate launch");
-    launches += 4;
+    launches += 2;
   }
   MLT_CUDA(launch_topk(s, n_total, k, dec0 ? dec0->first_index : 0, out_topk, sm_count(), &ss->total, st),
            "top-k launch");
@@ -748,7 +829,7 @@ int run_screen(cudaStream_t st, const float* feats, const DecodeParams* dec, lon
                float* out_pvalid, float* out_perf, int64_t* out_topk) {
   const int rc = ensure_scratch(n);
   if (rc != MLT_OK) return rc;
-  return run_screen_with(st, feats, dec, n, thr, k, out_pvalid, out_perf, out_topk, g_scr.s, true);
+  return run_screen_with(st, feats, dec, n, thr, k, out_pvalid, out_perf, out_topk, g_scr.s, false);
 }
 
 // Split table (kTableSplit, deep models V and P): validate like
@@ -974,6 +1055,13 @@ int install_model(int model_id, const std::vector<unsigned char>& packed, const 
   m.dm.table = d;
   m.dm.bytes = packed.size();
   if (dm.kind == kTableSplit) m.dm.tail = d + dm.tail_off;
+  OrdTable& o = m.dm.ord;
+  if (o.n_trees > 0) {
+    o.table = d + o.off_table;
+    o.image = d + o.off_image;
+    o.features = reinterpret_cast<const OrdFeature*>(d + o.off_features);
+    o.groups = reinterpret_cast<const OrdGroup*>(d + o.off_groups);
+  }
   return MLT_OK;
 }
 
@@ -984,8 +1072,10 @@ extern "C" {
 int mlt_set_num_features(int F) {
   if (F < 1 || F > kMaxF) return fail(MLT_EINVAL, "F must lie in [1, %d], got %d", kMaxF, F);
   std::lock_guard<std::mutex> lk(g_mu);
-  if (F != g_F)
+  if (F != g_F) {
     for (Model& m : g_models) free_model(m);
+    free_ord_buf();
+  }
   g_F = F;
   return MLT_OK;
 }
@@ -1005,6 +1095,7 @@ int mlt_load_ensemble(int model_id, const mlt_node* nodes, int n_trees, int dept
   int rc = split ? pack_split(nodes, n_trees, depth, g_F, g_head_levels, packed, dm)
                  : pack_ensemble(nodes, n_trees, depth, g_F, packed, dm);
   if (rc != MLT_OK) return rc;
+  if (dm.kind == kTableFull && model_id != MLT_MODEL_A) pack_ordinal(nodes, n_trees, depth, g_F, false, packed, dm.ord);
   return install_model(model_id, packed, dm);
 }
 
@@ -1054,6 +1145,7 @@ int mlt_load_ensemble_f16(int model_id, const mlt_node* nodes, int n_trees, int 
   DeviceModel dm;
   int rc = pack_ensemble_half(nodes, n_trees, depth, g_F, packed, dm);
   if (rc != MLT_OK) return rc;
+  pack_ordinal(nodes, n_trees, depth, g_F, true, packed, dm.ord);
   return install_model(model_id, packed, dm);
 }
 
@@ -1061,6 +1153,7 @@ int mlt_free_ensemble(int model_id) {
   if (model_id < MLT_MODEL_V || model_id > MLT_MODEL_A) return fail(MLT_EINVAL, "unknown model id %d", model_id);
   std::lock_guard<std::mutex> lk(g_mu);
   free_model(g_models[model_id]);
+  if (model_id != MLT_MODEL_A) free_ord_buf();
   return MLT_OK;
 }
 
@@ -1103,7 +1196,7 @@ int mlt_screen_noalloc(void* stream, const float* feats, int64_t n, float thr, i
   // the array keeps the previous call's contents; the selection state is
   // cleared at the start of the sequence, the error word only when
   // mlt_sync_status reads it (so a fault of this call stays visible)
-  return run_screen_with(st, feats, nullptr, n, thr, k, out_pvalid, out_perf, out_topk, s, false);
+  return run_screen_with(st, feats, nullptr, n, thr, k, out_pvalid, out_perf, out_topk, s, true);
 }
 
 int mlt_merge_topk(void* stream, const float* scores, const int64_t* indices, int64_t m, int k,
@@ -1190,7 +1283,7 @@ int mlt_sa_step(void* stream, const int32_t* radices, const float* option_values
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   MLT_CUDA(launch_sa_propose(d, space, parent, knob_draw, digit_draw, m, S.sa_prop, S.err, st), "propose launch");
   d.index_list = S.sa_prop;
-  rc = run_screen_with(st, nullptr, &d, m, thr, 1, S.sa_pvalid, S.sa_perf, S.sa_topk, g_scr.s, true);
+  rc = run_screen_with(st, nullptr, &d, m, thr, 1, S.sa_pvalid, S.sa_perf, S.sa_topk, g_scr.s, false);
   if (rc != MLT_OK) return rc;
   MLT_CUDA(launch_sa_accept(space, parent, parent_score, S.sa_prop, S.sa_perf, log_u, m, temperature, out_next,
                             out_next_score, out_accepted, st),
@@ -1367,7 +1460,7 @@ int mlt_screen_host_batches(void* stream, int64_t n_batches, const float* const*
     const int i = static_cast<int>(b & 1);
     MLT_CUDA(cudaStreamWaitEvent(sc, S.hb_in[i], 0), "cudaStreamWaitEvent");
     if (b >= 2) MLT_CUDA(cudaStreamWaitEvent(sc, S.hb_down[i], 0), "cudaStreamWaitEvent");
-    rc = run_screen_with(sc, S.hb_feats[i], nullptr, n, thr, k, S.hb_pvalid[i], S.hb_perf[i], S.hb_topk[i], S.s, true);
+    rc = run_screen_with(sc, S.hb_feats[i], nullptr, n, thr, k, S.hb_pvalid[i], S.hb_perf[i], S.hb_topk[i], S.s, false);
     if (rc != MLT_OK) return rc;
     MLT_CUDA(cudaEventRecord(S.hb_out[i], sc), "cudaEventRecord");
     if (b >= 1) {

@@ -137,6 +137,42 @@ constexpr uint32_t kCompactFeatureMask = 0x3FFu;  // bits 0..9
 constexpr uint32_t kCompactChildShift = 10;       // bits 10..29
 constexpr uint32_t kCompactChildMask = 0xFFFFFu;
 
+// Ordinal form of a full or half table (ordinal.cuh has the layout).
+constexpr int kOrdTreePad = 4;        // trees are padded to a multiple of this
+constexpr int kOrdMaxDistinct = 8191;  // distinct thresholds per feature
+constexpr int kOrdMaxBuckets = 2048;   // buckets of a feature's lookup table
+constexpr uint32_t kOrdNan = 0x8000u;  // ordinal of a missing value
+
+struct alignas(16) OrdFeature {
+  float lo;        // its smallest threshold
+  float add;       // c - lo: a bucket is taken from the bits of max(x, lo) + add
+  uint32_t base;   // bits of c
+  uint32_t shift;  // bits below a bucket
+  uint32_t last;   // last bucket
+  uint32_t steps;  // compares after the lookup, the same for eight features
+  uint32_t thr;    // byte offset of its thresholds in its group's image
+  uint32_t lut;    // byte offset of its lookup table
+};
+struct OrdGroup {
+  uint32_t first;  // first feature (a multiple of 8)
+  uint32_t count;  // features
+  uint32_t off;    // bytes from the start of `image`
+  uint32_t bytes;  // a multiple of 16
+};
+constexpr int kOrdMaxGroups = kMaxF / 8;
+struct OrdTable {
+  const unsigned char* table = nullptr;  // null: the model has no ordinal form
+  const unsigned char* image = nullptr;
+  const OrdFeature* features = nullptr;
+  const OrdGroup* groups = nullptr;
+  size_t off_table = 0, off_image = 0, off_features = 0, off_groups = 0;  // in the model's allocation
+  int n_trees = 0;         // padded
+  int n_groups = 0;
+  uint32_t max_bytes = 0;  // of a group's image
+  unsigned char chunks[kOrdMaxGroups] = {};  // of a group: its features / 8, rounded up
+  int round_half = 0;
+};
+
 struct DeviceModel {
   const unsigned char* table = nullptr;
   size_t bytes = 0;
@@ -147,6 +183,7 @@ struct DeviceModel {
   int head_levels = 0;      // split tables: H
   const unsigned char* tail = nullptr;  // split tables: the tail records
   size_t tail_off = 0;                  // split tables: byte offset of the tail records
+  OrdTable ord;                         // full and half tables: the ordinal form, when there is one
 };
 
 // ---------------------------------------------------------------------------
@@ -247,6 +284,12 @@ struct TraverseArgs {
   // stall_ns (-1: no CTA does)
   int stall_cta = -1;
   unsigned long long stall_ns = 0;
+  // ordinal walk: the candidates' ordinals and each block's missing-value
+  // flags, nan_groups a block
+  const uint32_t* ord = nullptr;
+  const unsigned char* nan_flags = nullptr;
+  int nan_groups = 0;
+  int groups = 1;  // tree groups of the CTA
 };
 
 struct ScreenShape {

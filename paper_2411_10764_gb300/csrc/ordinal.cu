@@ -1,0 +1,579 @@
+// Feature ordinals and the ordinal walk (layout and exactness: ordinal.cuh).
+// XGBoost gbtree prediction (Sec. 3, Table 3) for large batches of stored
+// rows: k_ordinals turns the rows into ordinals, k_walk_ord walks them.
+#include <algorithm>
+#include <cmath>
+
+#include "ordinal.cuh"
+#include "walk.cuh"
+
+namespace mlt {
+namespace {
+
+using namespace walk;
+
+constexpr int kOrdThreads = 1024;
+constexpr int kOrdRows = 2;  // blocks of 32 rows a warp takes together
+constexpr int kOrdMaxCta = 1024;
+constexpr size_t kSmPerSm = 228 * 1024;
+constexpr size_t kCtaReserve = 1024;
+constexpr size_t kStaticSmem = 1024;
+
+// `steps` compares from the bucket's start: p += 2^k entries wherever the
+// last of them is still <= x.  One load, one compare and one predicated add
+// each (the offsets are immediates).
+template <int K>
+__device__ __forceinline__ void ord_step(uint32_t (&p)[2][4], const float* x) {
+  float t[2][4];
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    asm("ld.shared.f32 %0, [%1 + %2];" : "=f"(t[r >> 2][r & 3]) : "r"(p[r >> 2][r & 3]), "n"((4 << K) - 4));
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    asm("{\n\t.reg .pred q;\n\tsetp.le.f32 q, %1, %2;\n\t@q add.u32 %0, %0, %3;\n\t}"
+        : "+r"(p[r >> 2][r & 3])
+        : "f"(t[r >> 2][r & 3]), "f"(x[r]), "n"(4 << K));
+}
+__device__ __forceinline__ void ord_search(uint32_t steps, uint32_t (&p)[2][4], const float* x) {
+  switch (steps) {
+    case 13: ord_step<12>(p, x); [[fallthrough]];
+    case 12: ord_step<11>(p, x); [[fallthrough]];
+    case 11: ord_step<10>(p, x); [[fallthrough]];
+    case 10: ord_step<9>(p, x); [[fallthrough]];
+    case 9: ord_step<8>(p, x); [[fallthrough]];
+    case 8: ord_step<7>(p, x); [[fallthrough]];
+    case 7: ord_step<6>(p, x); [[fallthrough]];
+    case 6: ord_step<5>(p, x); [[fallthrough]];
+    case 5: ord_step<4>(p, x); [[fallthrough]];
+    case 4: ord_step<3>(p, x); [[fallthrough]];
+    case 3: ord_step<2>(p, x); [[fallthrough]];
+    case 2: ord_step<1>(p, x); [[fallthrough]];
+    case 1: ord_step<0>(p, x); break;
+    default: break;
+  }
+}
+
+// A CTA holds one feature group's thresholds and lookup tables in shared
+// memory.  A warp takes 64 rows and 8 features (one 32-byte sector of each
+// row) at a time: lanes 2i and 2i + 1 read the two halves of a row's sector
+// together (16 lines a load, where a lane per row would touch 32), so an even
+// lane searches features 0-3 and an odd one 4-7, four rows each, two
+// features together (eight chains in flight).  Groups get CTAs in proportion to their
+// features.  Bound: the L1 data pipe (about 11 wavefronts of table loads and
+// 4 of row loads per 32 values) and integer issue.
+template <bool VEC, bool HALF>
+__global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_constant__ OrdArgs a) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) unsigned long long bar;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int gi = 0;
+  for (int hi = a.n_groups; gi + 1 < hi;) {
+    const int mid = (gi + hi) >> 1;
+    if (blockIdx.x >= a.first_cta[mid])
+      gi = mid;
+    else
+      hi = mid;
+  }
+  const int slab = blockIdx.x - a.first_cta[gi], slabs = a.first_cta[gi + 1] - a.first_cta[gi];
+  const OrdGroup g = a.groups[gi];
+  if (tid == 0) {
+    mbar_init(smem_u32(&bar), 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (tid == 0 && g.bytes > 0) {  // thresholds are static: before waiting on earlier kernels
+    mbar_expect_tx(smem_u32(&bar), g.bytes);
+    bulk_copy_g2s(smem_u32(smem), a.image + g.off, g.bytes, smem_u32(&bar));
+  }
+  pdl_wait();
+  pdl_trigger();
+  const bool skip = a.stream && *reinterpret_cast<volatile const unsigned*>(&a.stream->done);
+  const long long count = skip ? 0 : a.count ? static_cast<long long>(*a.count) : a.n;
+  const long long blocks = (count + 31) >> 5;
+  const int F2 = (a.F + 1) >> 1, F8 = (a.F + 7) >> 3;
+  const int nf = static_cast<int>(g.count), chunks = (nf + 7) >> 3;
+  const uint32_t items = static_cast<uint32_t>((blocks + kOrdRows - 1) / kOrdRows) * chunks;  // n x F fits memory
+  const OrdFeature* feat = a.features + g.first;
+  const uint32_t step = slabs * (blockDim.x >> 5);
+  const uint32_t sm = smem_u32(smem);
+  // every warp waits for the copy, also one without rows: it must land before
+  // the CTA's shared memory is released
+  if (g.bytes > 0 && !__all_sync(0xFFFFFFFFu, mbar_wait_bounded(smem_u32(&bar), 0u))) {
+    mbar_wait_bounded(smem_u32(&bar), 0u);
+    atomicOr(a.err, kErrWaitTimeout);
+    return;
+  }
+  for (uint32_t it = warp * slabs + slab; it < items; it += step) {
+    const uint32_t s32 = it / static_cast<uint32_t>(chunks);
+    const int f0 = static_cast<int>(it - s32 * chunks) * 8;
+    const long long sb = s32;
+    // row slot r of this lane: row 16 r + lane / 2 of the 64; features h0 .. h0 + 3
+    const int h0 = f0 + (lane & 1) * 4;
+    float x[4][4];  // [feature][row slot]
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const long long i = sb * (kOrdRows * 32) + r * 16 + (lane >> 1);
+      const bool in = i < count && h0 < nf;
+      const long long row = in ? (a.rows ? static_cast<long long>(a.rows[i]) : i) : 0;
+      const float* src = a.feats + row * a.F + g.first + h0;
+      if constexpr (VEC) {
+        const float4 v = in ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        x[0][r] = v.x;
+        x[1][r] = v.y;
+        x[2][r] = v.z;
+        x[3][r] = v.w;
+      } else {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) x[h][r] = in && h0 + h < nf ? __ldg(src + h) : 0.0f;
+      }
+    }
+    // ordinals of a row slot: words of pairs (h0, h0 + 1) and (h0 + 2, h0 + 3)
+    uint32_t* dst = a.out + (sb * kOrdRows * F2 + ((g.first + h0) >> 1)) * 32;
+    uint32_t missing = 0;  // bits: row slots of this lane that hold a missing value
+    const uint32_t steps = __ldg(&feat[f0].steps);
+#pragma unroll
+    for (int h = 0; h < 4; h += 2) {
+      uint32_t p[2][4], start[2], origin = 0;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {  // the table is padded to a multiple of 8 features
+        const float4 o0 = __ldg(reinterpret_cast<const float4*>(feat + h0 + h + e));
+        const uint4 o1 = __ldg(reinterpret_cast<const uint4*>(feat + h0 + h + e) + 1);
+        const uint32_t base = __float_as_uint(o0.z), shift = __float_as_uint(o0.w);
+        const uint32_t thr = sm + o1.z, lut = sm + o1.w;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (HALF) x[h + e][r] = __half2float(__float2half_rn(x[h + e][r]));
+          const uint32_t d = __float_as_uint(__fadd_rn(fmaxf(x[h + e][r], o0.x), o0.y)) - base;
+          p[e][r] = thr + lds_u16(lut + min(d >> shift, o1.x) * 2u) * 4u;
+        }
+        origin += e == 0 ? thr >> 2 : thr << 14;
+        start[e] = thr;
+      }
+      ord_search(steps, p, x[h]);
+      bool nan = false;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) nan |= x[h + (r >> 2)][r & 3] != x[h + (r >> 2)][r & 3];
+      if (nan) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          if (x[h + (r >> 2)][r & 3] != x[h + (r >> 2)][r & 3]) {
+            p[r >> 2][r & 3] = start[r >> 2] + kOrdNan * 4u;
+            missing |= 1u << (r & 3);
+          }
+      }
+      if (h0 + h < nf) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          // (p - thr) / 4 of the two features in the low and high halves; row
+          // slots 0, 1 are in the first block of 32, slots 2, 3 in the second
+          const uint32_t word = (p[0][r] >> 2) + (p[1][r] << 14) - origin;
+          if (sb * kOrdRows + (r >> 1) < blocks)
+            dst[((r >> 1) * F2 + (h >> 1)) * 32 + (r & 1) * 16 + (lane >> 1)] = word;
+        }
+      }
+    }
+    missing = __reduce_or_sync(0xFFFFFFFFu, missing);
+    if (lane < kOrdRows && sb * kOrdRows + lane < blocks)
+      a.nan_flags[(sb * kOrdRows + lane) * F8 + ((g.first + f0) >> 3)] = (missing >> (2 * lane)) & 3u ? 1 : 0;
+  }
+}
+
+// Leaves of G consecutive trees at tb for one candidate (its column of
+// ordinals at xw).
+template <int D, int G, bool NANP>
+__device__ __forceinline__ void walk_ord(const unsigned char* tb, const unsigned char* xw, float* leaf) {
+  constexpr uint32_t kTree = ord_tree_bytes(D);
+  uint32_t j[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) j[g] = 1u;
+#pragma unroll
+  for (int l = 0; l < D; ++l) {
+    uint32_t w[G], x[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) w[g] = ld_sm<uint32_t>(tb, g * kTree + j[g] * 4u);
+#pragma unroll
+    for (int g = 0; g < G; ++g) x[g] = ld_sm<unsigned short>(xw, w[g] & 0xFFFEu);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      if (NANP) x[g] &= ~(w[g] << 15);  // kOrdNan becomes 0 where a missing value goes left
+      j[g] = __funnelshift_l(w[g] - x[g] * 65536u, j[g], 1);
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < G; ++g) leaf[g] = ld_sm<float>(tb, g * kTree + j[g] * 4u);
+}
+
+// Leaves of nt <= U trees (a multiple of 4), up to 8 trees in flight.
+template <int D, int U, bool NANP>
+__device__ __forceinline__ void walk_ord_unit(const unsigned char* tb, int nt, const unsigned char* xw, float* leaf) {
+  constexpr uint32_t kTree = ord_tree_bytes(D);
+#pragma unroll
+  for (int t = 0; t < U; t += 8) {
+    if (U >= 8 && nt >= t + 8)
+      walk_ord<D, U >= 8 ? 8 : 4, NANP>(tb + t * kTree, xw, leaf + t);
+    else if (nt > t)
+      walk_ord<D, 4, NANP>(tb + t * kTree, xw, leaf + t);
+  }
+}
+
+// One tree group: trees [0, nt) of a chunk, leaves added in tree order.
+template <int D, bool NANP>
+__device__ __forceinline__ float walk_ord_sum(const unsigned char* tb, int nt, const unsigned char* xw, float acc) {
+  constexpr uint32_t kTree = ord_tree_bytes(D);
+  int t = 0;
+  for (; t + 8 <= nt; t += 8) {
+    float leaf[8];
+    walk_ord<D, 8, NANP>(tb + static_cast<uint32_t>(t) * kTree, xw, leaf);
+#pragma unroll
+    for (int g = 0; g < 8; ++g) acc += leaf[g];
+  }
+  if (t < nt) {  // trees are padded to 4
+    float leaf[4];
+    walk_ord<D, 4, NANP>(tb + static_cast<uint32_t>(t) * kTree, xw, leaf);
+#pragma unroll
+    for (int g = 0; g < 4; ++g) acc += leaf[g];
+  }
+  return acc;
+}
+
+struct OrdSmem {
+  size_t rows, sums, tbuf, bars, bytes;
+};
+// Q > 1 tree groups: the candidates' running sums and a barrier per group and
+// 32 candidates.
+__host__ __device__ inline OrdSmem ord_smem(int F, int TC, int Q, int nbuf, uint32_t chunk_bytes) {
+  OrdSmem s;
+  s.rows = static_cast<size_t>((F + 1) / 2) * TC * 4;  // a multiple of 128: TC is one of 32
+  s.sums = s.rows + static_cast<size_t>(TC) * 4;
+  s.tbuf = align_up(s.sums + (Q > 1 ? static_cast<size_t>(TC) * 4 : 0), 128);
+  s.bars = s.tbuf + static_cast<size_t>(nbuf) * chunk_bytes;
+  s.bytes = s.bars + 10 * 8 + (Q > 1 ? static_cast<size_t>(TC / 32) * Q * 8 : 0);
+  return s;
+}
+
+// The tile of a CTA in blocks of 32 candidates.  V pass: TC candidates each
+// (the tile counts are scanned and scattered by tile).  P pass: the blocks of
+// the survivors split evenly over whole waves of CTAs, as in cta_tile.
+__device__ __forceinline__ void ord_tile(const TraverseArgs& a, long long count, int TC, long long* tile0, int* len) {
+  if (!a.p_pass) {
+    cta_tile(a, count, TC, tile0, len);
+    return;
+  }
+  const uint32_t nb = (static_cast<uint32_t>(count) + 31u) >> 5, per = static_cast<uint32_t>(TC) >> 5;
+  const uint32_t wave = a.p_wave > 0 ? static_cast<uint32_t>(a.p_wave) : gridDim.x;
+  const uint32_t waves = (nb + per * wave - 1) / (per * wave);
+  const uint32_t tiles = min(min(waves * wave, nb), gridDim.x);
+  if (blockIdx.x >= tiles) {
+    *tile0 = count;
+    *len = 0;
+    return;
+  }
+  const uint32_t lo = split_start(nb, tiles, blockIdx.x), hi = split_start(nb, tiles, blockIdx.x + 1);
+  *tile0 = static_cast<long long>(lo) * 32;
+  *len = static_cast<int>(min(static_cast<long long>(hi) * 32, count) - *tile0);
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// Arrive on an mbarrier; returns the arrivals that were still pending before.
+__device__ __forceinline__ uint32_t mbar_arrive_pending(uint32_t bar) {
+  uint32_t pending;
+  asm volatile(
+      "{\n\t.reg .b64 st;\n\t"
+      "mbarrier.arrive.shared::cta.b64 st, [%1];\n\t"
+      "mbarrier.pending_count.b64 %0, st;\n\t}"
+      : "=r"(pending)
+      : "r"(bar)
+      : "memory");
+  return pending;
+}
+
+// One CTA = a tile of TC candidates and Q groups of TC threads: the tile's
+// ordinals arrive in one bulk copy, the trees in chunks through nbuf buffers
+// (a warp arrives on the buffer's second barrier when it is done with it, and
+// the last one to arrive refills it).  The groups take units of U trees in
+// turn (U = 0: one group, the sum stays in its register).  With Q > 1 a candidate's sum goes from group to group: a warp walks
+// its unit, waits for the sum of the trees before it, adds its leaves in tree
+// order and hands the sum on -- the same sequential fp32 sum as one walker.
+// A warp issues an instruction every other cycle at best, so the groups
+// multiply the warps where a tile's candidates alone leave an SM too few.
+// Bound: shared-memory wavefronts (one per ordinal gather, one to 3.4 per node
+// gather) and issue.
+template <int D, int U>
+__global__ void __launch_bounds__(kOrdMaxCta, 1) k_walk_ord(const __grid_constant__ TraverseArgs a) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ int last_issued[4];  // latest chunk copied into each buffer
+  constexpr bool kGroups = U > 0;
+  const int Q = kGroups ? a.groups : 1, TC = blockDim.x / Q, tid = threadIdx.x, lane = tid & 31;
+  const int cols = TC >> 5, q = (tid >> 5) / cols, col = (tid >> 5) - q * cols;  // warp-uniform
+  const int F2 = (a.F + 1) >> 1;
+  if (a.p_pass || a.stream) pdl_wait();
+  if (a.stream && *reinterpret_cast<volatile const unsigned*>(&a.stream->done)) return;
+  const long long count = a.p_pass ? static_cast<long long>(a.state->survivors) : a.n;
+  long long tile0;
+  int rows_here;
+  ord_tile(a, count, TC, &tile0, &rows_here);
+  if (rows_here <= 0) return;  // whole CTA, before any copy is issued
+
+  constexpr uint32_t kTree = ord_tree_bytes(D);
+  const uint32_t chunk_bytes = static_cast<uint32_t>(a.chunk_trees) * kTree;
+  const OrdSmem L = ord_smem(a.F, TC, Q, a.nbuf, chunk_bytes);
+  uint32_t* rowidx = reinterpret_cast<uint32_t*>(smem + L.rows);
+  float* sums = reinterpret_cast<float*>(smem + L.sums);
+  unsigned char* tbuf = smem + L.tbuf;
+  // [0, nbuf) chunk buffers full, [4] the tile, [5] never completed
+  // (self-test), [6, 6 + nbuf) chunk buffers empty, then the sums' barriers
+  unsigned long long* bars = reinterpret_cast<unsigned long long*>(smem + L.bars);
+  const int n_chunks = (a.n_trees + a.chunk_trees - 1) / a.chunk_trees;
+  const int live_cols = (rows_here + 31) >> 5;  // columns that hold candidates
+  const bool stall = static_cast<int>(blockIdx.x) == a.stall_cta;
+  if (tid == 0) {
+    for (int b = 0; b < 6; ++b) mbar_init(smem_u32(&bars[b]), 1);
+    for (int b = 0; b < 4; ++b) {
+      mbar_init(smem_u32(&bars[6 + b]), static_cast<uint32_t>(live_cols * Q));
+      last_issued[b] = b < a.nbuf && b < n_chunks ? b : -1;
+    }
+    if (kGroups)
+      for (int b = 0; b < cols * Q; ++b) mbar_init(smem_u32(&bars[10 + b]), 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  auto issue = [&](int ch, int b) {
+    const int first = ch * a.chunk_trees;
+    const uint32_t bytes = static_cast<uint32_t>(min(a.chunk_trees, a.n_trees - first)) * kTree;
+    const uint32_t bar = smem_u32(&bars[b]);
+    mbar_expect_tx(bar, bytes);
+    bulk_copy_g2s(smem_u32(tbuf + static_cast<size_t>(b) * chunk_bytes), a.table + static_cast<size_t>(first) * kTree,
+                  bytes, bar);
+  };
+  if (tid == 0)
+    for (int ch = 0; ch < a.nbuf && ch < n_chunks; ++ch) issue(ch, ch);  // tables are static
+  if (!a.p_pass && !a.stream) pdl_wait();
+  if (tid == 0) {
+    const uint32_t tile_bytes = static_cast<uint32_t>(live_cols) * static_cast<uint32_t>(F2) * 128u;
+    mbar_expect_tx(smem_u32(&bars[4]), tile_bytes);
+    bulk_copy_g2s(smem_u32(smem), a.ord + (tile0 >> 5) * F2 * 32, tile_bytes, smem_u32(&bars[4]));
+  }
+  if (a.p_pass && tid < rows_here) rowidx[tid] = a.rows[tile0 + tid];
+  bool nan = false;
+  if (col < live_cols) {
+    const unsigned char* fl = a.nan_flags + ((tile0 >> 5) + col) * a.nan_groups;
+    for (int g = lane; g < a.nan_groups; g += 32) nan |= fl[g] != 0;
+  }
+  nan = __any_sync(0xFFFFFFFFu, nan);
+  float acc = 0.0f;
+  bool timed_out = false;
+  if (col < live_cols) {
+    timed_out = !__all_sync(0xFFFFFFFFu, mbar_wait_bounded(smem_u32(&bars[4]), 0u));
+    const unsigned char* xw = smem + static_cast<uint32_t>(col) * static_cast<uint32_t>(F2) * 128u + lane * 4u;
+    const uint32_t turn = smem_u32(&bars[10 + col * Q + q]);
+    const uint32_t next_turn = smem_u32(&bars[10 + col * Q + (q + 1 == Q ? 0 : q + 1)]);
+    float* sum = sums + col * 32 + lane;
+    uint32_t turns = q == 0 ? 0u : 1u;  // waits done or due; group 0's first unit waits for nobody
+    for (int ch = 0, b = 0, ph = 0; ch < n_chunks && !timed_out; ++ch) {
+      const bool ok = stall && ch == 0 ? mbar_wait_bounded_ns(smem_u32(&bars[5]), 0u, a.stall_ns)
+                                       : mbar_wait_bounded(smem_u32(&bars[b]), static_cast<uint32_t>(ph));
+      if (!__all_sync(0xFFFFFFFFu, ok)) {
+        timed_out = true;
+        break;
+      }
+      const unsigned char* tb = tbuf + static_cast<uint32_t>(b) * chunk_bytes;
+      const int nt = min(a.chunk_trees, a.n_trees - ch * a.chunk_trees);
+      if constexpr (!kGroups) {
+        acc = nan ? walk_ord_sum<D, true>(tb, nt, xw, acc) : walk_ord_sum<D, false>(tb, nt, xw, acc);
+      } else {
+        for (int t = q * U; t < nt; t += Q * U) {
+          float leaf[U];
+          const int here = min(U, nt - t);
+          if (nan)
+            walk_ord_unit<D, U, true>(tb + static_cast<uint32_t>(t) * kTree, here, xw, leaf);
+          else
+            walk_ord_unit<D, U, false>(tb + static_cast<uint32_t>(t) * kTree, here, xw, leaf);
+          if ((ch | t) != 0) {  // the first unit starts from 0
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait_bounded(turn, (turns - 1u) & 1u))) {
+              timed_out = true;
+              break;
+            }
+            acc = *sum;
+          }
+#pragma unroll
+          for (int g = 0; g < U; g += 4)
+            if (g < here) {
+              acc += leaf[g];
+              acc += leaf[g + 1];
+              acc += leaf[g + 2];
+              acc += leaf[g + 3];
+            }
+          ++turns;
+          *sum = acc;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(next_turn);
+        }
+      }
+      __syncwarp();
+      if (lane == 0 && !timed_out && ch + a.nbuf < n_chunks && mbar_arrive_pending(smem_u32(&bars[6 + b])) == 1u) {
+        mbar_try_wait(smem_u32(&bars[6 + b]), static_cast<uint32_t>(ph));  // complete: every warp is out
+        last_issued[b] = ch + a.nbuf;
+        issue(ch + a.nbuf, b);
+      }
+      if (++b == a.nbuf) {
+        b = 0;
+        ph ^= 1;
+      }
+    }
+  }
+  if (__syncthreads_or(timed_out)) {
+    if (tid == 0) {
+      // every copy in flight lands before the CTA's shared memory is released
+      // (bounded waits), then the timeout is reported
+      mbar_wait_bounded(smem_u32(&bars[4]), 0u);
+      for (int b = 0; b < a.nbuf; ++b)
+        if (last_issued[b] >= 0)
+          mbar_wait_bounded(smem_u32(&bars[b]), static_cast<uint32_t>(last_issued[b] / a.nbuf) & 1u);
+      atomicOr(a.err, kErrWaitTimeout);
+    }
+    acc = -INFINITY;  // the tile's bookkeeping still completes, none of it valid
+    __syncthreads();
+  } else if (kGroups && tid < TC) {
+    acc = sums[tid];
+  }
+  pdl_trigger();
+  finish_tile(a, rowidx, tile0, rows_here, count, acc, TC);
+}
+
+template <int U>
+FullKernelPtr ord_kernel_for(int d) {
+  switch (d) {
+    case 1: return k_walk_ord<1, U>;
+    case 2: return k_walk_ord<2, U>;
+    case 3: return k_walk_ord<3, U>;
+    case 4: return k_walk_ord<4, U>;
+    case 5: return k_walk_ord<5, U>;
+    case 6: return k_walk_ord<6, U>;
+    case 7: return k_walk_ord<7, U>;
+    case 8: return k_walk_ord<8, U>;
+    case 9: return k_walk_ord<9, U>;
+    case 10: return k_walk_ord<10, U>;
+    default: return nullptr;
+  }
+}
+
+// Trees of a unit: 16 where every group gets one of each full chunk, else
+// fewer (the hand-over of the sums costs 16 / U as much).
+int ord_unit(int chunk, int groups) {
+  if (groups == 1) return 0;
+  return chunk % (16 * groups) == 0 ? 16 : chunk % (8 * groups) == 0 ? 8 : chunk % (4 * groups) == 0 ? 4 : -1;
+}
+FullKernelPtr ord_kernel(int d, int unit) {
+  return unit == 0 ? ord_kernel_for<0>(d) : unit == 4 ? ord_kernel_for<4>(d) : unit == 8 ? ord_kernel_for<8>(d)
+                                                                                         : ord_kernel_for<16>(d);
+}
+
+}  // namespace
+
+cudaError_t launch_ordinals(const OrdTable& t, OrdArgs a, long long n_max, int sms, cudaStream_t st) {
+  if (n_max <= 0) return cudaSuccess;
+  a.groups = t.groups;
+  a.features = t.features;
+  a.image = t.image;
+  a.n_groups = t.n_groups;
+  const size_t smem = std::max<size_t>(16, t.max_bytes);
+  // one wave of CTAs, spread over the groups by their features
+  int chunks = 0;
+  for (int g = 0; g < t.n_groups; ++g) chunks += t.chunks[g];
+  const int spare = std::max(0, sms - t.n_groups);  // one CTA of 32 warps an SM
+  a.first_cta[0] = 0;
+  for (int g = 0; g < t.n_groups; ++g) {
+    const long long supers = (n_max + 32 * kOrdRows - 1) / (32 * kOrdRows);
+    const long long ctas = std::min(supers * t.chunks[g], 1 + static_cast<long long>(spare) * t.chunks[g] / chunks);
+    a.first_cta[g + 1] = static_cast<unsigned short>(a.first_cta[g] + ctas);
+  }
+  auto k = a.vec4 ? (t.round_half ? k_ordinals<true, true> : k_ordinals<true, false>)
+                  : (t.round_half ? k_ordinals<false, true> : k_ordinals<false, false>);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k, dim3(a.first_cta[t.n_groups]), dim3(kOrdThreads), smem, st, a);
+}
+
+// Candidates per CTA, tree groups, trees per chunk and buffers of the ordinal
+// walk: the shape with the least estimated cycles of the busiest SM.  Fitted
+// to sweeps on GB300 (65,536 x 64 and 1,048,576 x 128, depth 8; 16,700,000 x
+// 96, depth 10): a warp visit costs 2.6 cycles of the shared-memory pipe, more
+// with few warps, and its share of the chunk's copy into shared memory.  Tree
+// groups pay where a tile's candidates leave an SM few warps (65,536 x 64, P
+// pass of 7 warps' candidates: 58.0 / 50.5 / 47.5 us with 1 / 2 / 4 groups)
+// and cost 5 % or more where they do not (1,048,576 x 128, V pass of 16 warps:
+// 1.53 ms with 1 group, 1.59 with 2).  A chunk's hand-off stalls its warps
+// together, and a tile's start about 6,000 cycles: another resident CTA hides
+// both.
+ScreenShape plan_ord(int F, const OrdTable& t, int depth, long long n_eff, int sms, int optin) {
+  ScreenShape best{};
+  if (sms < 1) sms = 1;
+  if (n_eff < 1) n_eff = 1;
+  const uint32_t tb = ord_tree_bytes(depth);
+  const int trees8 = (t.n_trees + 7) / 8 * 8;
+  double best_cost = 1e300;
+  for (int tc = 64; tc <= 768; tc += 32) {
+    for (int q : {1, 2, 4}) {
+      if (tc * q > kOrdMaxCta) continue;
+      for (int ch = 64; ch >= 8; ch -= 8) {
+        if (ch > trees8 && ch != 8) continue;
+        const int unit = ord_unit(ch, q);
+        if (unit < 0) continue;
+        for (int nb : {2, 3}) {
+          const size_t smem = ord_smem(F, tc, q, nb, static_cast<uint32_t>(ch) * tb).bytes;
+          if (smem + kStaticSmem > static_cast<size_t>(optin)) continue;
+          const long long tiles = (n_eff + tc - 1) / tc;
+          const long long tiles_sm = (tiles + sms - 1) / sms;
+          const long long fit =
+              std::min<long long>({static_cast<long long>(kSmPerSm / (smem + kStaticSmem + kCtaReserve)),
+                                   2048 / (tc * q), 65536 / (tc * q * 64)});
+          if (fit < 1) continue;
+          const long long res = std::min(fit, tiles_sm);
+          const double warps = static_cast<double>(res) * tc * q / 32;
+          const double visit = 2.6 + 30.0 / (warps * warps) + tb / 128.0 / (tc / 32.0) / depth +
+                               (unit ? 0.15 + 1.6 / unit : 0.0);
+          const double chunks = std::ceil(static_cast<double>(t.n_trees) / ch);
+          const double cost = static_cast<double>(tiles_sm) *
+                                  (tc / 32.0 * t.n_trees * depth * visit + chunks * (400.0 + 4000.0 / warps) / (res * res) +
+                                   (res == 1 ? 6000.0 : 2000.0 / res)) +
+                              40.0 * nb;
+          if (cost < best_cost) {
+            best_cost = cost;
+            best.threads = tc;
+            best.smem = smem;
+            best.chunk_trees = ch;
+            best.nbuf = nb;
+            best.group = 8;
+            best.lanes = q;
+            best.resident = static_cast<int>(res);
+            best.p_grid = sms * static_cast<int>(res);
+          }
+        }
+      }
+    }
+  }
+  if (best.threads) best = cap_residency(best, optin);
+  return best;
+}
+
+cudaError_t launch_walk_ord(int depth, const TraverseArgs& args, const ScreenShape& shape, long long n_tiles,
+                            cudaStream_t st) {
+  if (n_tiles <= 0) return cudaSuccess;
+  TraverseArgs a = args;
+  a.groups = shape.lanes;
+  long long ctas = n_tiles;
+  if (args.p_pass && shape.p_grid > 0) {
+    a.p_wave = shape.p_grid;
+    ctas = (n_tiles + shape.p_grid - 1) / shape.p_grid * shape.p_grid;
+  }
+  FullKernelPtr k = ord_kernel(depth, ord_unit(shape.chunk_trees, shape.lanes));
+  if (k == nullptr) return cudaErrorInvalidValue;
+  cudaError_t e =
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(shape.smem));
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k, dim3(static_cast<unsigned>(ctas)), dim3(shape.threads * shape.lanes), shape.smem, st, a);
+}
+
+}  // namespace mlt

@@ -1,0 +1,252 @@
+// Builds the ordinal form of a full-table model on the host (layout:
+// ordinal.cuh).  Host code only.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <limits>
+#include <thread>
+#include <vector>
+
+#include "mlt.h"
+#include <cuda_fp16.h>
+
+#include "ordinal.cuh"
+
+namespace mlt {
+namespace {
+
+// Bytes of thresholds and lookup tables that a feature group aims at: two
+// CTAs of the ordinal kernel share an SM.
+constexpr uint32_t kGroupBytes = 80 * 1024;
+constexpr uint32_t kGroupMaxBytes = 220 * 1024;  // more thresholds in eight features: no ordinal form
+
+// A threshold's place in the order of the floats (+0 counts as -0).
+uint32_t order_key(float v) {
+  uint32_t u;
+  if (v == 0.0f) v = -0.0f;
+  std::memcpy(&u, &v, 4);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+float order_value(uint32_t k) {
+  const uint32_t u = (k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k;
+  float v;
+  std::memcpy(&v, &u, 4);
+  return v;
+}
+uint32_t bits_of(float v) {
+  uint32_t u;
+  std::memcpy(&u, &v, 4);
+  return u;
+}
+
+// Lookup table over one feature's thresholds (ascending): the kernel's bucket
+// of a value, the number of buckets and the thresholds of the fullest one.
+struct Buckets {
+  float lo = 0.0f, add = 0.0f;
+  uint32_t base = 0, shift = 0, count = 1, most = 0;
+  uint32_t at(float t) const { return (bits_of(std::fmax(t, lo) + add) - base) >> shift; }
+};
+void fill(Buckets* b, const std::vector<float>& t) {
+  b->count = b->at(t.back()) + 1;
+  b->most = 0;
+  uint32_t run = 0, last = 0xFFFFFFFFu;
+  for (float v : t) {
+    const uint32_t at = b->at(v);
+    run = at == last ? run + 1 : 1;
+    last = at;
+    b->most = std::max(b->most, run);
+  }
+}
+// The most buckets allowed for offset c.
+Buckets buckets_for(const std::vector<float>& t, float c) {
+  Buckets b;
+  b.lo = t.front();
+  b.add = c - b.lo;
+  b.base = bits_of(b.lo + b.add);
+  while (b.at(t.back()) >= static_cast<uint32_t>(kOrdMaxBuckets)) ++b.shift;
+  fill(&b, t);
+  return b;
+}
+// Steps of a search among m thresholds.
+uint32_t steps_for(uint32_t m) {
+  uint32_t s = 0;
+  while ((1u << s) <= m) ++s;
+  return s;
+}
+
+template <typename F>
+void for_features(int n, F&& body) {
+  const int workers = std::max(1, std::min<int>({8, static_cast<int>(std::thread::hardware_concurrency()), n / 8}));
+  if (workers == 1) {
+    for (int f = 0; f < n; ++f) body(f);
+    return;
+  }
+  std::vector<std::thread> pool;
+  for (int w = 0; w < workers; ++w)
+    pool.emplace_back([&, w] {
+      for (int f = w; f < n; f += workers) body(f);
+    });
+  for (std::thread& t : pool) t.join();
+}
+
+}  // namespace
+
+bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
+                  std::vector<unsigned char>& out, OrdTable& t) {
+  const int slots = (2 << depth) - 1;
+  const int inner = (1 << depth) - 1;
+  const int padded = (n_trees + kOrdTreePad - 1) / kOrdTreePad * kOrdTreePad;
+  const uint32_t tree_words = ord_tree_bytes(depth) / 4;
+  auto value = [&](const mlt_node& nd) {
+    return round_half ? __half2float(__float2half_rn(nd.value)) : nd.value;
+  };
+  std::vector<uint32_t> words(static_cast<size_t>(padded) * tree_words, 0u);
+
+  // leaves and passed-through nodes; the split nodes of each feature as
+  // (threshold's order key, word index)
+  std::vector<uint32_t> per_feature(F + 1, 0u);
+  std::vector<unsigned char> reach(slots);
+  std::vector<float> inherit(slots);
+  struct Split {
+    uint32_t feature;
+    uint32_t key;
+    uint32_t word;
+  };
+  std::vector<Split> splits;
+  if (words.size() > 0xFFFFFFFFull) return false;
+  for (int tr = 0; tr < n_trees; ++tr) {
+    const mlt_node* nd = nodes + static_cast<size_t>(tr) * slots;
+    const size_t base = static_cast<size_t>(tr) * tree_words;
+    std::fill(reach.begin(), reach.end(), 0);
+    reach[0] = 1;
+    for (int j = 0; j < slots; ++j) {
+      const bool split = reach[j] && nd[j].feature >= 0;
+      if (split) {
+        reach[2 * j + 1] = reach[2 * j + 2] = 1;
+        const float v = value(nd[j]);
+        if (v == -INFINITY) return false;  // every number is >= it: no ordinal stands for that
+        splits.push_back({static_cast<uint32_t>(nd[j].feature), order_key(v), static_cast<uint32_t>(base + j + 1)});
+        ++per_feature[nd[j].feature];
+        words[base + j + 1] = ord_offset(nd[j].feature) | (nd[j].default_left ? 1u : 0u);
+      }
+      inherit[j] = !reach[j] ? inherit[(j - 1) / 2] : split ? 0.0f : value(nd[j]);
+      if (j >= inner) std::memcpy(&words[base + j + 1], &inherit[j], 4);
+    }
+  }
+
+  // thresholds of every feature in order, and each node's place among them
+  std::vector<size_t> start(F + 1, 0);
+  for (int f = 0; f < F; ++f) start[f + 1] = start[f] + per_feature[f];
+  std::vector<uint64_t> sorted(splits.size());
+  {
+    std::vector<size_t> at(start.begin(), start.end() - 1);
+    for (const Split& s : splits) sorted[at[s.feature]++] = (static_cast<uint64_t>(s.key) << 32) | s.word;
+  }
+  std::vector<std::vector<float>> keys(F);  // distinct thresholds, ascending
+  std::vector<Buckets> buckets(F);
+  std::vector<unsigned char> fits(F, 1);
+  for_features(F, [&](int f) {
+    auto b = sorted.begin() + start[f], e = sorted.begin() + start[f + 1];
+    std::sort(b, e);
+    std::vector<float>& k = keys[f];
+    uint32_t before = 0;
+    for (auto it = b; it != e; ++it) {
+      const uint32_t key = static_cast<uint32_t>(*it >> 32);
+      if (k.empty() || before != key) k.push_back(order_value(key));
+      before = key;
+      if (k.size() > static_cast<size_t>(kOrdMaxDistinct)) {
+        fits[f] = 0;
+        return;
+      }
+      words[static_cast<uint32_t>(*it)] |= static_cast<uint32_t>(k.size() - 1) << 16;
+    }
+    if (k.empty()) return;
+    // the offset that leaves the fewest steps; then the fewest buckets that
+    // leave as few
+    const double range = std::min(3.0e38, std::max(1e-30, static_cast<double>(k.back()) - k.front()));
+    Buckets best;
+    for (int q = 0; q < 26; ++q) {
+      const Buckets b2 = buckets_for(k, std::max(1e-30f, static_cast<float>(std::ldexp(range, 1 - q))));
+      if (q == 0 || steps_for(b2.most) < steps_for(best.most)) best = b2;
+    }
+    while (best.count > 1) {
+      Buckets less = best;
+      ++less.shift;
+      fill(&less, k);
+      if (steps_for(less.most) > steps_for(best.most)) break;
+      best = less;
+    }
+    buckets[f] = best;
+  });
+  if (std::find(fits.begin(), fits.end(), 0) != fits.end()) return false;
+  // the table is padded to a multiple of 8 features; one without thresholds
+  // has a bucket of its own and nothing but padding (ordinal 0)
+  const int F8 = (F + 7) / 8 * 8;
+  keys.resize(F8);
+  buckets.resize(F8);
+  std::vector<OrdFeature> feat(F8, OrdFeature{});
+  std::vector<OrdGroup> groups;
+  uint32_t total = 0;
+  t.max_bytes = 0;
+  for (int f = 0; f < F8; f += 8) {
+    // eight features are searched with the same number of compares; a search
+    // may read 2^steps - 1 entries past the bucket's start
+    uint32_t steps = 0;
+    for (int q = f; q < f + 8; ++q) steps = std::max(steps, steps_for(buckets[q].most));
+    auto thr_bytes = [&](int q) { return static_cast<uint32_t>((keys[q].size() + (1u << steps)) * 4 + 15) & ~15u; };
+    auto lut_bytes = [&](int q) { return (buckets[q].count * 2u + 15u) & ~15u; };
+    uint32_t eight = 0;
+    for (int q = f; q < f + 8; ++q) eight += thr_bytes(q) + lut_bytes(q);
+    if (eight > kGroupMaxBytes) return false;
+    if (groups.empty() || groups.back().bytes + eight > kGroupBytes) {
+      t.chunks[groups.size()] = 0;
+      groups.push_back({static_cast<uint32_t>(f), 0u, total, 0u});
+    }
+    OrdGroup& g = groups.back();
+    ++t.chunks[groups.size() - 1];
+    g.count += static_cast<uint32_t>(std::min(8, F - f));
+    for (int q = f; q < f + 8; ++q) {
+      feat[q].thr = g.bytes;
+      feat[q].lut = g.bytes + thr_bytes(q);
+      feat[q].lo = buckets[q].lo;
+      feat[q].add = buckets[q].add;
+      feat[q].base = buckets[q].base;
+      feat[q].shift = buckets[q].shift;
+      feat[q].last = buckets[q].count - 1;
+      feat[q].steps = steps;
+      g.bytes += thr_bytes(q) + lut_bytes(q);
+    }
+    total += eight;
+    t.max_bytes = std::max(t.max_bytes, g.bytes);
+  }
+  std::vector<unsigned char> image(total);
+  for (const OrdGroup& g : groups)
+    for (uint32_t q = g.first; q < (g.first + g.count + 7) / 8 * 8; ++q) {
+      float* thr = reinterpret_cast<float*>(image.data() + g.off + feat[q].thr);
+      uint16_t* lut = reinterpret_cast<uint16_t*>(image.data() + g.off + feat[q].lut);
+      for (uint32_t i = 0; i < (feat[q].lut - feat[q].thr) / 4; ++i)
+        thr[i] = i < keys[q].size() ? keys[q][i] : std::numeric_limits<float>::quiet_NaN();
+      uint32_t at = 0;
+      for (uint32_t b = 0; b < buckets[q].count; ++b) {
+        while (at < keys[q].size() && buckets[q].at(keys[q][at]) < b) ++at;
+        lut[b] = static_cast<uint16_t>(at);
+      }
+    }
+
+  auto append = [&](const void* p, size_t bytes) {
+    const size_t at = (out.size() + 127) & ~static_cast<size_t>(127);
+    out.resize(at + bytes);
+    if (bytes) std::memcpy(out.data() + at, p, bytes);
+    return at;
+  };
+  t.off_table = append(words.data(), words.size() * 4);
+  t.off_image = append(image.data(), image.size());
+  t.off_features = append(feat.data(), feat.size() * sizeof(OrdFeature));
+  t.off_groups = append(groups.data(), groups.size() * sizeof(OrdGroup));
+  t.n_trees = padded;
+  t.n_groups = static_cast<int>(groups.size());
+  t.round_half = round_half ? 1 : 0;
+  return true;
+}
+
+}  // namespace mlt
