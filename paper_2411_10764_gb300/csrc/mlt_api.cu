@@ -82,6 +82,51 @@ struct Model {
   unsigned char* owned = nullptr;
 };
 
+// A device buffer sized by n x F: grown on demand and given back when the
+// feature count changes or a V or P model is freed.  A stream capture never
+// grows it (an allocation would end the capture), and a buffer that captured
+// work refers to is set aside instead of freed when a larger one replaces it.
+struct GrowBuf {
+  void* p = nullptr;
+  size_t cap = 0;
+  bool captured = false;
+  std::vector<void*> aside;
+
+  bool ensure(size_t bytes, cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool unknown = cudaStreamIsCapturing(st, &cs) != cudaSuccess;
+    if (unknown) cudaGetLastError();  // the default stream beside a capture
+    const bool capturing = unknown || cs != cudaStreamCaptureStatusNone;
+    if (bytes > cap) {
+      if (capturing) return false;
+      void* q = nullptr;
+      if (p != nullptr && !captured) {
+        cudaDeviceSynchronize();  // queued work may still use it
+        cudaFree(p);
+        p = nullptr;
+        cap = 0;
+      }
+      if (cudaMalloc(&q, bytes) != cudaSuccess) {
+        cudaGetLastError();  // clear the allocation failure
+        return false;
+      }
+      if (p != nullptr) aside.push_back(p);
+      p = q;
+      cap = bytes;
+      captured = false;
+    }
+    captured = captured || capturing;
+    return true;
+  }
+  void release() {
+    if (p == nullptr && aside.empty()) return;
+    cudaDeviceSynchronize();
+    cudaFree(p);
+    for (void* q : aside) cudaFree(q);
+    *this = GrowBuf();
+  }
+};
+
 struct ScratchOwner {
   int device = -1;
   long long cap_n = -1;  // capacity in candidates
@@ -97,12 +142,8 @@ struct ScratchOwner {
   float* sa_pvalid = nullptr;
   float* sa_perf = nullptr;
   int64_t* sa_topk = nullptr;
-  // rows of compiled-decoder batches, grown with n x F
-  float* feat_buf = nullptr;
-  long long feat_cap = 0;
-  // candidates' ordinals, grown with n x F up to kOrdMaxBytes
-  unsigned char* ord_buf = nullptr;
-  size_t ord_cap = 0;
+  GrowBuf feats;  // rows of decoded batches
+  GrowBuf ord;    // candidates' ordinals
   // host-buffer entry point staging
   long long host_cap_n = -1;
   int host_cap_F = 0;
@@ -187,55 +228,15 @@ void free_model(Model& m) {
   m = Model();
 }
 
-// Scratch sized by n candidates (plus the fixed pieces).
-// The compiled decoder's row buffer: at least `elems` floats on the scratch
-// device (grown, never shrunk; kept until exit).  False when it cannot be
-// had (the caller then decodes inside the walks, which needs no buffer).
-bool try_feat_buf(long long elems) {
-  if (elems <= g_scr.feat_cap) return true;
-  if (g_scr.feat_buf != nullptr) {
-    cudaDeviceSynchronize();
-    cudaFree(g_scr.feat_buf);
-    g_scr.feat_buf = nullptr;
-    g_scr.feat_cap = 0;
-  }
-  void* p = nullptr;
-  if (cudaMalloc(&p, static_cast<size_t>(elems) * sizeof(float)) != cudaSuccess) {
-    cudaGetLastError();  // clear the allocation failure
-    return false;
-  }
-  g_scr.feat_buf = static_cast<float*>(p);
-  g_scr.feat_cap = elems;
-  return true;
-}
-
-// The ordinal buffer: at least `bytes` (grown, kept until the feature count
-// changes or a V or P model is freed).  False where it would be larger than
-// kOrdMaxBytes or cannot be had; the walk then reads the fp32 rows.
+// The ordinal buffer holds at most this; a larger batch walks the fp32 rows.
 constexpr size_t kOrdMaxBytes = 8ull << 30;
 
-void free_ord_buf() {
-  if (g_scr.ord_buf == nullptr) return;
-  cudaDeviceSynchronize();  // queued screens may still read it
-  cudaFree(g_scr.ord_buf);
-  g_scr.ord_buf = nullptr;
-  g_scr.ord_cap = 0;
+void release_buffers() {
+  g_scr.feats.release();
+  g_scr.ord.release();
 }
 
-bool try_ord_buf(size_t bytes) {
-  if (bytes <= g_scr.ord_cap) return true;
-  if (bytes > kOrdMaxBytes) return false;
-  free_ord_buf();
-  void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();  // clear the allocation failure
-    return false;
-  }
-  g_scr.ord_buf = static_cast<unsigned char*>(p);
-  g_scr.ord_cap = bytes;
-  return true;
-}
-
+// Scratch sized by n candidates (plus the fixed pieces).
 int ensure_scratch(long long n) {
   int dev = 0;
   int rc = current_device(&dev);
@@ -535,7 +536,8 @@ struct Pass {
 
 // Plans of both passes over n candidates.  stored: the rows are in memory and
 // the ordinal buffer may be allocated.
-void plan_passes(const DeviceModel& V, const DeviceModel& P, long long n, bool stored, Pass* pv, Pass* pp) {
+void plan_passes(const DeviceModel& V, const DeviceModel& P, long long n, bool stored, cudaStream_t st, Pass* pv,
+                 Pass* pp) {
   const DeviceModel* m[2] = {&V, &P};
   Pass* p[2] = {pv, pp};
   // the P pass walks the survivors; plan it for about half the batch
@@ -547,7 +549,7 @@ void plan_passes(const DeviceModel& V, const DeviceModel& P, long long n, bool s
     p[i]->ord = p[i]->ord && p[i]->shape.threads > 0;
     if (p[i]->ord) bytes = std::max(bytes, ord_bytes(n) + ord_flag_bytes(n));
   }
-  if (bytes > 0 && !try_ord_buf(bytes)) pv->ord = pp->ord = false;
+  if (bytes > 0 && (bytes > kOrdMaxBytes || !g_scr.ord.ensure(bytes, st))) pv->ord = pp->ord = false;
   for (int i = 0; i < 2; ++i)
     if (!p[i]->ord) p[i]->shape = plan_for(*m[i], g_F, n_eff[i], g_shape[i], i == 0);
 }
@@ -577,8 +579,8 @@ cudaError_t launch_pass(const DeviceModel& m, TraverseArgs a, const Pass& p, con
   o.rows = a.p_pass ? a.rows : nullptr;
   o.count = a.p_pass ? &a.state->survivors : nullptr;
   o.stream = a.stream;
-  o.out = reinterpret_cast<uint32_t*>(g_scr.ord_buf);
-  o.nan_flags = g_scr.ord_buf + ord_bytes(n);
+  o.out = static_cast<uint32_t*>(g_scr.ord.p);
+  o.nan_flags = static_cast<unsigned char*>(g_scr.ord.p) + ord_bytes(n);
   o.err = a.err;
   cudaError_t e = launch_ordinals(m.ord, o, n, sm_count(), st);
   if (e != cudaSuccess) return e;
@@ -587,6 +589,7 @@ cudaError_t launch_pass(const DeviceModel& m, TraverseArgs a, const Pass& p, con
   a.ord = o.out;
   a.nan_flags = o.nan_flags;
   a.nan_groups = (g_F + 7) / 8;
+
   return launch_walk_ord(m.depth, a, sh, tiles, st);
 }
 
@@ -603,22 +606,21 @@ int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec
   if (rc != MLT_OK) return rc;
   const DeviceModel& V = g_models[MLT_MODEL_V].dm;
   const DeviceModel& P = g_models[MLT_MODEL_P].dm;
-  // a large decoded batch: the compiled feature program writes its rows
-  // once, and the walks stage them like stored features (the same bits as
-  // decoding inside the walks); top-k positions stay candidate indices
+  // a decoded batch: its rows are written once, by the compiled feature
+  // program where the batch is large, and the walks read them like stored
+  // features (the same bits as decoding inside the walks, which remains where
+  // the buffer cannot be had); top-k positions stay candidate indices
   const long long topk_base = dec ? dec->first_index : 0;
-  const DecodeParams* jit_dec = nullptr;
+  const DecodeParams* rows_dec = nullptr;
   JitDecoder jd{};
-  if (dec != nullptr && g_jit_min_n > 0 && n >= g_jit_min_n) {
-    jd = jit_decoder_for(*dec, dev);
-    if (jd.fn != nullptr && try_feat_buf(n * static_cast<long long>(g_F))) {
-      jit_dec = dec;
-      feats = g_scr.feat_buf;
-      dec = nullptr;
-    }
+  if (dec != nullptr && n > 0 && g_scr.feats.ensure(static_cast<size_t>(n) * g_F * sizeof(float), st)) {
+    if (g_jit_min_n > 0 && n >= g_jit_min_n) jd = jit_decoder_for(*dec, dev);
+    rows_dec = dec;
+    feats = static_cast<const float*>(g_scr.feats.p);
+    dec = nullptr;
   }
   Pass pv, pp;
-  plan_passes(V, P, n, dec == nullptr && !fixed_scratch, &pv, &pp);
+  plan_passes(V, P, n, dec == nullptr && !fixed_scratch, st, &pv, &pp);
   const ScreenShape &sv = pv.shape, &sp = pp.shape;
   if (sv.threads == 0 || sp.threads == 0) return fail(MLT_EINVAL, "F=%d leaves no room for a shared-memory tile", g_F);
   TraverseArgs a{};
@@ -659,14 +661,18 @@ int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec
     g_events_used += kPhases + 1;
     MLT_CUDA(cudaEventRecord(ev[0], st), "cudaEventRecord");
   }
-  if (jit_dec != nullptr) {  // recorded with the V phase
-    MLT_CUDA(launch_jit_decode(jd, *jit_dec, n, g_scr.feat_buf, st), "compiled decoder launch");
+  if (rows_dec != nullptr) {  // recorded with the V phase
+    if (jd.fn != nullptr) {
+      MLT_CUDA(launch_jit_decode(jd, *rows_dec, n, static_cast<float*>(g_scr.feats.p), st), "compiled decoder launch");
+      g_jit_calls += 1;
+    } else {
+      MLT_CUDA(launch_decode_rows(*rows_dec, n, nullptr, static_cast<float*>(g_scr.feats.p), st), "decoder launch");
+    }
     g_launches += 1;
-    g_jit_calls += 1;
   }
   // a small batch of stored features: the whole step in one launch (its
   // time is recorded as the V phase)
-  if (dec == nullptr && jit_dec == nullptr && n <= g_small_max) {
+  if (dec == nullptr && n <= g_small_max) {
     const SmallPlan pl = plan_small(g_F, n, V, P, sm_count(), smem_optin());
     if (pl.threads > 0) {
       int stall = -1;
@@ -676,8 +682,8 @@ int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec
         stall_ns = g_stall_ns;
         g_stall_cta = -1;
       }
-      MLT_CUDA(launch_screen_small(pl, V, P, feats, g_F, n, a.tau, out_pvalid, out_perf, out_topk, k, s, stall,
-                                   stall_ns, st),
+      MLT_CUDA(launch_screen_small(pl, V, P, feats, g_F, n, a.tau, out_pvalid, out_perf, out_topk, topk_base, k, s,
+                                   stall, stall_ns, st),
                "small-batch screening launch");
       if (ev)
         for (int i = 1; i <= kPhases; ++i) MLT_CUDA(cudaEventRecord(ev[i], st), "cudaEventRecord");
@@ -757,8 +763,10 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
   const DeviceModel& V = g_models[MLT_MODEL_V].dm;
   const DeviceModel& P = g_models[MLT_MODEL_P].dm;
   const long long per = std::min(batch, std::max(1LL, n_total));
+  // decoded batches: each batch's rows are written first, as in run_screen_with
+  const bool rows = dec0 != nullptr && per > 0 && g_scr.feats.ensure(static_cast<size_t>(per) * g_F * sizeof(float), st);
   Pass pv, pp;
-  plan_passes(V, P, per, dec0 == nullptr, &pv, &pp);
+  plan_passes(V, P, per, dec0 == nullptr || rows, st, &pv, &pp);
   const ScreenShape &sv = pv.shape, &sp = pp.shape;
   if (sv.threads == 0 || sp.threads == 0) return fail(MLT_EINVAL, "F=%d leaves no room for a shared-memory tile", g_F);
   MLT_CUDA(cudaMemsetAsync(s.state, 0, sizeof(SelectState), st), "reset selection state");
@@ -776,7 +784,7 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
   a.tile_offsets = s.tile_offsets;
   a.state_rw = s.state;
   a.err = s.err;
-  a.decode = dec0 != nullptr;
+  a.decode = dec0 != nullptr && !rows;
   a.stream = ss;
   long long launches = 0;
   for (long long b0 = 0; b0 < n_total; b0 += batch) {
@@ -784,7 +792,7 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
     TraverseArgs ab = a;
     ab.n = nb;
     ab.pos_base = b0;
-    ab.feats = feats ? feats + b0 * g_F : nullptr;
+    ab.feats = rows ? static_cast<const float*>(g_scr.feats.p) : feats ? feats + b0 * g_F : nullptr;
     ab.vec4 = (ab.feats != nullptr && (reinterpret_cast<uintptr_t>(ab.feats) & 15u) == 0 && (g_F & 3) == 0) ? 1 : 0;
     ab.out_pvalid = out_pvalid ? out_pvalid + b0 : nullptr;
     ab.out_perf = out_perf ? out_perf + b0 : nullptr;
@@ -793,14 +801,19 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
       d = *dec0;
       d.first_index += b0;
     }
+    const DecodeParams* walk_dec = dec0 && !rows ? &d : nullptr;
+    if (rows) {
+      MLT_CUDA(launch_decode_rows(d, nb, nullptr, static_cast<float*>(g_scr.feats.p), st, ss), "decoder launch");
+      launches += 1;
+    }
     TraverseArgs av = ab;
     av.p_pass = 0;
     const long long tiles_v = (nb + sv.threads - 1) / sv.threads;
-    MLT_CUDA(launch_pass(V, av, pv, dec0 ? &d : nullptr, nb, st, &launches), "V pass launch");
+    MLT_CUDA(launch_pass(V, av, pv, walk_dec, nb, st, &launches), "V pass launch");
     MLT_CUDA(launch_compact(s, nb, sv.threads, tiles_v, ss, st), "compaction launch");
     TraverseArgs ap = ab;
     ap.p_pass = 1;
-    MLT_CUDA(launch_pass(P, ap, pp, dec0 ? &d : nullptr, nb, st, &launches), "P pass launch");
+    MLT_CUDA(launch_pass(P, ap, pp, walk_dec, nb, st, &launches), "P pass launch");
     MLT_CUDA(launch_accumulate(ss, s.state, nb, tgt, st), "accumulate launch");
     launches += 2;
   }
@@ -1074,7 +1087,7 @@ int mlt_set_num_features(int F) {
   std::lock_guard<std::mutex> lk(g_mu);
   if (F != g_F) {
     for (Model& m : g_models) free_model(m);
-    free_ord_buf();
+    release_buffers();
   }
   g_F = F;
   return MLT_OK;
@@ -1153,7 +1166,7 @@ int mlt_free_ensemble(int model_id) {
   if (model_id < MLT_MODEL_V || model_id > MLT_MODEL_A) return fail(MLT_EINVAL, "unknown model id %d", model_id);
   std::lock_guard<std::mutex> lk(g_mu);
   free_model(g_models[model_id]);
-  if (model_id != MLT_MODEL_A) free_ord_buf();
+  if (model_id != MLT_MODEL_A) release_buffers();
   return MLT_OK;
 }
 

@@ -360,8 +360,9 @@ cudaError_t launch_traverse(const DeviceModel& m, const TraverseArgs& args,
 cudaError_t launch_traverse_dec(const DeviceModel& m, const TraverseArgs& args,
                                 const DecodeParams& dec, const ScreenShape& shape,
                                 long long n_tiles, cudaStream_t st);
+// ss: batched accumulation, a batch after the target writes nothing (may be null)
 cudaError_t launch_decode_rows(const DecodeParams& dec, long long n, uint8_t* out_knobs,
-                               float* out_feats, cudaStream_t st);
+                               float* out_feats, cudaStream_t st, const StreamState* ss = nullptr);
 // Decoded batches of at least this many candidates build their rows with the
 // compiled feature program by default (mlt_tune_decode_jit changes it).
 constexpr long long kDecodeJitMinN = 1LL << 20;
@@ -439,7 +440,7 @@ struct SmallPlan {
 SmallPlan plan_small(int F, long long n, const DeviceModel& V, const DeviceModel& P, int sms, int device_smem_optin);
 cudaError_t launch_screen_small(const SmallPlan& pl, const DeviceModel& V, const DeviceModel& P, const float* feats,
                                 int F, long long n, float tau, float* out_pvalid, float* out_perf, int64_t* out_topk,
-                                int k, const Scratch& sc, int stall_cta, unsigned long long stall_ns,
+                                long long index_base, int k, const Scratch& sc, int stall_cta, unsigned long long stall_ns,
                                 cudaStream_t st);
 
 // selftest.cu: a bounded wait that runs out (failure-detection self-test)

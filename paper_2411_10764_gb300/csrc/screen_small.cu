@@ -47,6 +47,7 @@ struct SmallArgs {
   float* out_pvalid;
   float* out_perf;
   int64_t* out_topk;
+  long long base;  // candidate index of row 0
   int k;
   unsigned long long* keys;  // [n] scratch
   SelectState* state;        // survivors and ticket (zeroed before the launch)
@@ -113,7 +114,7 @@ __device__ __forceinline__ void select_small(const SmallArgs& s, unsigned m, uns
     if (m <= kSmallRankMax) {
       if (tid == 0 && (m & 1u)) ks[m] = 0ull;
       __syncthreads();
-      rank_and_write(ks, m, kk, 0, s.out_topk);
+      rank_and_write(ks, m, kk, s.base, s.out_topk);
     } else {
       lo = __reduce_min_sync(0xFFFFFFFFu, lo);
       hi = __reduce_max_sync(0xFFFFFFFFu, hi);
@@ -185,7 +186,7 @@ __device__ __forceinline__ void select_small(const SmallArgs& s, unsigned m, uns
       if (cnt <= kSmallRankMax) {
         if (tid == 0 && (cnt & 1u)) cs[cnt] = 0ull;
         __syncthreads();
-        rank_and_write(cs, cnt, kk, 0, s.out_topk);
+        rank_and_write(cs, cnt, kk, s.base, s.out_topk);
       } else {
         // a crowded bin: order every key
         int n2 = 2;
@@ -194,7 +195,7 @@ __device__ __forceinline__ void select_small(const SmallArgs& s, unsigned m, uns
         __syncthreads();
         sort_desc(ks, n2);
         for (unsigned r = tid; r < kk; r += T)
-          s.out_topk[r] = static_cast<int64_t>(0xFFFFFFFFu - static_cast<uint32_t>(ks[r] & 0xFFFFFFFFull));
+          s.out_topk[r] = s.base + static_cast<int64_t>(0xFFFFFFFFu - static_cast<uint32_t>(ks[r] & 0xFFFFFFFFull));
       }
     }
   }
@@ -342,7 +343,7 @@ SmallPlan plan_small(int F, long long n, const DeviceModel& V, const DeviceModel
 
 cudaError_t launch_screen_small(const SmallPlan& pl, const DeviceModel& V, const DeviceModel& P, const float* feats,
                                 int F, long long n, float tau, float* out_pvalid, float* out_perf, int64_t* out_topk,
-                                int k, const Scratch& sc, int stall_cta, unsigned long long stall_ns,
+                                long long index_base, int k, const Scratch& sc, int stall_cta, unsigned long long stall_ns,
                                 cudaStream_t st) {
   SmallKernelPtr kern = pl.groups == 8 ? small_for_depth<8>(V.depth) : pl.groups == 4 ? small_for_depth<4>(V.depth)
                                                                                          : nullptr;
@@ -361,6 +362,7 @@ cudaError_t launch_screen_small(const SmallPlan& pl, const DeviceModel& V, const
   s.out_pvalid = out_pvalid;
   s.out_perf = out_perf;
   s.out_topk = out_topk;
+  s.base = index_base;
   s.k = k;
   s.keys = sc.keys;
   s.state = sc.state;

@@ -452,8 +452,8 @@ def walk_shape(model_id: int, n: int, p_pass: bool = False) -> dict:
 
 def tune_decode_jit(min_n: int) -> None:
     """Decoded batches of at least min_n candidates build their rows with
-    the feature program compiled at run time (NVRTC) and screen those; 0
-    keeps every decoded batch on the interpreted in-walk path."""
+    the feature program compiled at run time (NVRTC); 0 keeps every decoded
+    batch on the interpreted program."""
     _check(lib().mlt_tune_decode_jit(int(min_n)))
 
 
