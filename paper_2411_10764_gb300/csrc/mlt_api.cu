@@ -521,7 +521,7 @@ constexpr int kOrdMinVisits = 16;  // per feature
 bool ord_wanted(const DeviceModel& m, const ShapeOverride& ov, long long n) {
   if (m.ord.table == nullptr || n < kOrdMinN) return false;
   if (ov.threads || ov.chunk_trees || ov.nbuf || ov.lanes || ov.group) return false;  // a fixed shape of the fp32 walk
-  return static_cast<long long>(m.n_trees) * m.depth >= static_cast<long long>(kOrdMinVisits) * g_F;
+  return m.ord.visits >= static_cast<float>(kOrdMinVisits) * g_F;
 }
 
 // Bytes of the ordinals of n candidates, and of their missing-value flags.
@@ -589,7 +589,8 @@ cudaError_t launch_pass(const DeviceModel& m, TraverseArgs a, const Pass& p, con
   a.ord = o.out;
   a.nan_flags = o.nan_flags;
   a.nan_groups = (g_F + 7) / 8;
-
+  a.tail = reinterpret_cast<const uint2*>(m.ord.tail);
+  a.max_depth = m.ord.rounds;
   return launch_walk_ord(m.depth, a, sh, tiles, st);
 }
 
@@ -1071,6 +1072,7 @@ int install_model(int model_id, const std::vector<unsigned char>& packed, const 
   OrdTable& o = m.dm.ord;
   if (o.n_trees > 0) {
     o.table = d + o.off_table;
+    o.tail = reinterpret_cast<const uint4*>(d + o.off_tail);
     o.image = d + o.off_image;
     o.features = reinterpret_cast<const OrdFeature*>(d + o.off_features);
     o.groups = reinterpret_cast<const OrdGroup*>(d + o.off_groups);
@@ -1108,7 +1110,8 @@ int mlt_load_ensemble(int model_id, const mlt_node* nodes, int n_trees, int dept
   int rc = split ? pack_split(nodes, n_trees, depth, g_F, g_head_levels, packed, dm)
                  : pack_ensemble(nodes, n_trees, depth, g_F, packed, dm);
   if (rc != MLT_OK) return rc;
-  if (dm.kind == kTableFull && model_id != MLT_MODEL_A) pack_ordinal(nodes, n_trees, depth, g_F, false, packed, dm.ord);
+  if ((dm.kind == kTableFull || dm.kind == kTableSplit) && model_id != MLT_MODEL_A)
+    pack_ordinal(nodes, n_trees, depth, g_F, false, packed, dm.ord);
   return install_model(model_id, packed, dm);
 }
 

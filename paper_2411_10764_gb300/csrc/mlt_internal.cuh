@@ -138,6 +138,9 @@ constexpr uint32_t kCompactChildShift = 10;       // bits 10..29
 constexpr uint32_t kCompactChildMask = 0xFFFFFu;
 
 // Ordinal form of a full or half table (ordinal.cuh has the layout).
+constexpr int kOrdHead = 6;             // levels of a deep model's tree in shared memory
+constexpr uint32_t kOrdExitLeaf = 0x80000000u;
+constexpr int kOrdBlockBits = 25;       // block index in a tail block's word 0
 constexpr int kOrdTreePad = 4;        // trees are padded to a multiple of this
 constexpr int kOrdMaxDistinct = 8191;  // distinct thresholds per feature
 constexpr int kOrdMaxBuckets = 2048;   // buckets of a feature's lookup table
@@ -165,7 +168,10 @@ struct OrdTable {
   const unsigned char* image = nullptr;
   const OrdFeature* features = nullptr;
   const OrdGroup* groups = nullptr;
-  size_t off_table = 0, off_image = 0, off_features = 0, off_groups = 0;  // in the model's allocation
+  const uint4* tail = nullptr;  // deep models: blocks below the heads
+  float visits = 0;  // node tests a candidate is expected to meet
+  int rounds = 0;    // deep models: most blocks on a path (0: a full table)
+  size_t off_tail = 0, off_table = 0, off_image = 0, off_features = 0, off_groups = 0;  // in the model's allocation
   int n_trees = 0;         // padded
   int n_groups = 0;
   uint32_t max_bytes = 0;  // of a group's image

@@ -15,6 +15,8 @@ using namespace walk;
 constexpr int kOrdThreads = 1024;
 constexpr int kOrdRows = 2;  // blocks of 32 rows a warp takes together
 constexpr int kOrdMaxCta = 1024;
+constexpr int kOrdDeepUnit = 8;    // trees a tree group takes at a time
+constexpr int kOrdDeepFlight = 4;  // trees a thread walks at once
 constexpr size_t kSmPerSm = 228 * 1024;
 constexpr size_t kCtaReserve = 1024;
 constexpr size_t kStaticSmem = 1024;
@@ -178,6 +180,34 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
   }
 }
 
+// The ordinal that a node word tests (xw: the candidate's column).
+__device__ __forceinline__ uint32_t ord_at(const unsigned char* xw, uint32_t w) {
+  return ld_sm<unsigned short>(xw, w & 0xFFFEu);
+}
+// Heap index of the child that ordinal x takes below node i; a missing x
+// (kOrdNan) becomes 0 where the word's flag sends it left.
+template <bool NANP>
+__device__ __forceinline__ uint32_t ord_child(uint32_t i, uint32_t w, uint32_t x) {
+  if (NANP) x &= ~(w << 15);
+  return __funnelshift_l(w - x * 65536u, i, 1);
+}
+// The same for a deep model's words, whose flag is at kOrdNan's bit.
+__device__ __forceinline__ uint32_t deep_at(const unsigned char* xw, uint32_t w) {
+  return ld_sm<unsigned short>(xw, w & 0x7FFEu);
+}
+template <bool NANP>
+__device__ __forceinline__ uint32_t deep_child(uint32_t i, uint32_t w, uint32_t x) {
+  if (NANP) x &= ~(w & kOrdNan);
+  return __funnelshift_l(w - x * 65536u, i, 1);
+}
+
+// A 32-byte block (one sector), kept in L2.
+__device__ __forceinline__ void ldg_block(const uint4* ptr, unsigned long long pol, uint32_t (&b)[8]) {
+  asm("ld.global.nc.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
+      : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7])
+      : "l"(ptr), "l"(pol));
+}
+
 // Leaves of G consecutive trees at tb for one candidate (its column of
 // ordinals at xw).
 template <int D, int G, bool NANP>
@@ -192,12 +222,9 @@ __device__ __forceinline__ void walk_ord(const unsigned char* tb, const unsigned
 #pragma unroll
     for (int g = 0; g < G; ++g) w[g] = ld_sm<uint32_t>(tb, g * kTree + j[g] * 4u);
 #pragma unroll
-    for (int g = 0; g < G; ++g) x[g] = ld_sm<unsigned short>(xw, w[g] & 0xFFFEu);
+    for (int g = 0; g < G; ++g) x[g] = ord_at(xw, w[g]);
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      if (NANP) x[g] &= ~(w[g] << 15);  // kOrdNan becomes 0 where a missing value goes left
-      j[g] = __funnelshift_l(w[g] - x[g] * 65536u, j[g], 1);
-    }
+    for (int g = 0; g < G; ++g) j[g] = ord_child<NANP>(j[g], w[g], x[g]);
   }
 #pragma unroll
   for (int g = 0; g < G; ++g) leaf[g] = ld_sm<float>(tb, g * kTree + j[g] * 4u);
@@ -214,6 +241,89 @@ __device__ __forceinline__ void walk_ord_unit(const unsigned char* tb, int nt, c
     else if (nt > t)
       walk_ord<D, 4, NANP>(tb + t * kTree, xw, leaf + t);
   }
+}
+
+// Leaves of G consecutive trees of a deep model: H head levels and the exit
+// from shared memory, then `rounds` blocks of three levels from global memory.
+// Every walker runs every round -- some lane of a warp nearly always goes to
+// the bottom, and a vote per round would tie the G walkers' loads together; a
+// walker that has its leaf reads block 0, one line for all of them.  Bound: the
+// L1 data pipe, about 23 wavefronts a warp and tree for the head and 38 for
+// the tail (4,194,304 x 256, 1,000 trees of depth 12: 73 cycles a warp and tree
+// on an SM, where the split table's 8-byte records took 94).
+template <int H, int G, bool NANP>
+__device__ __forceinline__ void walk_ord_deep(const unsigned char* tb, const unsigned char* xw, const uint4* tail,
+                                              int rounds, float* leaf) {
+  constexpr uint32_t kTree = ord_head_bytes(H);
+  uint32_t j[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) j[g] = 1u;
+#pragma unroll
+  for (int l = 0; l < H; ++l) {
+    uint32_t w[G], x[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) w[g] = ld_sm<uint32_t>(tb, g * kTree + j[g] * 4u);
+#pragma unroll
+    for (int g = 0; g < G; ++g) x[g] = deep_at(xw, w[g]);
+#pragma unroll
+    for (int g = 0; g < G; ++g) j[g] = deep_child<NANP>(j[g], w[g], x[g]);
+  }
+  uint32_t val[G], at[G];
+  bool live[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    // exit j - 2^H of the tree: 8 bytes at (4 << H) + 8 (j - 2^H)
+    const uint2 e = ld_sm<uint2>(tb, g * kTree + j[g] * 8u - (4u << H));
+    live[g] = !(e.y & kOrdExitLeaf);
+    val[g] = e.x;
+    const uint32_t w = live[g] ? e.x : 0u;  // a leaf's bits are no index
+    at[g] = live[g] ? e.y + (deep_child<NANP>(0u, w, deep_at(xw, w)) & 1u) : 0u;
+  }
+  const unsigned long long keep = policy_evict_last();
+  for (int s = 0; s < rounds; ++s) {
+    uint32_t b[G][8], i[G], w[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) ldg_block(tail + 2ull * at[g], keep, b[g]);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      i[g] = 1u;
+      w[g] = b[g][1];
+    }
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      uint32_t x[G];
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const bool is_leaf = ((b[g][0] >> i[g]) & (1u << (kOrdBlockBits - 1))) != 0u;
+        if (is_leaf && live[g]) val[g] = w[g];
+        live[g] = live[g] && !is_leaf;
+        w[g] = is_leaf ? 0u : w[g];
+        x[g] = deep_at(xw, w[g]);
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        i[g] = deep_child<NANP>(i[g], w[g], x[g]);
+        if (l == 0) w[g] = (i[g] & 1u) ? b[g][3] : b[g][2];
+        if (l == 1) {
+          const uint32_t lo = (i[g] & 1u) ? b[g][5] : b[g][4], hi = (i[g] & 1u) ? b[g][7] : b[g][6];
+          w[g] = (i[g] & 2u) ? hi : lo;
+        }
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) at[g] = live[g] ? (b[g][0] & ((1u << kOrdBlockBits) - 1u)) + i[g] - 8u : 0u;
+  }
+#pragma unroll
+  for (int g = 0; g < G; ++g) leaf[g] = __uint_as_float(val[g]);
+}
+
+// Leaves of nt <= U trees (a multiple of 4) of a deep model.
+template <int H, int U, int G, bool NANP>
+__device__ __forceinline__ void walk_deep_unit(const unsigned char* tb, int nt, const unsigned char* xw,
+                                               const uint4* tail, int rounds, float* leaf) {
+#pragma unroll
+  for (int t = 0; t < U; t += G)
+    if (nt > t) walk_ord_deep<H, G, NANP>(tb + t * ord_head_bytes(H), xw, tail, rounds, leaf + t);
 }
 
 // One tree group: trees [0, nt) of a chunk, leaves added in tree order.
@@ -239,15 +349,15 @@ __device__ __forceinline__ float walk_ord_sum(const unsigned char* tb, int nt, c
 struct OrdSmem {
   size_t rows, sums, tbuf, bars, bytes;
 };
-// Q > 1 tree groups: the candidates' running sums and a barrier per group and
-// 32 candidates.
+// Q > 0: tree groups that hand the sums on (the candidates' running sums and a
+// barrier per group and 32 candidates); 0: one group that keeps them.
 __host__ __device__ inline OrdSmem ord_smem(int F, int TC, int Q, int nbuf, uint32_t chunk_bytes) {
   OrdSmem s;
   s.rows = static_cast<size_t>((F + 1) / 2) * TC * 4;  // a multiple of 128: TC is one of 32
   s.sums = s.rows + static_cast<size_t>(TC) * 4;
-  s.tbuf = align_up(s.sums + (Q > 1 ? static_cast<size_t>(TC) * 4 : 0), 128);
+  s.tbuf = align_up(s.sums + (Q > 0 ? static_cast<size_t>(TC) * 4 : 0), 128);
   s.bars = s.tbuf + static_cast<size_t>(nbuf) * chunk_bytes;
-  s.bytes = s.bars + 10 * 8 + (Q > 1 ? static_cast<size_t>(TC / 32) * Q * 8 : 0);
+  s.bytes = s.bars + 10 * 8 + static_cast<size_t>(TC / 32) * Q * 8;
   return s;
 }
 
@@ -300,7 +410,8 @@ __device__ __forceinline__ uint32_t mbar_arrive_pending(uint32_t bar) {
 // multiply the warps where a tile's candidates alone leave an SM too few.
 // Bound: shared-memory wavefronts (one per ordinal gather, one to 3.4 per node
 // gather) and issue.
-template <int D, int U>
+// DEEP: a deep model's heads (D head levels) and tail.
+template <int D, int U, int DEEP = 0>
 __global__ void __launch_bounds__(kOrdMaxCta, 1) k_walk_ord(const __grid_constant__ TraverseArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int last_issued[4];  // latest chunk copied into each buffer
@@ -316,9 +427,9 @@ __global__ void __launch_bounds__(kOrdMaxCta, 1) k_walk_ord(const __grid_constan
   ord_tile(a, count, TC, &tile0, &rows_here);
   if (rows_here <= 0) return;  // whole CTA, before any copy is issued
 
-  constexpr uint32_t kTree = ord_tree_bytes(D);
+  constexpr uint32_t kTree = DEEP ? ord_head_bytes(D) : ord_tree_bytes(D);
   const uint32_t chunk_bytes = static_cast<uint32_t>(a.chunk_trees) * kTree;
-  const OrdSmem L = ord_smem(a.F, TC, Q, a.nbuf, chunk_bytes);
+  const OrdSmem L = ord_smem(a.F, TC, kGroups ? Q : 0, a.nbuf, chunk_bytes);
   uint32_t* rowidx = reinterpret_cast<uint32_t*>(smem + L.rows);
   float* sums = reinterpret_cast<float*>(smem + L.sums);
   unsigned char* tbuf = smem + L.tbuf;
@@ -386,7 +497,14 @@ __global__ void __launch_bounds__(kOrdMaxCta, 1) k_walk_ord(const __grid_constan
         for (int t = q * U; t < nt; t += Q * U) {
           float leaf[U];
           const int here = min(U, nt - t);
-          if (nan)
+          if constexpr (DEEP > 0) {
+            const unsigned char* tt = tb + static_cast<uint32_t>(t) * kTree;
+            const uint4* tail = reinterpret_cast<const uint4*>(a.tail);
+            if (nan)
+              walk_deep_unit<D, U, DEEP, true>(tt, here, xw, tail, a.max_depth, leaf);
+            else
+              walk_deep_unit<D, U, DEEP, false>(tt, here, xw, tail, a.max_depth, leaf);
+          } else if (nan)
             walk_ord_unit<D, U, true>(tb + static_cast<uint32_t>(t) * kTree, here, xw, leaf);
           else
             walk_ord_unit<D, U, false>(tb + static_cast<uint32_t>(t) * kTree, here, xw, leaf);
@@ -496,6 +614,57 @@ cudaError_t launch_ordinals(const OrdTable& t, OrdArgs a, long long n_max, int s
   return launch_pdl(k, dim3(a.first_cta[t.n_groups]), dim3(kOrdThreads), smem, st, a);
 }
 
+// Shape of the ordinal walk over a deep model: a warp's tree waits on its tail
+// loads, so the shape that puts the most warps on the busiest SM's candidates,
+// then the largest tile (each tile streams every head).  Measured V passes of
+// 4,194,304 x 256, 1,000 trees of depth 12: 33.3 ms with 256 candidates x 4
+// groups, 34.5 with 192 x 4, 37.9 with 256 x 2, 38.3 with 128 x 2 twice an SM.
+ScreenShape plan_ord_deep(int F, const OrdTable& t, long long n_eff, int sms, int optin) {
+  ScreenShape best{};
+  if (sms < 1) sms = 1;
+  if (n_eff < 1) n_eff = 1;
+  const uint32_t tb = ord_head_bytes(kOrdHead);
+  double best_cost = 1e300;
+  for (int tc = 32; tc <= 512; tc += 32) {
+    for (int q : {1, 2, 3, 4, 6, 8}) {
+      if (tc * q > kOrdMaxCta) continue;
+      for (int ch = 48; ch >= 8; ch -= 8) {
+        if (ch % (kOrdDeepUnit * q) != 0) continue;
+        for (int nb : {2, 3}) {
+          const size_t smem = ord_smem(F, tc, q, nb, static_cast<uint32_t>(ch) * tb).bytes;
+          if (smem + kStaticSmem > static_cast<size_t>(optin)) continue;
+          const long long tiles = (n_eff + tc - 1) / tc;
+          const long long tiles_sm = (tiles + sms - 1) / sms;
+          const long long fit =
+              std::min<long long>({static_cast<long long>(kSmPerSm / (smem + kStaticSmem + kCtaReserve)),
+                                   2048 / (tc * q), 65536 / (tc * q * 64)});
+          if (fit < 1) continue;
+          const long long res = std::min(fit, tiles_sm);
+          const double warps = static_cast<double>(res) * tc * q / 32;
+          const double tree = 45.0 + 400.0 / warps + tb / 128.0 / (tc / 32.0) * 2.0;
+          const double chunks = std::ceil(static_cast<double>(t.n_trees) / ch);
+          const double cost = static_cast<double>(tiles_sm) * (tc / 32.0 * t.n_trees * tree + chunks * 500.0 / (res * res) +
+                                                               (res == 1 ? 6000.0 : 2000.0 / res)) +
+                              40.0 * nb;
+          if (cost < best_cost) {
+            best_cost = cost;
+            best.threads = tc;
+            best.smem = smem;
+            best.chunk_trees = ch;
+            best.nbuf = nb;
+            best.group = kOrdDeepFlight;
+            best.lanes = q;
+            best.resident = static_cast<int>(res);
+            best.p_grid = sms * static_cast<int>(res);
+          }
+        }
+      }
+    }
+  }
+  if (best.threads) best = cap_residency(best, optin);
+  return best;
+}
+
 // Candidates per CTA, tree groups, trees per chunk and buffers of the ordinal
 // walk: the shape with the least estimated cycles of the busiest SM.  Fitted
 // to sweeps on GB300 (65,536 x 64 and 1,048,576 x 128, depth 8; 16,700,000 x
@@ -508,6 +677,7 @@ cudaError_t launch_ordinals(const OrdTable& t, OrdArgs a, long long n_max, int s
 // together, and a tile's start about 6,000 cycles: another resident CTA hides
 // both.
 ScreenShape plan_ord(int F, const OrdTable& t, int depth, long long n_eff, int sms, int optin) {
+  if (t.rounds > 0) return plan_ord_deep(F, t, n_eff, sms, optin);
   ScreenShape best{};
   if (sms < 1) sms = 1;
   if (n_eff < 1) n_eff = 1;
@@ -522,7 +692,7 @@ ScreenShape plan_ord(int F, const OrdTable& t, int depth, long long n_eff, int s
         const int unit = ord_unit(ch, q);
         if (unit < 0) continue;
         for (int nb : {2, 3}) {
-          const size_t smem = ord_smem(F, tc, q, nb, static_cast<uint32_t>(ch) * tb).bytes;
+          const size_t smem = ord_smem(F, tc, q > 1 ? q : 0, nb, static_cast<uint32_t>(ch) * tb).bytes;
           if (smem + kStaticSmem > static_cast<size_t>(optin)) continue;
           const long long tiles = (n_eff + tc - 1) / tc;
           const long long tiles_sm = (tiles + sms - 1) / sms;
@@ -568,7 +738,8 @@ cudaError_t launch_walk_ord(int depth, const TraverseArgs& args, const ScreenSha
     a.p_wave = shape.p_grid;
     ctas = (n_tiles + shape.p_grid - 1) / shape.p_grid * shape.p_grid;
   }
-  FullKernelPtr k = ord_kernel(depth, ord_unit(shape.chunk_trees, shape.lanes));
+  FullKernelPtr k = depth > kMaxFullDepth ? k_walk_ord<kOrdHead, kOrdDeepUnit, kOrdDeepFlight>
+                                          : ord_kernel(depth, ord_unit(shape.chunk_trees, shape.lanes));
   if (k == nullptr) return cudaErrorInvalidValue;
   cudaError_t e =
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(shape.smem));

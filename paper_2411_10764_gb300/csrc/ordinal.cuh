@@ -17,15 +17,25 @@
 // kOrdNan.
 //
 // Node word: ordinal i (15 bits) << 16 | byte offset of the feature in a block
-// ((f >> 1) * 128 + (f & 1) * 2) | NaN-goes-left flag (bit 0).  With x the
-// feature's ordinal, the sign of word - (x << 16) is the branch: set iff
-// x > i (the low 16 bits of the word never reach the sign).  kOrdNan << 16 is
-// the sign bit, so a missing x goes right; the flag clears it to 0, which
-// goes left.
+// ((f >> 1) * 128 + (f & 1) * 2) | NaN-goes-left flag (bit 0; bit 15 in a deep
+// model).  With x the feature's ordinal, the sign of word - (x << 16) is the
+// branch: set iff x > i (the low 16 bits of the word never reach the sign).
+// kOrdNan << 16 is the sign bit, so a missing x goes right; the flag clears it
+// to 0, which goes left.
 //
 // Tree: 2^(D+1) words, node j (1-based heap index) at word j, the leaf of
 // child index c (2^D <= c) as an fp32 at word c; word 0 is unused.  Trees are
 // padded with zero trees (leaves +0) to a multiple of kOrdTreePad.
+//
+// Deep models (depth > kMaxFullDepth): the first H = kOrdHead levels of a tree
+// are such a heap, streamed through shared memory; then come 2^H exits of 8
+// bytes: a leaf {fp32, kOrdExitLeaf}, or the level-H split {word, index of the
+// block of its left child; the right child's follows}.  The rest of a tree
+// stays in global memory as 32-byte blocks of three levels (one sector, one
+// load): word 0 = index of the first of 8 child blocks | leaf flags of nodes
+// 1 .. 7 << kOrdBlockBits, words 1 .. 7 = a 3-level heap of node words or fp32
+// leaves.  A path that leaves the head takes one load per three levels, where
+// 8-byte records took one per level.
 //
 // Search of a feature's ordinal: its distinct thresholds in ascending order,
 // padded with NaN (never <= x), and a lookup table of buckets: lut[b] =
@@ -46,7 +56,9 @@
 namespace mlt {
 
 __host__ __device__ constexpr uint32_t ord_tree_bytes(int D) { return 8u << D; }
+__host__ __device__ constexpr uint32_t ord_head_bytes(int H) { return 12u << H; }
 __host__ __device__ constexpr uint32_t ord_offset(uint32_t f) { return (f >> 1) * 128u + (f & 1u) * 2u; }
+constexpr int kOrdDeepMaxF = 512;  // offsets below bit 15
 
 struct OrdArgs {
   const float* feats;      // [n][F]
@@ -66,8 +78,7 @@ struct OrdArgs {
   unsigned short first_cta[kOrdMaxGroups + 1];  // CTAs [first_cta[g], first_cta[g + 1]) take group g
 };
 
-// ordinal_pack.cu: appends the ordinal form of a validated ensemble of depth
-// <= kMaxFullDepth to `out` and describes it in t (offsets into `out`).
+// ordinal_pack.cu: appends the ordinal form of a validated ensemble to `out` and describes it in t (offsets into `out`).
 // round_half: thresholds, leaves and features rounded to binary16.  False
 // when a feature has too many distinct thresholds (or one of -inf).
 bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,

@@ -94,16 +94,17 @@ void for_features(int n, F&& body) {
 bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
                   std::vector<unsigned char>& out, OrdTable& t) {
   const int slots = (2 << depth) - 1;
-  const int inner = (1 << depth) - 1;
+  const bool deep = depth > kMaxFullDepth;
   const int padded = (n_trees + kOrdTreePad - 1) / kOrdTreePad * kOrdTreePad;
-  const uint32_t tree_words = ord_tree_bytes(depth) / 4;
+  if (deep && F > kOrdDeepMaxF) return false;
+  const uint32_t tree_words = (deep ? ord_head_bytes(kOrdHead) : ord_tree_bytes(depth)) / 4;
   auto value = [&](const mlt_node& nd) {
     return round_half ? __half2float(__float2half_rn(nd.value)) : nd.value;
   };
   std::vector<uint32_t> words(static_cast<size_t>(padded) * tree_words, 0u);
 
-  // leaves and passed-through nodes; the split nodes of each feature as
-  // (threshold's order key, word index)
+  // the tables with every word but the ordinals, and the split nodes of each
+  // feature as (threshold's order key, word index)
   std::vector<uint32_t> per_feature(F + 1, 0u);
   std::vector<unsigned char> reach(slots);
   std::vector<float> inherit(slots);
@@ -113,26 +114,104 @@ bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool rou
     uint32_t word;
   };
   std::vector<Split> splits;
-  if (words.size() > 0xFFFFFFFFull) return false;
-  for (int tr = 0; tr < n_trees; ++tr) {
+  std::vector<uint32_t> blocks;  // deep: the tail
+  struct Root {
+    uint32_t block;
+    int node;
+  };
+  std::vector<Root> queue;
+  bool usable = words.size() < 0x7FFFFFFFull;
+  double visits = 0.0;
+  auto put_split = [&](const mlt_node& nd, int j, size_t word, uint32_t* at) {
+    const float v = value(nd);
+    usable = usable && v != -INFINITY;  // every number is >= it: no ordinal stands for that
+    splits.push_back({static_cast<uint32_t>(nd.feature), order_key(v), static_cast<uint32_t>(word)});
+    ++per_feature[nd.feature];
+    *at = ord_offset(nd.feature) | (nd.default_left ? (deep ? kOrdNan : 1u) : 0u);
+    int level = 0;
+    while ((2 << level) - 1 <= j) ++level;
+    visits += std::ldexp(1.0, -level);  // share of the candidates that a random path brings here
+  };
+  const int levels = deep ? kOrdHead : depth;  // of the complete heap
+  const int inner = (1 << levels) - 1;
+  const size_t tail_word = words.size();  // the tail follows the heads
+  for (int tr = 0; tr < n_trees && usable; ++tr) {
     const mlt_node* nd = nodes + static_cast<size_t>(tr) * slots;
     const size_t base = static_cast<size_t>(tr) * tree_words;
     std::fill(reach.begin(), reach.end(), 0);
     reach[0] = 1;
-    for (int j = 0; j < slots; ++j) {
+    for (int j = 0; j < slots; ++j)
+      if (reach[j] && nd[j].feature >= 0) reach[2 * j + 1] = reach[2 * j + 2] = 1;
+    queue.clear();
+    auto new_blocks = [&](uint32_t count) {
+      const uint32_t first = static_cast<uint32_t>(blocks.size() / 8);
+      blocks.resize(blocks.size() + 8 * count, 0u);
+      return first;
+    };
+    for (int j = 0; j < 2 * inner + 1; ++j) {
       const bool split = reach[j] && nd[j].feature >= 0;
-      if (split) {
-        reach[2 * j + 1] = reach[2 * j + 2] = 1;
-        const float v = value(nd[j]);
-        if (v == -INFINITY) return false;  // every number is >= it: no ordinal stands for that
-        splits.push_back({static_cast<uint32_t>(nd[j].feature), order_key(v), static_cast<uint32_t>(base + j + 1)});
-        ++per_feature[nd[j].feature];
-        words[base + j + 1] = ord_offset(nd[j].feature) | (nd[j].default_left ? 1u : 0u);
-      }
       inherit[j] = !reach[j] ? inherit[(j - 1) / 2] : split ? 0.0f : value(nd[j]);
-      if (j >= inner) std::memcpy(&words[base + j + 1], &inherit[j], 4);
+      if (j < inner) {
+        if (split) put_split(nd[j], j, base + j + 1, &words[base + j + 1]);
+        continue;
+      }
+      // the leaves below each path (full), or the exits (deep)
+      const size_t w = deep ? base + (1u << levels) + 2 * (j - inner) : base + j + 1;
+      if (!split) {
+        std::memcpy(&words[w], &inherit[j], 4);
+        if (deep) words[w + 1] = kOrdExitLeaf;
+        continue;
+      }
+      put_split(nd[j], j, w, &words[w]);
+      const uint32_t first = new_blocks(2);
+      words[w + 1] = first;
+      queue.push_back({first, 2 * j + 1});
+      queue.push_back({first + 1, 2 * j + 2});
     }
+    for (size_t q = 0; q < queue.size(); ++q) {
+      const Root root = queue[q];
+      const size_t at = static_cast<size_t>(root.block) * 8;
+      int node[8];
+      uint32_t leaves = 0;
+      bool more = false;
+      node[1] = root.node;
+      for (int i = 1; i < 8; ++i) {
+        if (i > 1) node[i] = node[i >> 1] < 0 ? -1 : 2 * node[i >> 1] + 1 + (i & 1);
+        if (node[i] < 0 || node[i] >= slots || !reach[node[i]]) {
+          node[i] = -1;
+          continue;
+        }
+        const mlt_node& n = nd[node[i]];
+        if (n.feature < 0) {
+          const float v = value(n);
+          std::memcpy(&blocks[at + i], &v, 4);
+          leaves |= 1u << i;
+        } else {
+          uint32_t word;
+          put_split(n, node[i], tail_word + at + i, &word);
+          blocks[at + i] = word;
+          more = more || i >= 4;
+        }
+      }
+      uint32_t next = 0;
+      if (more) {
+        next = new_blocks(8);
+        for (int i = 4; i < 8; ++i)
+          if (node[i] >= 0 && nd[node[i]].feature >= 0)
+            for (int side = 0; side < 2; ++side)
+              queue.push_back({next + static_cast<uint32_t>(2 * (i - 4) + side), 2 * node[i] + 1 + side});
+      }
+      blocks[at] = next | (leaves >> 1) << kOrdBlockBits;
+    }
+    usable = usable && blocks.size() / 8 < (1u << kOrdBlockBits);
   }
+  if (!usable) return false;
+  if (blocks.empty()) blocks.resize(8, 0u);  // finished walkers read block 0
+  if (deep)  // the padding trees' exits are leaves of +0
+    for (int tr = n_trees; tr < padded; ++tr)
+      for (uint32_t e = 0; e < (1u << levels); ++e)
+        words[static_cast<size_t>(tr) * tree_words + (1u << levels) + 2 * e + 1] = kOrdExitLeaf;
+  words.insert(words.end(), blocks.begin(), blocks.end());
 
   // thresholds of every feature in order, and each node's place among them
   std::vector<size_t> start(F + 1, 0);
@@ -240,6 +319,9 @@ bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool rou
     return at;
   };
   t.off_table = append(words.data(), words.size() * 4);
+  t.off_tail = t.off_table + tail_word * 4;
+  t.visits = deep ? static_cast<float>(visits) : static_cast<float>(n_trees) * depth;  // a full walk has no early end
+  t.rounds = deep ? (depth - kOrdHead + 2) / 3 : 0;
   t.off_image = append(image.data(), image.size());
   t.off_features = append(feat.data(), feat.size() * sizeof(OrdFeature));
   t.off_groups = append(groups.data(), groups.size() * sizeof(OrdGroup));

@@ -167,3 +167,27 @@ def test_accumulation_batches():
     assert stats.cpu().tolist() == [used, int(valid[:used].sum()), 2]
     assert np.array_equal(pf.cpu().numpy()[:used].view(np.uint32), opf[:used].view(np.uint32))
     assert np.array_equal(tk.cpu().numpy(), O.topk(opf[:used], valid[:used], 50)[0])
+
+
+@pytest.mark.parametrize("vd,pd,split", [(11, 14, 0.9), (12, 11, 0.97), (13, 13, 0.6), (14, 12, 0.8), (5, 14, 0.75)])
+@pytest.mark.parametrize("nan", [0.0, 0.2])
+def test_deep_models(vd, pd, split, nan):
+    """Heads, exits and tail blocks: leaves at every level of a block, paths
+    that end in the head, at an exit and at the bottom."""
+    rng = np.random.default_rng(100 * vd + pd)
+    F = 3 + vd % 4
+    pool = _pool(rng, 400)
+    x = _rows(rng, N0 + 47, F, pool, nan=nan)
+    v = _trees(rng, F, 61, vd, pool, split=split if vd > 10 else 1.0)
+    _check(x, v, _trees(rng, F, 70, pd, pool, split=split), 0.5, 100)
+
+
+@pytest.mark.parametrize("trees", [1, 4, 7, 8, 9, 49, 100])
+def test_deep_tree_counts(trees):
+    rng = np.random.default_rng(trees)
+    pool = _pool(rng, 60)
+    x = _rows(rng, N0, 1, pool, nan=0.1)
+    # more trees than the rule asks for come from V; P's take the count's remainders
+    v = _trees(rng, 1, 20, 11, pool, split=0.9)
+    p = _trees(rng, 1, trees, 12, pool, split=0.95)
+    _check(x, v, p, 0.5, 64, launches=6 if trees >= 2 else 5)
