@@ -455,6 +455,19 @@ int mlt_walk_shape(int model_id, int64_t n, int p_pass, int32_t *out);
  * Results never depend on the path.  Host-only. */
 int mlt_tune_fused_small(int max_n);
 
+/* Tuning: walking in ordinal form.  Every V and P model with at most 8,191
+ * distinct thresholds per feature is also stored with each threshold as its
+ * place among them; a screening pass over stored or decoded rows can then turn
+ * the rows into such places once and compare small integers, which decides
+ * every node as the fp32 comparison does (the same results, bit for bit).
+ *   mode  1 (default): where the library expects it to be faster; 2: wherever
+ *         the model has the form; 0: never
+ * Needs a library-owned device buffer of 2 bytes per feature and candidate
+ * (at most 8 GB, grown as needed, given back like the decoded rows'); where it
+ * cannot be had, and in mlt_screen_noalloc, the fp32 form is walked.
+ * Host-only. */
+int mlt_tune_ordinal(int mode);
+
 /* Tuning: the table format of models V and P deeper than 10 levels, for
  * ensembles loaded after this call.  levels = 6 (the default) or 7: a
  * split table, whose first `levels` levels stream through shared memory

@@ -349,6 +349,58 @@ ScreenShape plan_for(const DeviceModel& dm, int F, long long n_eff, const ShapeO
   return s;
 }
 
+// Plans of recent calls: a plan depends on the sizes in its key alone, and the
+// search for one costs tens of microseconds of host time, more than a small
+// batch takes.
+struct PlanKey {
+  long long n_eff;
+  int kind, F, n_trees, depth, tree_bytes, rounds, ov[5], sms, optin;
+};
+constexpr size_t kPlanSlots = 64;
+std::vector<std::pair<PlanKey, ScreenShape>> g_plans;
+size_t g_plan_next = 0;
+
+template <typename Make>
+ScreenShape remembered_plan(const PlanKey& key, Make&& make) {
+  for (const auto& p : g_plans)
+    if (std::memcmp(&p.first, &key, sizeof(key)) == 0) return p.second;
+  const ScreenShape s = make();
+  if (g_plans.size() < kPlanSlots)
+    g_plans.emplace_back(key, s);
+  else
+    g_plans[g_plan_next++ % kPlanSlots] = {key, s};
+  return s;
+}
+
+PlanKey plan_key(int kind, int n_trees, int depth, uint32_t tree_bytes, int rounds, long long n_eff,
+                 const ShapeOverride& ov) {
+  PlanKey k;
+  std::memset(&k, 0, sizeof(k));  // padding takes part in the comparison
+  k.n_eff = n_eff;
+  k.kind = kind;
+  k.F = g_F;
+  k.n_trees = n_trees;
+  k.depth = depth;
+  k.tree_bytes = static_cast<int>(tree_bytes);
+  k.rounds = rounds;
+  const int o[5] = {ov.threads, ov.chunk_trees, ov.nbuf, ov.lanes, ov.group};
+  std::memcpy(k.ov, o, sizeof(o));
+  k.sms = sm_count();
+  k.optin = smem_optin();
+  return k;
+}
+
+ScreenShape plan_walk(const DeviceModel& dm, long long n_eff, const ShapeOverride& ov, bool v_pass) {
+  return remembered_plan(plan_key(dm.kind, dm.n_trees, dm.depth, dm.tree_bytes, 0, n_eff, ov),
+                         [&] { return plan_for(dm, g_F, n_eff, ov, v_pass); });
+}
+
+constexpr int kPlanOrdinal = 100;  // the table kinds are below
+ScreenShape plan_ordinal(const DeviceModel& dm, long long n_eff) {
+  return remembered_plan(plan_key(kPlanOrdinal, dm.ord.n_trees, dm.depth, 0, dm.ord.rounds, n_eff, ShapeOverride()),
+                         [&] { return plan_ord(g_F, dm.ord, dm.depth, n_eff, sm_count(), smem_optin()); });
+}
+
 int build_decoder(const int32_t* radices, const float* option_values, int n_knobs,
                   const mlt_feat_op* program, int F, long long first_index, long long n,
                   DecodeParams* d) {
@@ -510,18 +562,34 @@ int pack_ensemble(const mlt_node* nodes, int n_trees, int depth, int F, std::vec
   return MLT_OK;
 }
 
-// Ordinal walk of a pass over stored rows: the rule of sizes.  Making the
-// ordinals costs about 17 shared-memory cycles per warp and feature (10
-// search steps), and a visit of the ordinal walk about 1.5 cycles less than
-// the fp32 walk's, so a candidate's visits must outweigh its features; below
-// kOrdMinN candidates the extra launch costs more than the walk saves.
-constexpr long long kOrdMinN = 16384;
-constexpr int kOrdMinVisits = 16;  // per feature
+// Ordinal walk of a pass over stored rows: taken where it is expected to save
+// time.  With n_eff candidates to walk it saves, per 32 candidates on an SM, a
+// visit's cycles beyond the ordinal walk's 2.8 (the fp32 walk needs 3.6 and 16
+// shared by the warps whose rows fit beside the tree chunks, one more where a
+// chunk holds under 8 trees, and deep models' 8-byte tail records about 4 more)
+// and spends 20 cycles a feature on the ordinals; a small batch waits on its
+// visits one after another and saves about 6 ns for each; the extra launch
+// costs 7 us.  Measured on both sides (whole calls, fp32 -> ordinal in both
+// passes): 13,397 x 20, 2,530 + 3,300 visits 84 -> 49 us; 39,844 x 118, 1,287 +
+// 1,561 visits 130 -> 91 us; 1,622 x 53, deep, about 7,000 visits 166 -> 71 us;
+// against it 3,818 x 24, 749 + 1,323 visits 36 -> 43 us; 43,767 x 82, V of 336
+// visits 57 -> 63 us.
+constexpr long long kOrdMinN = 256;
+int g_ord_mode = 1;  // 0: never, 1: by the rule, 2: wherever a model has an ordinal form
 
-bool ord_wanted(const DeviceModel& m, const ShapeOverride& ov, long long n) {
-  if (m.ord.table == nullptr || n < kOrdMinN) return false;
+bool ord_wanted(const DeviceModel& m, const ShapeOverride& ov, long long n, long long n_eff) {
+  if (m.ord.table == nullptr || g_ord_mode == 0) return false;
   if (ov.threads || ov.chunk_trees || ov.nbuf || ov.lanes || ov.group) return false;  // a fixed shape of the fp32 walk
-  return m.ord.visits >= static_cast<float>(kOrdMinVisits) * g_F;
+  if (g_ord_mode == 2) return n > 0;
+  if (n < kOrdMinN) return false;
+  const double F = g_F, visits = m.ord.visits;
+  const double warps = std::max(1.0, std::min(16.0, std::floor(190.0 * 1024 / (128.0 * F))));
+  double fp32 = 3.6 + 16.0 / warps;
+  if (m.kind == kTableSplit) fp32 += 4.0;
+  if (m.kind == kTableFull && m.depth > 9) fp32 += 1.0;
+  const double cycles = visits * (fp32 - 2.8) - 20.0 * F;
+  const double us = static_cast<double>(n_eff) / 32.0 * cycles / (sm_count() * 2070.0) + 0.006 * visits;
+  return us > 7.0;
 }
 
 // Bytes of the ordinals of n candidates, and of their missing-value flags.
@@ -544,14 +612,14 @@ void plan_passes(const DeviceModel& V, const DeviceModel& P, long long n, bool s
   const long long n_eff[2] = {n, (n + 1) / 2};
   size_t bytes = 0;
   for (int i = 0; i < 2; ++i) {
-    p[i]->ord = stored && ord_wanted(*m[i], g_shape[i], n);
-    if (p[i]->ord) p[i]->shape = plan_ord(g_F, m[i]->ord, m[i]->depth, n_eff[i], sm_count(), smem_optin());
+    p[i]->ord = stored && ord_wanted(*m[i], g_shape[i], n, n_eff[i]);
+    if (p[i]->ord) p[i]->shape = plan_ordinal(*m[i], n_eff[i]);
     p[i]->ord = p[i]->ord && p[i]->shape.threads > 0;
     if (p[i]->ord) bytes = std::max(bytes, ord_bytes(n) + ord_flag_bytes(n));
   }
   if (bytes > 0 && (bytes > kOrdMaxBytes || !g_scr.ord.ensure(bytes, st))) pv->ord = pp->ord = false;
   for (int i = 0; i < 2; ++i)
-    if (!p[i]->ord) p[i]->shape = plan_for(*m[i], g_F, n_eff[i], g_shape[i], i == 0);
+    if (!p[i]->ord) p[i]->shape = plan_walk(*m[i], n_eff[i], g_shape[i], i == 0);
 }
 
 cudaError_t launch_pass(const DeviceModel& m, TraverseArgs a, const Pass& p, const DecodeParams* dec, long long n,
@@ -1122,6 +1190,13 @@ int mlt_tune_decode_jit(int64_t min_n) {
   return MLT_OK;
 }
 
+int mlt_tune_ordinal(int mode) {
+  if (mode < 0 || mode > 2) return fail(MLT_EINVAL, "mode must be 0, 1 or 2, got %d", mode);
+  std::lock_guard<std::mutex> lk(g_mu);
+  g_ord_mode = mode;
+  return MLT_OK;
+}
+
 int mlt_decode_jit_available(void) {
   std::lock_guard<std::mutex> lk(g_mu);
   return jit_available() ? 1 : 0;
@@ -1657,7 +1732,7 @@ int mlt_walk_peak(void* stream, int model_id, const float* feats, int64_t n, int
   a.n_trees = dm.n_trees;
   a.tree_bytes = dm.tree_bytes;
   a.err = g_scr.err;
-  MLT_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)),
+  MLT_CUDA(allow_smem(reinterpret_cast<const void*>(k), smem),
            "walk-rate kernel attribute");
   const long long tiles = (n + tc - 1) / tc;
   k<<<dim3(static_cast<unsigned>(tiles)), dim3(tc), smem, static_cast<cudaStream_t>(stream)>>>(a, resident, rounds,

@@ -386,6 +386,10 @@ bool jit_available();
 cudaError_t launch_jit_decode(const JitDecoder& jd, const DecodeParams& d, long long n, float* out,
                               cudaStream_t st);
 
+// Allow a kernel `bytes` of dynamic shared memory on the current device; the
+// driver is asked only when that is more than it was last asked for.
+cudaError_t allow_smem(const void* kernel, size_t bytes);
+
 // Launch with programmatic dependent launch allowed: the kernel may start
 // while the previous kernel on the stream finishes; it must execute
 // pdl_wait() before it touches anything that kernel (or any earlier one)

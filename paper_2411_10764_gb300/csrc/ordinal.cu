@@ -609,7 +609,7 @@ cudaError_t launch_ordinals(const OrdTable& t, OrdArgs a, long long n_max, int s
   }
   auto k = a.vec4 ? (t.round_half ? k_ordinals<true, true> : k_ordinals<true, false>)
                   : (t.round_half ? k_ordinals<false, true> : k_ordinals<false, false>);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(k, dim3(a.first_cta[t.n_groups]), dim3(kOrdThreads), smem, st, a);
 }
@@ -626,9 +626,9 @@ ScreenShape plan_ord_deep(int F, const OrdTable& t, long long n_eff, int sms, in
   const uint32_t tb = ord_head_bytes(kOrdHead);
   double best_cost = 1e300;
   for (int tc = 32; tc <= 512; tc += 32) {
-    for (int q : {1, 2, 3, 4, 6, 8}) {
+    for (int q : {1, 2, 3, 4, 6, 8, 12, 16}) {
       if (tc * q > kOrdMaxCta) continue;
-      for (int ch = 48; ch >= 8; ch -= 8) {
+      for (int ch = 128; ch >= 8; ch -= 8) {
         if (ch % (kOrdDeepUnit * q) != 0) continue;
         for (int nb : {2, 3}) {
           const size_t smem = ord_smem(F, tc, q, nb, static_cast<uint32_t>(ch) * tb).bytes;
@@ -684,11 +684,11 @@ ScreenShape plan_ord(int F, const OrdTable& t, int depth, long long n_eff, int s
   const uint32_t tb = ord_tree_bytes(depth);
   const int trees8 = (t.n_trees + 7) / 8 * 8;
   double best_cost = 1e300;
-  for (int tc = 64; tc <= 768; tc += 32) {
-    for (int q : {1, 2, 4}) {
+  for (int tc = 32; tc <= 768; tc += 32) {
+    for (int q : {1, 2, 4, 8, 16}) {
       if (tc * q > kOrdMaxCta) continue;
-      for (int ch = 64; ch >= 8; ch -= 8) {
-        if (ch > trees8 && ch != 8) continue;
+      for (int ch = 128; ch >= 8; ch -= 8) {
+        if (ch > std::max(trees8, 4 * q) && ch != 8) continue;
         const int unit = ord_unit(ch, q);
         if (unit < 0) continue;
         for (int nb : {2, 3}) {
@@ -742,7 +742,7 @@ cudaError_t launch_walk_ord(int depth, const TraverseArgs& args, const ScreenSha
                                           : ord_kernel(depth, ord_unit(shape.chunk_trees, shape.lanes));
   if (k == nullptr) return cudaErrorInvalidValue;
   cudaError_t e =
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(shape.smem));
+      allow_smem(reinterpret_cast<const void*>(k), shape.smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(k, dim3(static_cast<unsigned>(ctas)), dim3(shape.threads * shape.lanes), shape.smem, st, a);
 }

@@ -176,8 +176,7 @@ cudaError_t launch_rerank(const DeviceModel& A, const float* feats, int F, long 
   int m2 = 1;
   while (m2 < m) m2 <<= 1;
   const size_t smem = static_cast<size_t>(m2) * 8;
-  cudaError_t e = cudaFuncSetAttribute(k_rerank_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_rerank_select), smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_rerank_select, dim3(1), dim3(kSelectThreads), smem, st,
                     static_cast<const unsigned long long*>(keys), m, m2, n_final, out_final);

@@ -369,7 +369,7 @@ cudaError_t launch_screen_small(const SmallPlan& pl, const DeviceModel& V, const
   s.err = sc.err;
   s.stall_cta = stall_cta;
   s.stall_ns = stall_ns;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pl.smem));
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), pl.smem);
   if (e != cudaSuccess) return e;
   e = launch_pdl(kern, dim3(static_cast<unsigned>(pl.ctas)), dim3(kSmallThreads), pl.smem, st, s);
   if (e != cudaSuccess) return e;

@@ -321,7 +321,7 @@ cudaError_t launch_topk(const Scratch& s, long long n, int k, long long index_ba
   int n2k = 2;
   while (n2k < k) n2k <<= 1;
   const size_t smem = static_cast<size_t>(kSortMin + n2k) * 8;
-  cudaError_t e = cudaFuncSetAttribute(k_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_topk), smem);
   if (e != cudaSuccess) return e;
   long long g = (n + 1023) / 1024;  // about one pass of the collection loop per warp
   if (g < 1) g = 1;

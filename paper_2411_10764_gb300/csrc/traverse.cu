@@ -3,6 +3,8 @@
 // that build features from candidate indices.
 #include <algorithm>
 #include <cmath>
+#include <mutex>
+#include <vector>
 
 #include "walk.cuh"
 
@@ -16,6 +18,30 @@ constexpr size_t kCtaReserve = 1024;     // reserved per resident CTA
 constexpr size_t kStaticSmem = 512;      // finish_tile and scan_tiles statics
 
 }  // namespace
+
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+  struct Allowed {
+    const void* kernel;
+    int device;
+    size_t bytes;
+  };
+  static std::mutex mu;
+  static std::vector<Allowed> allowed;  // at most one entry per kernel and device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  for (Allowed& a : allowed)
+    if (a.kernel == kernel && a.device == dev) {
+      if (bytes <= a.bytes) return cudaSuccess;
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+      if (e == cudaSuccess) a.bytes = bytes;
+      return e;
+    }
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e == cudaSuccess) allowed.push_back({kernel, dev, bytes});
+  return e;
+}
 
 FullKernelPtr full_kernel_q1(int depth, int group) { return full_kernel_q<1>(depth, group); }
 
@@ -317,16 +343,14 @@ cudaError_t launch_traverse(const DeviceModel& m, const TraverseArgs& args, cons
                       : m.kind == kTableSplit ? split_kernel(m.head_levels, shape.group, q)
                                               : full_kernel(m.depth, shape.group, q);
     if (k == nullptr) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(shape.smem));
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), shape.smem);
     if (e != cudaSuccess) return e;
     e = launch_pdl(k, grid, dim3(shape.threads * shape.lanes), shape.smem, st, a);
     if (e != cudaSuccess) return e;
   } else {
     CompactKernel k = compact_kernel(shape.group, shape.lanes);
     if (k == nullptr) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(shape.smem));
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), shape.smem);
     if (e != cudaSuccess) return e;
     e = launch_pdl(k, grid, dim3(shape.threads * shape.lanes), shape.smem, st, a);
     if (e != cudaSuccess) return e;

@@ -187,16 +187,14 @@ cudaError_t launch_traverse_dec(const DeviceModel& m, const TraverseArgs& args, 
     FullDecKernelPtr k = m.kind == kTableSplit ? split_dec_kernel(m.head_levels, shape.group, q)
                                                : full_dec_kernel(m.depth, shape.group, q);
     if (k == nullptr) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(shape.smem));
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), shape.smem);
     if (e != cudaSuccess) return e;
     e = launch_pdl(k, grid, dim3(shape.threads * shape.lanes), shape.smem, st, a, dec);
     if (e != cudaSuccess) return e;
   } else {
     CompactDecKernel k = compact_dec_kernel(shape.group, shape.lanes);
     if (k == nullptr) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(shape.smem));
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), shape.smem);
     if (e != cudaSuccess) return e;
     e = launch_pdl(k, grid, dim3(shape.threads * shape.lanes), shape.smem, st, a, dec);
     if (e != cudaSuccess) return e;
@@ -224,7 +222,7 @@ cudaError_t launch_decode_rows(const DecodeParams& dec, long long n, uint8_t* ou
   }
   const size_t smem = smem_of(tile);
   auto k = k_decode_rows;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), smem);
   if (e != cudaSuccess) return e;
   const int vec4 = (dec.F & 3) == 0 && (reinterpret_cast<uintptr_t>(out_feats) & 15u) == 0 ? 1 : 0;
   return launch_pdl(k, dim3(static_cast<unsigned>((n + tile - 1) / tile)), dim3(tile), smem, st, dec, n, tile + 1,

@@ -77,6 +77,7 @@ def lib(build_if_missing: bool = True):
             "mlt_tune_head_levels": [i32],
             "mlt_tune_fused_small": [i32],
             "mlt_tune_decode_jit": [i64],
+            "mlt_tune_ordinal": [i32],
             "mlt_decode_jit_available": [],
             "mlt_walk_peak": [P, i32, P, i64, i32, P, P],
             "mlt_screen_noalloc": [P, P, i64, f32, i32, P, P, P],
@@ -455,6 +456,12 @@ def tune_decode_jit(min_n: int) -> None:
     the feature program compiled at run time (NVRTC); 0 keeps every decoded
     batch on the interpreted program."""
     _check(lib().mlt_tune_decode_jit(int(min_n)))
+
+
+def tune_ordinal(mode: int) -> None:
+    """Walk rows in ordinal form (same results): 1 where the library expects
+    it to be faster (the default), 2 wherever a model has that form, 0 never."""
+    _check(lib().mlt_tune_ordinal(int(mode)))
 
 
 def decode_jit_available() -> bool:

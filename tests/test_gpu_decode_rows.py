@@ -39,8 +39,8 @@ def test_rows_and_digits(F, knobs):
 
 @pytest.mark.parametrize("n,first", [(1, 7), (3000, 123456), (8193, 40), (16384, 5), (30001, 999999)])
 def test_screening_from_rows(n, first):
-    """One launch (n <= 8,192), the fp32 walk and the ordinal walk; top-k
-    holds candidate indices."""
+    """One launch (n <= 8,192) and the ordinal walk; top-k holds candidate
+    indices."""
     import torch
 
     d = W.conv2d_decoder(3, 70)

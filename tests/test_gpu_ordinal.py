@@ -12,7 +12,15 @@ from paper_2411_10764_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-N0 = 16384  # smallest batch that takes the ordinal walk
+N0 = 16384
+
+
+@pytest.fixture(autouse=True)
+def _always_ordinal():
+    """These models are smaller than the rule's, so the walk is asked for."""
+    mlt.tune_ordinal(2)
+    yield
+    mlt.tune_ordinal(1)
 
 
 def _trees(rng, F, trees, depth, pool, split=1.0):
@@ -187,7 +195,39 @@ def test_deep_tree_counts(trees):
     rng = np.random.default_rng(trees)
     pool = _pool(rng, 60)
     x = _rows(rng, N0, 1, pool, nan=0.1)
-    # more trees than the rule asks for come from V; P's take the count's remainders
     v = _trees(rng, 1, 20, 11, pool, split=0.9)
     p = _trees(rng, 1, trees, 12, pool, split=0.95)
-    _check(x, v, p, 0.5, 64, launches=6 if trees >= 2 else 5)
+    _check(x, v, p, 0.5, 64, launches=6)
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 500, 4097])
+@pytest.mark.parametrize("vd,pd", [(6, 6), (4, 10), (12, 13)])
+def test_small_batches(n, vd, pd):
+    """Tiles of one block, more tree groups than trees, waves with idle CTAs."""
+    rng = np.random.default_rng(n + vd)
+    pool = _pool(rng, 100)
+    mlt.tune_fused_small(0)
+    try:
+        x = _rows(rng, n, 9, pool, nan=0.05, special=n > 40)
+        v, p = (_trees(rng, 9, t, d, pool, split=0.95 if d > 10 else 1.0) for t, d in ((37, vd), (5, pd)))
+        _check(x, v, p, 0.5, 64)
+    finally:
+        mlt.tune_fused_small(8192)
+
+
+@pytest.mark.parametrize("F,n,trees,depth,launches", [
+    (20, 13397, 500, 5, 6), (24, 3818, 107, 7, 4), (82, 43767, 56, 6, 4), (64, 65536, 200, 8, 6), (30, 200, 900, 8, 4)])
+def test_rule(F, n, trees, depth, launches):
+    """Which batches take the ordinal walk by default (two more launches)."""
+    import torch
+
+    mlt.tune_ordinal(1)
+    rng = np.random.default_rng(1)
+    e = _trees(rng, F, trees, depth, _pool(rng, 500))
+    mlt.set_num_features(F)
+    for m in (mlt.MLT_MODEL_V, mlt.MLT_MODEL_P):
+        mlt.load_ensemble(m, e.nodes, e.n_trees, e.depth)
+    before = mlt.kernel_launches()
+    mlt.screen(torch.zeros((n, F), device="cuda"), 0.5, 10)
+    mlt.sync_status()
+    assert mlt.kernel_launches() - before == launches
