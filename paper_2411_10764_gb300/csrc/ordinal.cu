@@ -180,9 +180,17 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
   }
 }
 
-// The ordinal that a node word tests (xw: the candidate's column).
-__device__ __forceinline__ uint32_t ord_at(const unsigned char* xw, uint32_t w) {
-  return ld_sm<unsigned short>(xw, w & 0xFFFEu);
+// A candidate's ordinals: its warp's blocks and its lane's bytes in a row of
+// them.  Bits 2 to 6 of a word's offset are zero, so the lane is merged by the
+// operation that masks the offset and the warp-uniform base goes into the
+// load's address: one integer operation a visit less than adding a pointer.
+struct OrdRow {
+  const unsigned char* warp;
+  uint32_t lane4;
+};
+// The ordinal that a node word tests.
+__device__ __forceinline__ uint32_t ord_at(const OrdRow& x, uint32_t w) {
+  return ld_sm<unsigned short>(x.warp, (w & 0xFFFEu) | x.lane4);
 }
 // Heap index of the child that ordinal x takes below node i; a missing x
 // (kOrdNan) becomes 0 where the word's flag sends it left.
@@ -192,8 +200,8 @@ __device__ __forceinline__ uint32_t ord_child(uint32_t i, uint32_t w, uint32_t x
   return __funnelshift_l(w - x * 65536u, i, 1);
 }
 // The same for a deep model's words, whose flag is at kOrdNan's bit.
-__device__ __forceinline__ uint32_t deep_at(const unsigned char* xw, uint32_t w) {
-  return ld_sm<unsigned short>(xw, w & 0x7FFEu);
+__device__ __forceinline__ uint32_t deep_at(const OrdRow& x, uint32_t w) {
+  return ld_sm<unsigned short>(x.warp, (w & 0x7FFEu) | x.lane4);
 }
 template <bool NANP>
 __device__ __forceinline__ uint32_t deep_child(uint32_t i, uint32_t w, uint32_t x) {
@@ -208,10 +216,9 @@ __device__ __forceinline__ void ldg_block(const uint4* ptr, unsigned long long p
       : "l"(ptr), "l"(pol));
 }
 
-// Leaves of G consecutive trees at tb for one candidate (its column of
-// ordinals at xw).
+// Leaves of G consecutive trees at tb for one candidate.
 template <int D, int G, bool NANP>
-__device__ __forceinline__ void walk_ord(const unsigned char* tb, const unsigned char* xw, float* leaf) {
+__device__ __forceinline__ void walk_ord(const unsigned char* tb, const OrdRow& xw, float* leaf) {
   constexpr uint32_t kTree = ord_tree_bytes(D);
   uint32_t j[G];
 #pragma unroll
@@ -232,7 +239,7 @@ __device__ __forceinline__ void walk_ord(const unsigned char* tb, const unsigned
 
 // Leaves of nt <= U trees (a multiple of 4), up to 8 trees in flight.
 template <int D, int U, bool NANP>
-__device__ __forceinline__ void walk_ord_unit(const unsigned char* tb, int nt, const unsigned char* xw, float* leaf) {
+__device__ __forceinline__ void walk_ord_unit(const unsigned char* tb, int nt, const OrdRow& xw, float* leaf) {
   constexpr uint32_t kTree = ord_tree_bytes(D);
 #pragma unroll
   for (int t = 0; t < U; t += 8) {
@@ -252,7 +259,7 @@ __device__ __forceinline__ void walk_ord_unit(const unsigned char* tb, int nt, c
 // the tail (4,194,304 x 256, 1,000 trees of depth 12: 73 cycles a warp and tree
 // on an SM, where the split table's 8-byte records took 94).
 template <int H, int G, bool NANP>
-__device__ __forceinline__ void walk_ord_deep(const unsigned char* tb, const unsigned char* xw, const uint4* tail,
+__device__ __forceinline__ void walk_ord_deep(const unsigned char* tb, const OrdRow& xw, const uint4* tail,
                                               int rounds, float* leaf) {
   constexpr uint32_t kTree = ord_head_bytes(H);
   uint32_t j[G];
@@ -319,7 +326,7 @@ __device__ __forceinline__ void walk_ord_deep(const unsigned char* tb, const uns
 
 // Leaves of nt <= U trees (a multiple of 4) of a deep model.
 template <int H, int U, int G, bool NANP>
-__device__ __forceinline__ void walk_deep_unit(const unsigned char* tb, int nt, const unsigned char* xw,
+__device__ __forceinline__ void walk_deep_unit(const unsigned char* tb, int nt, const OrdRow& xw,
                                                const uint4* tail, int rounds, float* leaf) {
 #pragma unroll
   for (int t = 0; t < U; t += G)
@@ -328,7 +335,7 @@ __device__ __forceinline__ void walk_deep_unit(const unsigned char* tb, int nt, 
 
 // One tree group: trees [0, nt) of a chunk, leaves added in tree order.
 template <int D, bool NANP>
-__device__ __forceinline__ float walk_ord_sum(const unsigned char* tb, int nt, const unsigned char* xw, float acc) {
+__device__ __forceinline__ float walk_ord_sum(const unsigned char* tb, int nt, const OrdRow& xw, float acc) {
   constexpr uint32_t kTree = ord_tree_bytes(D);
   int t = 0;
   for (; t + 8 <= nt; t += 8) {
@@ -477,7 +484,8 @@ __global__ void __launch_bounds__(kOrdMaxCta, 1) k_walk_ord(const __grid_constan
   bool timed_out = false;
   if (col < live_cols) {
     timed_out = !__all_sync(0xFFFFFFFFu, mbar_wait_bounded(smem_u32(&bars[4]), 0u));
-    const unsigned char* xw = smem + static_cast<uint32_t>(col) * static_cast<uint32_t>(F2) * 128u + lane * 4u;
+    const OrdRow xw{smem + static_cast<uint32_t>(__shfl_sync(0xFFFFFFFFu, col, 0)) * static_cast<uint32_t>(F2) * 128u,
+                    static_cast<uint32_t>(lane) * 4u};  // the shuffle makes the base warp-uniform to the compiler
     const uint32_t turn = smem_u32(&bars[10 + col * Q + q]);
     const uint32_t next_turn = smem_u32(&bars[10 + col * Q + (q + 1 == Q ? 0 : q + 1)]);
     float* sum = sums + col * 32 + lane;
