@@ -300,6 +300,9 @@ bool cut_passes(float m, float thr) {
 }
 
 float validity_cut(float thr) {
+  // the last answer: long double arithmetic is a software library on some hosts
+  thread_local float last_thr = 0.0f, last_cut = 0.0f;  // thr lies in (0, 1)
+  if (thr == last_thr) return last_cut;
   float m = static_cast<float>(std::log(static_cast<double>(thr) / (1.0 - static_cast<double>(thr))));
   if (!cut_passes(m, thr)) {
     while (!cut_passes(m, thr)) m = std::nextafterf(m, INFINITY);
@@ -310,7 +313,9 @@ float validity_cut(float thr) {
       m = d;
     }
   }
-  return m == 0.0f ? 0.0f : m;
+  last_thr = thr;
+  last_cut = m == 0.0f ? 0.0f : m;
+  return last_cut;
 }
 
 int check_screen_args(long long n, float thr, int k) {
