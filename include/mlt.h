@@ -209,6 +209,9 @@ int mlt_screen_host_batches(void *stream, int64_t n_batches, const float *const 
  * device adds the batch's valid candidates to a running count, and once
  * that count reaches `target` every later batch is skipped on the device
  * (all batches are enqueued up front; no host round trip per batch).
+ * V may score a group of consecutive batches at once; the batch that reaches
+ * the target is still the last one consumed, and of later ones nothing is
+ * kept or written.
  * out_topk = the k best valid candidates over every batch screened, by the
  * same order as mlt_screen -- identical to mlt_screen over the consumed
  * prefix [0, consumed).

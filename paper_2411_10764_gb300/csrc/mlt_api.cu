@@ -816,12 +816,19 @@ int noalloc_scratch(int dev, Scratch* out) {
 }
 
 // Batched accumulation (ML^2Tuner Sec. 2: the explorer applies P and V
-// until (alpha+1)N configurations have accumulated): batches of `batch`
-// candidates are all enqueued; after each, a one-thread kernel adds the
-// batch's survivors to the running count and raises a device flag once it
-// reaches `target`, which makes every later batch's kernels return at once.
-// One top-k then ranks all survivors kept.  The result equals screening the
-// consumed prefix of the candidates as a single batch.
+// until (alpha+1)N configurations have accumulated).  Batches are screened in
+// groups: a batch of a few thousand candidates leaves most of the GPU waiting,
+// and every later batch's kernels cost a launch each to find out that the
+// target was reached.  V walks a group of consecutive batches at once; k_cut
+// finds the batch that reaches `target` and drops the survivors past it; P
+// walks the rest.  A group holds at least kStreamRows candidates (one batch if
+// that is larger) and each is twice the one before, so that V walks at most
+// about twice what is consumed and a long run needs few launches.  One top-k
+// then ranks all survivors kept.  The result equals screening the consumed
+// prefix of the candidates as a single batch.
+constexpr long long kStreamRows = 24576;
+constexpr long long kStreamMostRows = 196608;
+
 int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, long long n_total, long long batch,
                long long target, float thr, int k, float* out_pvalid, float* out_perf, int64_t* out_topk,
                int64_t* out_stats) {
@@ -836,13 +843,22 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
   StreamState* ss = g_scr.stream;
   const DeviceModel& V = g_models[MLT_MODEL_V].dm;
   const DeviceModel& P = g_models[MLT_MODEL_P].dm;
-  const long long per = std::min(batch, std::max(1LL, n_total));
-  // decoded batches: each batch's rows are written first, as in run_screen_with
+  // the groups: whole batches, but the last one of the call
+  std::vector<long long> groups;
+  long long per = 1;  // candidates of the largest
+  for (long long at = 0, least = kStreamRows; at < n_total; least = std::min(2 * least, kStreamMostRows)) {
+    const long long g = std::min((least + batch - 1) / batch * batch, n_total - at);
+    groups.push_back(g);
+    per = std::max(per, g);
+    at += g;
+  }
+  // decoded batches: each group's rows are written first, as in run_screen_with
   const bool rows = dec0 != nullptr && per > 0 && g_scr.feats.ensure(static_cast<size_t>(per) * g_F * sizeof(float), st);
-  Pass pv, pp;
+  Pass pv, pp;  // of the largest group: the buffers it needs, and that a shape exists
   plan_passes(V, P, per, dec0 == nullptr || rows, st, &pv, &pp);
-  const ScreenShape &sv = pv.shape, &sp = pp.shape;
-  if (sv.threads == 0 || sp.threads == 0) return fail(MLT_EINVAL, "F=%d leaves no room for a shared-memory tile", g_F);
+  if (pv.shape.threads == 0 || pp.shape.threads == 0)
+    return fail(MLT_EINVAL, "F=%d leaves no room for a shared-memory tile", g_F);
+  float* group_pvalid = reinterpret_cast<float*>(s.cand);  // unused until the top-k
   MLT_CUDA(cudaMemsetAsync(s.state, 0, sizeof(SelectState), st), "reset selection state");
   MLT_CUDA(cudaMemsetAsync(ss, 0, sizeof(StreamState), st), "reset stream state");
   const unsigned tgt = static_cast<unsigned>(std::min<long long>(target, 0xFFFFFFFFLL));
@@ -861,15 +877,15 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
   a.decode = dec0 != nullptr && !rows;
   a.stream = ss;
   long long launches = 0;
-  for (long long b0 = 0; b0 < n_total; b0 += batch) {
-    const long long nb = std::min(batch, n_total - b0);
+  long long b0 = 0;
+  for (const long long nb : groups) {
+    plan_passes(V, P, nb, dec0 == nullptr || rows, st, &pv, &pp);
+    const ScreenShape& sv = pv.shape;
     TraverseArgs ab = a;
     ab.n = nb;
     ab.pos_base = b0;
     ab.feats = rows ? static_cast<const float*>(g_scr.feats.p) : feats ? feats + b0 * g_F : nullptr;
     ab.vec4 = (ab.feats != nullptr && (reinterpret_cast<uintptr_t>(ab.feats) & 15u) == 0 && (g_F & 3) == 0) ? 1 : 0;
-    ab.out_pvalid = out_pvalid ? out_pvalid + b0 : nullptr;
-    ab.out_perf = out_perf ? out_perf + b0 : nullptr;
     DecodeParams d;
     if (dec0) {
       d = *dec0;
@@ -882,14 +898,24 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
     }
     TraverseArgs av = ab;
     av.p_pass = 0;
+    av.out_pvalid = out_pvalid ? group_pvalid : nullptr;
     const long long tiles_v = (nb + sv.threads - 1) / sv.threads;
     MLT_CUDA(launch_pass(V, av, pv, walk_dec, nb, st, &launches), "V pass launch");
     MLT_CUDA(launch_compact(s, nb, sv.threads, tiles_v, ss, st), "compaction launch");
+    MLT_CUDA(launch_cut(ss, s.state, s.rows, nb, batch, tgt, st), "cut launch");
+    if (out_pvalid || out_perf) {
+      MLT_CUDA(launch_stream_out(ss, group_pvalid, s.masks, nb, out_pvalid ? out_pvalid + b0 : nullptr,
+                                 out_perf ? out_perf + b0 : nullptr, st),
+               "output launch");
+      launches += 1;
+    }
     TraverseArgs ap = ab;
     ap.p_pass = 1;
+    ap.out_perf = out_perf ? out_perf + b0 : nullptr;
     MLT_CUDA(launch_pass(P, ap, pp, walk_dec, nb, st, &launches), "P pass launch");
-    MLT_CUDA(launch_accumulate(ss, s.state, nb, tgt, st), "accumulate launch");
-    launches += 2;
+    MLT_CUDA(launch_accumulate(ss, s.state, tgt, st), "accumulate launch");
+    launches += 3;
+    b0 += nb;
   }
   MLT_CUDA(launch_topk(s, n_total, k, dec0 ? dec0->first_index : 0, out_topk, sm_count(), &ss->total, st),
            "top-k launch");

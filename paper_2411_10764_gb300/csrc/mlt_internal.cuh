@@ -228,13 +228,15 @@ struct SelectState {
 };
 
 // Batched accumulation (mlt_screen_until): bookkeeping carried on the device
-// across the batches of one call.  Once `done` is set, every later batch's
-// kernels return at once (no host round trip decides when to stop).
+// across the groups of batches of one call.  Once `done` is set, every later
+// group's kernels return at once (no host round trip decides when to stop).
 struct StreamState {
   unsigned int total;           // survivors accumulated so far
   unsigned int done;            // the target count was reached
   unsigned int batches;         // batches screened
-  unsigned int pad;
+  unsigned int cut_batches;     // of the group at hand: batches consumed,
+  unsigned int cut_rows;        // their candidates,
+  unsigned int last_survivors;  // and the valid ones of the last of them
   unsigned long long consumed;  // candidates screened
 };
 
@@ -424,8 +426,14 @@ cudaError_t launch_topk(const Scratch& s, long long n, int k, long long index_ba
 // the k best of m (score, global index) pairs (cross-rank merge)
 cudaError_t launch_merge_topk(const float* scores, const int64_t* idx, long long m, int k, int64_t* out,
                               cudaStream_t st);
-cudaError_t launch_accumulate(StreamState* ss, const SelectState* st_, long long n_batch,
-                              unsigned target, cudaStream_t st);
+// a group of batches of `batch` candidates, n in all: where the target is
+// reached (the survivor list is complete)
+cudaError_t launch_cut(StreamState* ss, SelectState* st_, const uint32_t* rows, long long n, long long batch,
+                       unsigned target, cudaStream_t st);
+// pvalid and the invalid candidates' perf of the group's consumed candidates
+cudaError_t launch_stream_out(const StreamState* ss, const float* pvalid, const uint32_t* masks, long long n,
+                              float* out_pvalid, float* out_perf, cudaStream_t st);
+cudaError_t launch_accumulate(StreamState* ss, SelectState* st_, unsigned target, cudaStream_t st);
 cudaError_t launch_stream_stats(const StreamState* ss, int64_t* out_stats, cudaStream_t st);
 
 // sa.cu (explorer proposal step)

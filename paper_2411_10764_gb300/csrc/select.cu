@@ -228,14 +228,65 @@ cudaError_t launch_compact(const Scratch& s, long long n, int tile, long long n_
 
 namespace {
 
-// After a batch: add its survivors and candidates to the running counts and
+// Survivors among rows[0, S) at positions below `row` (ascending list), by a
+// whole block: a sample of the list, then the piece that holds the answer.
+__device__ __forceinline__ unsigned survivors_below(const uint32_t* rows, unsigned S, unsigned long long row) {
+  const unsigned T = blockDim.x, t = threadIdx.x, piece = (S + T - 1) / T;
+  const unsigned at = t * piece;  // S < 2^31
+  const unsigned before = __syncthreads_count(at < S && rows[at] < row);
+  if (before == 0) return 0u;
+  // the sample before - 1 is below `row`, the next one is not
+  const unsigned lo = (before - 1) * piece;
+  unsigned n = 0;
+  for (unsigned i = 0; i < piece; i += T)
+    n += __syncthreads_count(i + t < piece && lo + i + t < S && rows[lo + i + t] < row);
+  return lo + n;
+}
+
+// A group of batches has its survivor list: the batch in which the running
+// count reaches the target is the last one consumed, whole; the survivors
+// past it leave the list (it is ascending, so a shorter count drops them).
+__global__ void __launch_bounds__(1024)
+    k_cut(StreamState* ss, SelectState* st, const uint32_t* rows, long long n, long long batch, unsigned target) {
+  pdl_wait();
+  pdl_trigger();
+  if (*reinterpret_cast<volatile const unsigned*>(&ss->done)) return;
+  const unsigned S = *reinterpret_cast<volatile const unsigned*>(&st->survivors);
+  const unsigned need = target - ss->total;  // not done: total < target
+  unsigned long long last = static_cast<unsigned long long>(n - 1) / batch;  // last batch consumed
+  if (need <= S) last = rows[need - 1] / static_cast<unsigned long long>(batch);
+  const unsigned long long first = last * batch;
+  const unsigned long long cut = min(static_cast<unsigned long long>(n), first + batch);
+  const unsigned count = survivors_below(rows, S, cut);
+  const unsigned before = survivors_below(rows, S, first);
+  if (threadIdx.x == 0) {
+    st->survivors = count;
+    ss->cut_rows = static_cast<unsigned>(cut);
+    ss->cut_batches = static_cast<unsigned>(last) + 1u;
+    ss->last_survivors = count - before;
+  }
+}
+
+__global__ void __launch_bounds__(256)
+    k_stream_out(const StreamState* ss, const float* pvalid, const uint32_t* masks, float* out_pvalid, float* out_perf) {
+  pdl_wait();
+  pdl_trigger();
+  if (*reinterpret_cast<volatile const unsigned*>(&ss->done)) return;
+  const unsigned i = blockIdx.x * 256u + threadIdx.x;
+  if (i >= ss->cut_rows) return;
+  if (out_pvalid) out_pvalid[i] = pvalid[i];
+  if (out_perf && !((masks[i >> 5] >> (i & 31u)) & 1u)) out_perf[i] = -INFINITY;
+}
+
+// After a group: add its survivors and candidates to the running counts and
 // raise `done` once the target is reached.
-__global__ void k_accumulate(StreamState* ss, const SelectState* st, long long n_batch, unsigned target) {
+__global__ void k_accumulate(StreamState* ss, SelectState* st, unsigned target) {
   pdl_wait();
   if (threadIdx.x != 0 || ss->done) return;
   ss->total += st->survivors;
-  ss->consumed += static_cast<unsigned long long>(n_batch);
-  ss->batches += 1u;
+  ss->consumed += ss->cut_rows;
+  ss->batches += ss->cut_batches;
+  st->survivors = ss->last_survivors;  // what the last batch by itself had
   if (ss->total >= target) ss->done = 1u;
 }
 
@@ -250,9 +301,19 @@ __global__ void k_stream_stats(const StreamState* ss, int64_t* out) {
 
 }  // namespace
 
-cudaError_t launch_accumulate(StreamState* ss, const SelectState* st_, long long n_batch, unsigned target,
-                              cudaStream_t st) {
-  return launch_pdl(k_accumulate, dim3(1), dim3(32), 0, st, ss, st_, n_batch, target);
+cudaError_t launch_cut(StreamState* ss, SelectState* st_, const uint32_t* rows, long long n, long long batch,
+                       unsigned target, cudaStream_t st) {
+  return launch_pdl(k_cut, dim3(1), dim3(1024), 0, st, ss, st_, rows, n, batch, target);
+}
+
+cudaError_t launch_stream_out(const StreamState* ss, const float* pvalid, const uint32_t* masks, long long n,
+                              float* out_pvalid, float* out_perf, cudaStream_t st) {
+  return launch_pdl(k_stream_out, dim3(static_cast<unsigned>((n + 255) / 256)), dim3(256), 0, st, ss, pvalid, masks,
+                    out_pvalid, out_perf);
+}
+
+cudaError_t launch_accumulate(StreamState* ss, SelectState* st_, unsigned target, cudaStream_t st) {
+  return launch_pdl(k_accumulate, dim3(1), dim3(32), 0, st, ss, st_, target);
 }
 
 cudaError_t launch_stream_stats(const StreamState* ss, int64_t* out_stats, cudaStream_t st) {
