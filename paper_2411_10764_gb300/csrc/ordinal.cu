@@ -13,7 +13,6 @@ namespace {
 using namespace walk;
 
 constexpr int kOrdThreads = 1024;
-constexpr int kOrdRows = 2;  // blocks of 32 rows a warp takes together
 constexpr int kOrdMaxCta = 1024;
 constexpr int kOrdDeepUnit = 8;    // trees a tree group takes at a time
 constexpr int kOrdDeepFlight = 4;  // trees a thread walks at once
@@ -24,19 +23,20 @@ constexpr size_t kStaticSmem = 1024;
 // `steps` compares from the bucket's start: p += 2^k entries wherever the
 // last of them is still <= x.  One load, one compare and one predicated add
 // each (the offsets are immediates).
-template <int K>
-__device__ __forceinline__ void ord_step(uint32_t (&p)[2][4], const float* x) {
-  float t[2][4];
+template <int K, int S>
+__device__ __forceinline__ void ord_step(uint32_t (&p)[S], const float (&x)[S]) {
+  float t[S];
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
-    asm("ld.shared.f32 %0, [%1 + %2];" : "=f"(t[r >> 2][r & 3]) : "r"(p[r >> 2][r & 3]), "n"((4 << K) - 4));
+  for (int r = 0; r < S; ++r)
+    asm("ld.shared.f32 %0, [%1 + %2];" : "=f"(t[r]) : "r"(p[r]), "n"((4 << K) - 4));
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int r = 0; r < S; ++r)
     asm("{\n\t.reg .pred q;\n\tsetp.le.f32 q, %1, %2;\n\t@q add.u32 %0, %0, %3;\n\t}"
-        : "+r"(p[r >> 2][r & 3])
-        : "f"(t[r >> 2][r & 3]), "f"(x[r]), "n"(4 << K));
+        : "+r"(p[r])
+        : "f"(t[r]), "f"(x[r]), "n"(4 << K));
 }
-__device__ __forceinline__ void ord_search(uint32_t steps, uint32_t (&p)[2][4], const float* x) {
+template <int S>
+__device__ __forceinline__ void ord_search(uint32_t steps, uint32_t (&p)[S], const float (&x)[S]) {
   switch (steps) {
     case 13: ord_step<12>(p, x); [[fallthrough]];
     case 12: ord_step<11>(p, x); [[fallthrough]];
@@ -56,15 +56,20 @@ __device__ __forceinline__ void ord_search(uint32_t steps, uint32_t (&p)[2][4], 
 }
 
 // A CTA holds one feature group's thresholds and lookup tables in shared
-// memory.  A warp takes 64 rows and 8 features (one 32-byte sector of each
+// memory.  A warp takes 16 S rows and 8 features (one 32-byte sector of each
 // row) at a time: lanes 2i and 2i + 1 read the two halves of a row's sector
 // together (16 lines a load, where a lane per row would touch 32), so an even
-// lane searches features 0-3 and an odd one 4-7, four rows each, two
-// features together (eight chains in flight).  Groups get CTAs in proportion to their
-// features.  Bound: the L1 data pipe (about 11 wavefronts of table loads and
-// 4 of row loads per 32 values) and integer issue.
-template <bool VEC, bool HALF>
+// lane searches features 0-3 and an odd one 4-7, S rows of a feature together
+// (S chains in flight; its parameters are read once for them).
+// Groups get CTAs in proportion to their features.  Bound: the L1 data pipe,
+// about 14 wavefronts of table loads and 5 of row loads per 32 values.  V's
+// ordinals of 1,048,576 x 128 take 0.315 ms (0.344 with four rows a lane; 0.72
+// with a lane per row and feature parameters per row pair).  S is 8, or 4 where
+// that leaves warps without work (20,011 x 47, whole call: 71.3 us with 8, 69.7
+// with 4).
+template <bool VEC, bool HALF, int S>
 __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_constant__ OrdArgs a) {
+  constexpr int kRows = S / 2;  // blocks of 32 rows a warp takes together
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) unsigned long long bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -94,7 +99,7 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
   const long long blocks = (count + 31) >> 5;
   const int F2 = (a.F + 1) >> 1, F8 = (a.F + 7) >> 3;
   const int nf = static_cast<int>(g.count), chunks = (nf + 7) >> 3;
-  const uint32_t items = static_cast<uint32_t>((blocks + kOrdRows - 1) / kOrdRows) * chunks;  // n x F fits memory
+  const uint32_t items = static_cast<uint32_t>((blocks + kRows - 1) / kRows) * chunks;  // n x F fits memory
   const OrdFeature* feat = a.features + g.first;
   const uint32_t step = slabs * (blockDim.x >> 5);
   const uint32_t sm = smem_u32(smem);
@@ -109,12 +114,12 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
     const uint32_t s32 = it / static_cast<uint32_t>(chunks);
     const int f0 = static_cast<int>(it - s32 * chunks) * 8;
     const long long sb = s32;
-    // row slot r of this lane: row 16 r + lane / 2 of the 64; features h0 .. h0 + 3
+    // row slot r of this lane: row 16 r + lane / 2 of the item; features h0 .. h0 + 3
     const int h0 = f0 + (lane & 1) * 4;
-    float x[4][4];  // [feature][row slot]
+    float x[4][S];  // [feature][row slot]
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const long long i = sb * (kOrdRows * 32) + r * 16 + (lane >> 1);
+    for (int r = 0; r < S; ++r) {
+      const long long i = sb * (kRows * 32) + r * 16 + (lane >> 1);
       const bool in = i < count && h0 < nf;
       const long long row = in ? (a.rows ? static_cast<long long>(a.rows[i]) : i) : 0;
       const float* src = a.feats + row * a.F + g.first + h0;
@@ -130,53 +135,50 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
       }
     }
     // ordinals of a row slot: words of pairs (h0, h0 + 1) and (h0 + 2, h0 + 3)
-    uint32_t* dst = a.out + (sb * kOrdRows * F2 + ((g.first + h0) >> 1)) * 32;
+    uint32_t* dst = a.out + (sb * kRows * F2 + ((g.first + h0) >> 1)) * 32 + (lane >> 1);
     uint32_t missing = 0;  // bits: row slots of this lane that hold a missing value
-    const uint32_t steps = __ldg(&feat[f0].steps);
+    uint32_t word[S];
 #pragma unroll
-    for (int h = 0; h < 4; h += 2) {
-      uint32_t p[2][4], start[2], origin = 0;
+    for (int h = 0; h < 4; ++h) {  // the table is padded to a multiple of 8 features
+      const float4 o0 = __ldg(reinterpret_cast<const float4*>(feat + h0 + h));
+      const uint4 o1 = __ldg(reinterpret_cast<const uint4*>(feat + h0 + h) + 1);
+      const uint32_t base = __float_as_uint(o0.z), shift = __float_as_uint(o0.w);
+      const uint32_t thr = sm + o1.z, lut = sm + o1.w;
+      uint32_t p[S];
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {  // the table is padded to a multiple of 8 features
-        const float4 o0 = __ldg(reinterpret_cast<const float4*>(feat + h0 + h + e));
-        const uint4 o1 = __ldg(reinterpret_cast<const uint4*>(feat + h0 + h + e) + 1);
-        const uint32_t base = __float_as_uint(o0.z), shift = __float_as_uint(o0.w);
-        const uint32_t thr = sm + o1.z, lut = sm + o1.w;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          if (HALF) x[h + e][r] = __half2float(__float2half_rn(x[h + e][r]));
-          const uint32_t d = __float_as_uint(__fadd_rn(fmaxf(x[h + e][r], o0.x), o0.y)) - base;
-          p[e][r] = thr + lds_u16(lut + min(d >> shift, o1.x) * 2u) * 4u;
-        }
-        origin += e == 0 ? thr >> 2 : thr << 14;
-        start[e] = thr;
+      for (int r = 0; r < S; ++r) {
+        if (HALF) x[h][r] = __half2float(__float2half_rn(x[h][r]));
+        const uint32_t d = __float_as_uint(__fadd_rn(fmaxf(x[h][r], o0.x), o0.y)) - base;
+        p[r] = thr + lds_u16(lut + min(d >> shift, o1.x) * 2u) * 4u;
       }
-      ord_search(steps, p, x[h]);
+      // lanes 2i search feature h0 + h, lanes 2i + 1 feature h0 + h + 4, which
+      // has the same number of steps
+      ord_search(__shfl_sync(0xFFFFFFFFu, o1.y, 0), p, x[h]);
       bool nan = false;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) nan |= x[h + (r >> 2)][r & 3] != x[h + (r >> 2)][r & 3];
+      for (int r = 0; r < S; ++r) nan |= x[h][r] != x[h][r];
       if (nan) {
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
-          if (x[h + (r >> 2)][r & 3] != x[h + (r >> 2)][r & 3]) {
-            p[r >> 2][r & 3] = start[r >> 2] + kOrdNan * 4u;
-            missing |= 1u << (r & 3);
+        for (int r = 0; r < S; ++r)
+          if (x[h][r] != x[h][r]) {
+            p[r] = thr + kOrdNan * 4u;
+            missing |= 1u << r;
           }
       }
-      if (h0 + h < nf) {
+      // (p - thr) / 4 of the pair in the low and high halves
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          // (p - thr) / 4 of the two features in the low and high halves; row
-          // slots 0, 1 are in the first block of 32, slots 2, 3 in the second
-          const uint32_t word = (p[0][r] >> 2) + (p[1][r] << 14) - origin;
-          if (sb * kOrdRows + (r >> 1) < blocks)
-            dst[((r >> 1) * F2 + (h >> 1)) * 32 + (r & 1) * 16 + (lane >> 1)] = word;
-        }
+      for (int r = 0; r < S; ++r)
+        word[r] = (h & 1) == 0 ? (p[r] - thr) >> 2 : word[r] + ((p[r] - thr) << 14);
+      if ((h & 1) == 1 && h0 + h - 1 < nf) {
+        // row slots 2b, 2b + 1 are the halves of block b of the item
+#pragma unroll
+        for (int r = 0; r < S; ++r)
+          if (sb * kRows + (r >> 1) < blocks) dst[((r >> 1) * F2 + (h >> 1)) * 32 + (r & 1) * 16] = word[r];
       }
     }
     missing = __reduce_or_sync(0xFFFFFFFFu, missing);
-    if (lane < kOrdRows && sb * kOrdRows + lane < blocks)
-      a.nan_flags[(sb * kOrdRows + lane) * F8 + ((g.first + f0) >> 3)] = (missing >> (2 * lane)) & 3u ? 1 : 0;
+    if (lane < kRows && sb * kRows + lane < blocks)
+      a.nan_flags[(sb * kRows + lane) * F8 + ((g.first + f0) >> 3)] = (missing >> (2 * lane)) & 3u ? 1 : 0;
   }
 }
 
@@ -608,15 +610,19 @@ cudaError_t launch_ordinals(const OrdTable& t, OrdArgs a, long long n_max, int s
   // one wave of CTAs, spread over the groups by their features
   int chunks = 0;
   for (int g = 0; g < t.n_groups; ++g) chunks += t.chunks[g];
+  const bool wide = n_max / 128 * chunks >= static_cast<long long>(sms) * (kOrdThreads / 32);
+  const long long supers = (n_max + (wide ? 127 : 63)) / (wide ? 128 : 64);
   const int spare = std::max(0, sms - t.n_groups);  // one CTA of 32 warps an SM
   a.first_cta[0] = 0;
   for (int g = 0; g < t.n_groups; ++g) {
-    const long long supers = (n_max + 32 * kOrdRows - 1) / (32 * kOrdRows);
     const long long ctas = std::min(supers * t.chunks[g], 1 + static_cast<long long>(spare) * t.chunks[g] / chunks);
     a.first_cta[g + 1] = static_cast<unsigned short>(a.first_cta[g] + ctas);
   }
-  auto k = a.vec4 ? (t.round_half ? k_ordinals<true, true> : k_ordinals<true, false>)
-                  : (t.round_half ? k_ordinals<false, true> : k_ordinals<false, false>);
+  auto pick = [&](auto narrow_k, auto wide_k) { return wide ? wide_k : narrow_k; };
+  auto k = a.vec4 ? (t.round_half ? pick(k_ordinals<true, true, 4>, k_ordinals<true, true, 8>)
+                                  : pick(k_ordinals<true, false, 4>, k_ordinals<true, false, 8>))
+                  : (t.round_half ? pick(k_ordinals<false, true, 4>, k_ordinals<false, true, 8>)
+                                  : pick(k_ordinals<false, false, 4>, k_ordinals<false, false, 8>));
   cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(k, dim3(a.first_cta[t.n_groups]), dim3(kOrdThreads), smem, st, a);

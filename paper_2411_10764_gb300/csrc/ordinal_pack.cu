@@ -15,9 +15,9 @@
 namespace mlt {
 namespace {
 
-// Bytes of thresholds and lookup tables that a feature group aims at: two
-// CTAs of the ordinal kernel share an SM.
-constexpr uint32_t kGroupBytes = 80 * 1024;
+// Bytes of thresholds and lookup tables that a feature group aims at (every CTA
+// of the ordinal kernel copies its group's).
+constexpr uint32_t kGroupBytes = 120 * 1024;
 constexpr uint32_t kGroupMaxBytes = 220 * 1024;  // more thresholds in eight features: no ordinal form
 
 // A threshold's place in the order of the floats (+0 counts as -0).
@@ -268,11 +268,15 @@ bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool rou
   uint32_t total = 0;
   t.max_bytes = 0;
   for (int f = 0; f < F8; f += 8) {
-    // eight features are searched with the same number of compares; a search
-    // may read 2^steps - 1 entries past the bucket's start
-    uint32_t steps = 0;
-    for (int q = f; q < f + 8; ++q) steps = std::max(steps, steps_for(buckets[q].most));
-    auto thr_bytes = [&](int q) { return static_cast<uint32_t>((keys[q].size() + (1u << steps)) * 4 + 15) & ~15u; };
+    // features 4 apart are searched together with the larger number of
+    // compares; a search may read 2^steps - 1 entries past the bucket's start
+    auto steps_of = [&](int q) {
+      const int other = (q & 4) ? q - 4 : q + 4;  // f is a multiple of 8
+      return std::max(steps_for(buckets[q].most), steps_for(buckets[other].most));
+    };
+    auto thr_bytes = [&](int q) {
+      return static_cast<uint32_t>((keys[q].size() + (1u << steps_of(q))) * 4 + 15) & ~15u;
+    };
     auto lut_bytes = [&](int q) { return (buckets[q].count * 2u + 15u) & ~15u; };
     uint32_t eight = 0;
     for (int q = f; q < f + 8; ++q) eight += thr_bytes(q) + lut_bytes(q);
@@ -292,7 +296,7 @@ bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool rou
       feat[q].base = buckets[q].base;
       feat[q].shift = buckets[q].shift;
       feat[q].last = buckets[q].count - 1;
-      feat[q].steps = steps;
+      feat[q].steps = steps_of(q);
       g.bytes += thr_bytes(q) + lut_bytes(q);
     }
     total += eight;
