@@ -244,8 +244,9 @@ int ensure_scratch(long long n) {
   if (g_scr.err == nullptr || g_scr.device != dev) {
     if (g_scr.device != -1 && g_scr.device != dev)
       return fail(MLT_EINVAL, "libmlt scratch lives on device %d, current device is %d", g_scr.device, dev);
-    MLT_CUDA(cudaMalloc(&g_scr.err, sizeof(unsigned int)), "cudaMalloc(error word)");
-    MLT_CUDA(cudaMemset(g_scr.err, 0, sizeof(unsigned int)), "cudaMemset(error word)");
+    // the error word, and the rerank's ticket after it
+    MLT_CUDA(cudaMalloc(&g_scr.err, 2 * sizeof(unsigned int)), "cudaMalloc(error word)");
+    MLT_CUDA(cudaMemset(g_scr.err, 0, 2 * sizeof(unsigned int)), "cudaMemset(error word)");
     MLT_CUDA(cudaMalloc(&g_scr.state, sizeof(SelectState)), "cudaMalloc(select state)");
     MLT_CUDA(cudaMemset(g_scr.state, 0, sizeof(SelectState)), "cudaMemset(select state)");
     MLT_CUDA(cudaMalloc(&g_scr.rerank_keys, sizeof(unsigned long long) * kMaxK), "cudaMalloc(rerank keys)");
@@ -1433,9 +1434,9 @@ int mlt_rerank(void* stream, const float* feats, int64_t n, const int64_t* cand,
   rc = ensure_scratch(0);
   if (rc != MLT_OK) return rc;
   MLT_CUDA(launch_rerank(A.dm, feats, g_F, n, cand, m, n_final, out_score, out_final, g_scr.rerank_keys, g_scr.err,
-                         static_cast<cudaStream_t>(stream)),
+                         g_scr.err + 1, static_cast<cudaStream_t>(stream)),
            "rerank launch");
-  g_launches += (m > 0 ? 1 : 0) + 1;
+  g_launches += m > 0 && !rerank_fused(m) ? 2 : 1;
   return MLT_OK;
 }
 

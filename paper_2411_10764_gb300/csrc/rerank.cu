@@ -9,8 +9,9 @@
 // different trees straight from global memory (L1/L2) -- one tree each when
 // the batch is small enough to spread over the GPU -- leaves parked in
 // shared memory and added by one thread in tree order (the same exact fp32
-// sequential sum as the screening walk).  One CTA then sorts the 64-bit keys
-// (score, index).
+// sequential sum as the screening walk).  The 64-bit keys (score, index) are
+// then ordered: up to 512 by the last walk CTA to finish (a ticket), each key
+// counting the better ones; more by a CTA of its own with a bitonic sort.
 #include <algorithm>
 
 #include "mlt_internal.cuh"
@@ -20,6 +21,7 @@ namespace {
 
 constexpr int kTreeChunk = 1024;  // leaves parked before summing
 constexpr int kSelectThreads = 1024;
+constexpr int kRerankFused = 512;  // candidates that the last walk CTA orders itself
 
 __device__ __forceinline__ uint32_t go_right_nan(float x, uint32_t thr_bits, uint32_t meta) {
   uint32_t right = x >= __uint_as_float(thr_bits) ? 1u : 0u;
@@ -76,12 +78,38 @@ struct RerankArgs {
   float* out_score;
   unsigned long long* keys;
   unsigned* err;
+  // fused selection (ticket null: k_rerank_select follows)
+  unsigned* ticket;  // zero before and after the call
+  int n_final;
+  int64_t* out_final;
 };
 
-__global__ void __launch_bounds__(1024) k_rerank_walk(const __grid_constant__ RerankArgs a) {
-  __shared__ float parked[kTreeChunk];
-  pdl_wait();
-  const int i = blockIdx.x;  // one candidate per CTA
+// The place of every key among keys[0, m) (larger first, equal keys by
+// position) by the whole CTA; out[r] for r < n_final.  `part` threads share a
+// key's comparisons.
+__device__ void rank_keys(const unsigned long long* keys, int m, int n_final, int64_t* out, unsigned long long* sk) {
+  const int T = blockDim.x, tid = threadIdx.x;
+  for (int i = tid; i < m; i += T) sk[i] = __ldcg(keys + i);
+  for (int r = m + tid; r < n_final; r += T) out[r] = -1;
+  __syncthreads();
+  int part = 1;
+  while (part < 32 && 2 * part * m <= T) part <<= 1;
+  const int span = m * part;
+  for (int t0 = 0; t0 < span; t0 += T) {  // the same trip count in every thread
+    const int t = t0 + tid, i = t / part;
+    unsigned long long key = 0;
+    int r = 0;
+    if (t < span) {
+      key = sk[i];
+      for (int j = t % part; j < m; j += part) r += sk[j] > key || (sk[j] == key && j < i);
+    }
+    for (int o = 1; o < part; o <<= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
+    if (t < span && t % part == 0 && r < n_final)
+      out[r] = key == 0ull ? -1 : static_cast<int64_t>(0xFFFFFFFFu - static_cast<uint32_t>(key & 0xFFFFFFFFull));
+  }
+}
+
+__device__ void rerank_score(const RerankArgs& a, int i, float* parked) {
   const long long c = a.cand[i];
   if (c < 0 || c >= a.n) {
     if (threadIdx.x == 0) {
@@ -115,6 +143,24 @@ __global__ void __launch_bounds__(1024) k_rerank_walk(const __grid_constant__ Re
   }
 }
 
+__global__ void __launch_bounds__(1024) k_rerank_walk(const __grid_constant__ RerankArgs a) {
+  __shared__ float parked[kTreeChunk];
+  __shared__ unsigned long long sk[kRerankFused];
+  __shared__ unsigned last;
+  pdl_wait();
+  rerank_score(a, blockIdx.x, parked);  // one candidate per CTA
+  if (a.ticket == nullptr) return;
+  if (threadIdx.x == 0) {  // wrote this CTA's key
+    __threadfence();
+    last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x == 0) *a.ticket = 0u;
+  rank_keys(a.keys, a.m, a.n_final, a.out_final, sk);
+}
+
 __global__ void __launch_bounds__(kSelectThreads)
     k_rerank_select(const unsigned long long* keys, int m, int m2, int n_final, int64_t* out) {
   extern __shared__ __align__(16) unsigned long long sk[];
@@ -145,9 +191,12 @@ __global__ void __launch_bounds__(kSelectThreads)
 
 }  // namespace
 
+bool rerank_fused(int m) { return m > 0 && m <= kRerankFused; }
+
 cudaError_t launch_rerank(const DeviceModel& A, const float* feats, int F, long long n, const int64_t* cand, int m,
                           int n_final, float* out_score, int64_t* out_final, unsigned long long* keys,
-                          unsigned* err, cudaStream_t st) {
+                          unsigned* err, unsigned* ticket, cudaStream_t st) {
+  const bool fused = rerank_fused(m);
   if (m > 0) {
     RerankArgs a{};
     a.feats = feats;
@@ -163,6 +212,9 @@ cudaError_t launch_rerank(const DeviceModel& A, const float* feats, int F, long 
     a.out_score = out_score;
     a.keys = keys;
     a.err = err;
+    a.ticket = fused ? ticket : nullptr;
+    a.n_final = n_final;
+    a.out_final = out_final;
     // threads per candidate: one per tree (a multiple of 32, at most 1,024),
     // fewer when the batch would hold more than 2,048 threads per SM
     int sms = 0, dev = 0;
@@ -171,7 +223,7 @@ cudaError_t launch_rerank(const DeviceModel& A, const float* feats, int F, long 
     const long long fill = std::max(32LL, static_cast<long long>(sms > 0 ? sms : 1) * 2048 / m / 32 * 32);
     const int threads = static_cast<int>(std::min<long long>({(A.n_trees + 31) / 32 * 32, 1024LL, fill}));
     cudaError_t e = launch_pdl(k_rerank_walk, dim3(static_cast<unsigned>(m)), dim3(threads), 0, st, a);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || fused) return e;
   }
   int m2 = 1;
   while (m2 < m) m2 <<= 1;
