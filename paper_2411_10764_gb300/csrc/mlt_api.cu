@@ -1144,17 +1144,26 @@ int pack_ensemble_half(const mlt_node* nodes, int n_trees, int depth, int F, std
 }
 
 // Upload a packed table into model slot `model_id` (lock held).
-int install_model(int model_id, const std::vector<unsigned char>& packed, const DeviceModel& dm) {
+// `base` bytes of it are the model; the rest is its ordinal form, left out
+// where the device has no room for both.
+int install_model(int model_id, const std::vector<unsigned char>& packed, size_t base, DeviceModel dm) {
   int dev = 0;
   int rc = current_device(&dev);
   if (rc != MLT_OK) return rc;
   unsigned char* d = nullptr;
-  cudaError_t e = cudaMalloc(&d, packed.size());
+  size_t bytes = packed.size();
+  cudaError_t e = cudaMalloc(&d, bytes);
+  if (e != cudaSuccess && bytes > base) {
+    cudaGetLastError();
+    bytes = base;
+    dm.ord = OrdTable();
+    e = cudaMalloc(&d, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
-    return fail(MLT_ENOMEM, "cannot allocate %zu bytes for the ensemble", packed.size());
+    return fail(MLT_ENOMEM, "cannot allocate %zu bytes for the ensemble", bytes);
   }
-  e = cudaMemcpy(d, packed.data(), packed.size(), cudaMemcpyHostToDevice);
+  e = cudaMemcpy(d, packed.data(), bytes, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(d);
     return cuda_fail(e, "ensemble upload");
@@ -1167,7 +1176,7 @@ int install_model(int model_id, const std::vector<unsigned char>& packed, const 
   m.owned = d;
   m.dm = dm;
   m.dm.table = d;
-  m.dm.bytes = packed.size();
+  m.dm.bytes = base;
   if (dm.kind == kTableSplit) m.dm.tail = d + dm.tail_off;
   OrdTable& o = m.dm.ord;
   if (o.n_trees > 0) {
@@ -1210,9 +1219,10 @@ int mlt_load_ensemble(int model_id, const mlt_node* nodes, int n_trees, int dept
   int rc = split ? pack_split(nodes, n_trees, depth, g_F, g_head_levels, packed, dm)
                  : pack_ensemble(nodes, n_trees, depth, g_F, packed, dm);
   if (rc != MLT_OK) return rc;
+  const size_t base = packed.size();
   if ((dm.kind == kTableFull || dm.kind == kTableSplit) && model_id != MLT_MODEL_A)
     pack_ordinal(nodes, n_trees, depth, g_F, false, packed, dm.ord);
-  return install_model(model_id, packed, dm);
+  return install_model(model_id, packed, base, dm);
 }
 
 int mlt_tune_decode_jit(int64_t min_n) {
@@ -1268,8 +1278,9 @@ int mlt_load_ensemble_f16(int model_id, const mlt_node* nodes, int n_trees, int 
   DeviceModel dm;
   int rc = pack_ensemble_half(nodes, n_trees, depth, g_F, packed, dm);
   if (rc != MLT_OK) return rc;
+  const size_t base = packed.size();
   pack_ordinal(nodes, n_trees, depth, g_F, true, packed, dm.ord);
-  return install_model(model_id, packed, dm);
+  return install_model(model_id, packed, base, dm);
 }
 
 int mlt_free_ensemble(int model_id) {

@@ -1,6 +1,7 @@
 // Builds the ordinal form of a full-table model on the host (layout:
 // ordinal.cuh).  Host code only.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <limits>
@@ -74,25 +75,37 @@ uint32_t steps_for(uint32_t m) {
   return s;
 }
 
+// body(f) for f in [0, n) on a few threads; false if one could not finish (no
+// exception leaves a thread, and a thread that cannot be had is done without).
 template <typename F>
-void for_features(int n, F&& body) {
+bool for_features(int n, F&& body) {
   const int workers = std::max(1, std::min<int>({8, static_cast<int>(std::thread::hardware_concurrency()), n / 8}));
-  if (workers == 1) {
-    for (int f = 0; f < n; ++f) body(f);
-    return;
-  }
-  std::vector<std::thread> pool;
-  for (int w = 0; w < workers; ++w)
-    pool.emplace_back([&, w] {
+  std::atomic<bool> ok{true};
+  auto share = [&](int w) {
+    try {
       for (int f = w; f < n; f += workers) body(f);
-    });
+    } catch (...) {
+      ok = false;
+    }
+  };
+  std::vector<std::thread> pool;
+  pool.reserve(workers);
+  int started = 1;
+  try {
+    for (; started < workers; ++started) pool.emplace_back(share, started);
+  } catch (...) {
+  }
+  share(0);
+  for (int w = started; w < workers; ++w) share(w);
   for (std::thread& t : pool) t.join();
+  return ok;
 }
 
 }  // namespace
 
-bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
-                  std::vector<unsigned char>& out, OrdTable& t) {
+namespace {
+bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half, std::vector<unsigned char>& out,
+          OrdTable& t) {
   const int slots = (2 << depth) - 1;
   const bool deep = depth > kMaxFullDepth;
   const int padded = (n_trees + kOrdTreePad - 1) / kOrdTreePad * kOrdTreePad;
@@ -224,7 +237,7 @@ bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool rou
   std::vector<std::vector<float>> keys(F);  // distinct thresholds, ascending
   std::vector<Buckets> buckets(F);
   std::vector<unsigned char> fits(F, 1);
-  for_features(F, [&](int f) {
+  if (!for_features(F, [&](int f) {
     auto b = sorted.begin() + start[f], e = sorted.begin() + start[f + 1];
     std::sort(b, e);
     std::vector<float>& k = keys[f];
@@ -256,7 +269,8 @@ bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool rou
       best = less;
     }
     buckets[f] = best;
-  });
+      }))
+    return false;
   if (std::find(fits.begin(), fits.end(), 0) != fits.end()) return false;
   // the table is padded to a multiple of 8 features; one without thresholds
   // has a bucket of its own and nothing but padding (ordinal 0)
@@ -333,6 +347,22 @@ bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool rou
   t.n_groups = static_cast<int>(groups.size());
   t.round_half = round_half ? 1 : 0;
   return true;
+}
+}  // namespace
+
+bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
+                  std::vector<unsigned char>& out, OrdTable& t) {
+  const size_t before = out.size();
+  bool ok = false;
+  try {
+    ok = pack(nodes, n_trees, depth, F, round_half, out, t);
+  } catch (const std::exception&) {  // no memory: the model does without
+  }
+  if (!ok) {
+    out.resize(before);
+    t = OrdTable();
+  }
+  return ok;
 }
 
 }  // namespace mlt

@@ -74,3 +74,16 @@ def test_screening_from_rows(n, first):
         g.replay()
         mlt.sync_status()
         assert_parity((outs[0].cpu().numpy(), outs[1].cpu().numpy(), outs[2].cpu().numpy(), s), (opv, opf, otk, s))
+        # with the buffers in place the capture holds the row decoder and the
+        # ordinal walk; other calls in between leave the replay its results
+        mlt.screen_decoded(d.radices, d.option_values, d.program, first, n, 0.5, 200)
+        g2 = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g2):
+            mlt.screen_decoded(d.radices, d.option_values, d.program, first, n, 0.5, 200, out_pvalid=outs[0],
+                               out_perf=outs[1], out_topk=outs[2])
+        mlt.screen(torch.zeros((n, 70), device="cuda"), 0.5, 200)
+        for t in outs:
+            t.zero_()
+        g2.replay()
+        mlt.sync_status()
+        assert_parity((outs[0].cpu().numpy(), outs[1].cpu().numpy(), outs[2].cpu().numpy(), s), (opv, opf, otk, s))
