@@ -155,7 +155,7 @@ struct alignas(16) OrdFeature {
   uint32_t base;   // bits of c
   uint32_t shift;  // bits below a bucket
   uint32_t last;   // last bucket
-  uint32_t steps;  // compares after the lookup, the same for features f and f ^ 4
+  uint32_t steps;  // compares after the lookup: of features f and f ^ 4 together, of all 8 << 8
   uint32_t thr;    // byte offset of its thresholds in its group's image
   uint32_t lut;    // byte offset of its lookup table
 };

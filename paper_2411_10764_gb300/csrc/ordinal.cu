@@ -55,6 +55,58 @@ __device__ __forceinline__ void ord_search(uint32_t steps, uint32_t (&p)[S], con
   }
 }
 
+// Rows without 16-byte alignment: a warp takes 32 rows and 8 features, a lane one
+// feature of every fourth row (slot r: row 4 r + lane / 8), so a load covers
+// four rows' 32 bytes where four scalar loads of a half row each touched 16
+// lines.  Neighbouring lanes then exchange ordinals: an even lane stores the
+// pair's word of slots 0, 2, 4, 6, the odd one of slots 1, 3, 5, 7.  300,007 x
+// 101 with missing values, whole call: 540 us with scalar loads of half rows,
+// 503 so.
+template <bool HALF>
+__device__ __forceinline__ void ord_unaligned(const OrdArgs& a, const OrdFeature* feat, uint32_t sm, int first, int f0,
+                                              int nf, long long block, long long count, int F2, int F8) {
+  const int lane = threadIdx.x & 31, h = lane & 7;
+  const bool mine = f0 + h < nf;
+  float x[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const long long i = block * 32 + r * 4 + (lane >> 3);
+    const bool in = i < count && mine;
+    const long long row = in ? (a.rows ? static_cast<long long>(a.rows[i]) : i) : 0;
+    x[r] = in ? __ldg(a.feats + row * a.F + first + f0 + h) : 0.0f;
+    if (HALF) x[r] = __half2float(__float2half_rn(x[r]));
+  }
+  const float4 o0 = __ldg(reinterpret_cast<const float4*>(feat + f0 + h));
+  const uint4 o1 = __ldg(reinterpret_cast<const uint4*>(feat + f0 + h) + 1);
+  const uint32_t base = __float_as_uint(o0.z), shift = __float_as_uint(o0.w);
+  const uint32_t thr = sm + o1.z, lut = sm + o1.w;
+  uint32_t p[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const uint32_t d = __float_as_uint(__fadd_rn(fmaxf(x[r], o0.x), o0.y)) - base;
+    p[r] = thr + lds_u16(lut + min(d >> shift, o1.x) * 2u) * 4u;
+  }
+  ord_search(__shfl_sync(0xFFFFFFFFu, o1.y >> 8, 0), p, x);  // the compares of all eight features
+  bool nan = false;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const bool missing = x[r] != x[r];
+    nan |= missing;
+    p[r] = missing ? kOrdNan : (p[r] - thr) >> 2;
+  }
+  const bool odd = lane & 1;
+  uint32_t* dst = a.out + (block * F2 + ((first + f0 + h) >> 1)) * 32 + (lane >> 3);
+#pragma unroll
+  for (int r = 0; r < 8; r += 2) {
+    // the even lane gives slot r + 1 and gets the odd lane's slot r
+    const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, odd ? p[r] : p[r + 1], 1);
+    const uint32_t word = odd ? (other | p[r + 1] << 16) : (p[r] | other << 16);
+    if (f0 + (h & ~1) < nf) dst[(odd ? r + 1 : r) * 4] = word;
+  }
+  const bool any = __any_sync(0xFFFFFFFFu, nan);
+  if (lane == 0) a.nan_flags[block * F8 + ((first + f0) >> 3)] = any ? 1 : 0;
+}
+
 // A CTA holds one feature group's thresholds and lookup tables in shared
 // memory.  A warp takes 16 S rows and 8 features (one 32-byte sector of each
 // row) at a time: lanes 2i and 2i + 1 read the two halves of a row's sector
@@ -69,7 +121,8 @@ __device__ __forceinline__ void ord_search(uint32_t steps, uint32_t (&p)[S], con
 // with 4).
 template <bool VEC, bool HALF, int S>
 __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_constant__ OrdArgs a) {
-  constexpr int kRows = S / 2;  // blocks of 32 rows a warp takes together
+  constexpr int kRows = VEC ? S / 2 : 1;  // blocks of 32 rows a warp takes together
+  static_assert(VEC || S == 8, "unaligned rows: 8 slots of 4 rows");
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) unsigned long long bar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -114,6 +167,10 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
     const uint32_t s32 = it / static_cast<uint32_t>(chunks);
     const int f0 = static_cast<int>(it - s32 * chunks) * 8;
     const long long sb = s32;
+    if constexpr (!VEC) {
+      ord_unaligned<HALF>(a, feat, sm, static_cast<int>(g.first), f0, nf, sb, count, F2, F8);
+      continue;
+    }
     // row slot r of this lane: row 16 r + lane / 2 of the item; features h0 .. h0 + 3
     const int h0 = f0 + (lane & 1) * 4;
     float x[4][S];  // [feature][row slot]
@@ -123,16 +180,11 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
       const bool in = i < count && h0 < nf;
       const long long row = in ? (a.rows ? static_cast<long long>(a.rows[i]) : i) : 0;
       const float* src = a.feats + row * a.F + g.first + h0;
-      if constexpr (VEC) {
-        const float4 v = in ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        x[0][r] = v.x;
-        x[1][r] = v.y;
-        x[2][r] = v.z;
-        x[3][r] = v.w;
-      } else {
-#pragma unroll
-        for (int h = 0; h < 4; ++h) x[h][r] = in && h0 + h < nf ? __ldg(src + h) : 0.0f;
-      }
+      const float4 v = in ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      x[0][r] = v.x;
+      x[1][r] = v.y;
+      x[2][r] = v.z;
+      x[3][r] = v.w;
     }
     // ordinals of a row slot: words of pairs (h0, h0 + 1) and (h0 + 2, h0 + 3)
     uint32_t* dst = a.out + (sb * kRows * F2 + ((g.first + h0) >> 1)) * 32 + (lane >> 1);
@@ -153,7 +205,7 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
       }
       // lanes 2i search feature h0 + h, lanes 2i + 1 feature h0 + h + 4, which
       // has the same number of steps
-      ord_search(__shfl_sync(0xFFFFFFFFu, o1.y, 0), p, x[h]);
+      ord_search(__shfl_sync(0xFFFFFFFFu, o1.y & 0xFFu, 0), p, x[h]);
       bool nan = false;
 #pragma unroll
       for (int r = 0; r < S; ++r) nan |= x[h][r] != x[h][r];
@@ -610,8 +662,9 @@ cudaError_t launch_ordinals(const OrdTable& t, OrdArgs a, long long n_max, int s
   // one wave of CTAs, spread over the groups by their features
   int chunks = 0;
   for (int g = 0; g < t.n_groups; ++g) chunks += t.chunks[g];
-  const bool wide = n_max / 128 * chunks >= static_cast<long long>(sms) * (kOrdThreads / 32);
-  const long long supers = (n_max + (wide ? 127 : 63)) / (wide ? 128 : 64);
+  const bool wide = a.vec4 && n_max / 128 * chunks >= static_cast<long long>(sms) * (kOrdThreads / 32);
+  const int rows = !a.vec4 ? 32 : wide ? 128 : 64;  // of a warp at a time
+  const long long supers = (n_max + rows - 1) / rows;
   const int spare = std::max(0, sms - t.n_groups);  // one CTA of 32 warps an SM
   a.first_cta[0] = 0;
   for (int g = 0; g < t.n_groups; ++g) {
@@ -621,8 +674,7 @@ cudaError_t launch_ordinals(const OrdTable& t, OrdArgs a, long long n_max, int s
   auto pick = [&](auto narrow_k, auto wide_k) { return wide ? wide_k : narrow_k; };
   auto k = a.vec4 ? (t.round_half ? pick(k_ordinals<true, true, 4>, k_ordinals<true, true, 8>)
                                   : pick(k_ordinals<true, false, 4>, k_ordinals<true, false, 8>))
-                  : (t.round_half ? pick(k_ordinals<false, true, 4>, k_ordinals<false, true, 8>)
-                                  : pick(k_ordinals<false, false, 4>, k_ordinals<false, false, 8>));
+                  : (t.round_half ? k_ordinals<false, true, 8> : k_ordinals<false, false, 8>);
   cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(k, dim3(a.first_cta[t.n_groups]), dim3(kOrdThreads), smem, st, a);

@@ -257,7 +257,7 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
     // leave as few
     const double range = std::min(3.0e38, std::max(1e-30, static_cast<double>(k.back()) - k.front()));
     Buckets best;
-    for (int q = 0; q < 26; ++q) {
+    for (int q = 0; q < 26; q += 2) {
       const Buckets b2 = buckets_for(k, std::max(1e-30f, static_cast<float>(std::ldexp(range, 1 - q))));
       if (q == 0 || steps_for(b2.most) < steps_for(best.most)) best = b2;
     }
@@ -288,9 +288,9 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
       const int other = (q & 4) ? q - 4 : q + 4;  // f is a multiple of 8
       return std::max(steps_for(buckets[q].most), steps_for(buckets[other].most));
     };
-    auto thr_bytes = [&](int q) {
-      return static_cast<uint32_t>((keys[q].size() + (1u << steps_of(q))) * 4 + 15) & ~15u;
-    };
+    uint32_t most = 0;  // unaligned rows: all eight together
+    for (int q = f; q < f + 8; ++q) most = std::max(most, steps_for(buckets[q].most));
+    auto thr_bytes = [&](int q) { return static_cast<uint32_t>((keys[q].size() + (1u << most)) * 4 + 15) & ~15u; };
     auto lut_bytes = [&](int q) { return (buckets[q].count * 2u + 15u) & ~15u; };
     uint32_t eight = 0;
     for (int q = f; q < f + 8; ++q) eight += thr_bytes(q) + lut_bytes(q);
@@ -310,7 +310,7 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
       feat[q].base = buckets[q].base;
       feat[q].shift = buckets[q].shift;
       feat[q].last = buckets[q].count - 1;
-      feat[q].steps = steps_of(q);
+      feat[q].steps = steps_of(q) | most << 8;
       g.bytes += thr_bytes(q) + lut_bytes(q);
     }
     total += eight;
