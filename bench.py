@@ -228,6 +228,7 @@ def walk_source_hash() -> str:
     files = [os.path.join(csrc, "walk.cuh"), os.path.join(csrc, "mlt_internal.cuh")]
     files += sorted(glob.glob(os.path.join(csrc, "traverse*.cu")))
     files += [os.path.join(csrc, "jit_decode.cu")]
+    files += sorted(glob.glob(os.path.join(csrc, "ordinal*")))
     h = hashlib.sha256()
     for path in files:
         with open(path, "rb") as f:
@@ -598,7 +599,7 @@ def measure_workload(ctx, w, args, headline: bool):
                                   "kernel instead)" if launches == steps else "planned shape of each pass's walk"}
     if w.decoder is not None:
         rec["decode_path"] = ("compiled feature program (NVRTC): rows written once per step, then screened"
-                              if jit_steps == steps else "interpreted inside the walk kernels")
+                              if jit_steps == steps else "interpreted: rows written once per step, then screened")
     if ctx.rank == 0 and ctx.world == 1 and not args.no_cpu_baseline:
         rec["cpu_baseline"] = cpu_baseline(w, args.cpu_seconds if headline else args.cpu_seconds_per_config)
     return rec, bufs
