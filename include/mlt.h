@@ -380,8 +380,10 @@ int mlt_selftest_walk_timeout(int cta, int64_t limit_ns);
  * collected keys, two CTA tickets) of the selection state that the
  * allocating entry points (static_scratch = 0) or mlt_screen_noalloc
  * (static_scratch != 0) use on the current device, as a call that stopped
- * part-way could leave them.  Every screening call clears that state before
- * its kernels run, so results must not change.  Synchronous. */
+ * part-way could leave them, and with static_scratch = 0 also its low 16
+ * bits into the arrival count of mlt_rerank's last call.  Every screening call
+ * clears that state before its kernels run and every rerank counts from a
+ * number of its own, so results must not change.  Synchronous. */
 int mlt_selftest_poison_state(int static_scratch, uint32_t value);
 
 /* Number of valid candidates found by the last screening call (waits for

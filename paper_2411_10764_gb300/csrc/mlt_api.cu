@@ -82,6 +82,14 @@ struct Model {
   unsigned char* owned = nullptr;
 };
 
+// Whether `st` is being captured into a graph.
+bool is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const bool unknown = cudaStreamIsCapturing(st, &cs) != cudaSuccess;
+  if (unknown) cudaGetLastError();  // the default stream beside a capture
+  return unknown || cs != cudaStreamCaptureStatusNone;
+}
+
 // A device buffer sized by n x F: grown on demand and given back when the
 // feature count changes or a V or P model is freed.  A stream capture never
 // grows it (an allocation would end the capture), and a buffer that captured
@@ -93,10 +101,7 @@ struct GrowBuf {
   std::vector<void*> aside;
 
   bool ensure(size_t bytes, cudaStream_t st) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const bool unknown = cudaStreamIsCapturing(st, &cs) != cudaSuccess;
-    if (unknown) cudaGetLastError();  // the default stream beside a capture
-    const bool capturing = unknown || cs != cudaStreamCaptureStatusNone;
+    const bool capturing = is_capturing(st);
     if (bytes > cap) {
       if (capturing) return false;
       void* q = nullptr;
@@ -134,6 +139,8 @@ struct ScratchOwner {
   void* block = nullptr;  // one allocation for everything sized by n
   SelectState* state = nullptr;
   unsigned int* err = nullptr;
+  unsigned long long* rerank_arrivals = nullptr;  // after the error word
+  unsigned long long rerank_calls = 0;
   unsigned long long* rerank_keys = nullptr;  // [kMaxK]
   StreamState* stream = nullptr;              // batched accumulation
   // explorer proposal step buffers, grown with m
@@ -244,9 +251,10 @@ int ensure_scratch(long long n) {
   if (g_scr.err == nullptr || g_scr.device != dev) {
     if (g_scr.device != -1 && g_scr.device != dev)
       return fail(MLT_EINVAL, "libmlt scratch lives on device %d, current device is %d", g_scr.device, dev);
-    // the error word, and the rerank's ticket after it
-    MLT_CUDA(cudaMalloc(&g_scr.err, 2 * sizeof(unsigned int)), "cudaMalloc(error word)");
-    MLT_CUDA(cudaMemset(g_scr.err, 0, 2 * sizeof(unsigned int)), "cudaMemset(error word)");
+    // the error word, and the rerank's arrivals in the next 8 bytes
+    MLT_CUDA(cudaMalloc(&g_scr.err, 16), "cudaMalloc(error word)");
+    MLT_CUDA(cudaMemset(g_scr.err, 0, 16), "cudaMemset(error word)");
+    g_scr.rerank_arrivals = reinterpret_cast<unsigned long long*>(g_scr.err + 2);
     MLT_CUDA(cudaMalloc(&g_scr.state, sizeof(SelectState)), "cudaMalloc(select state)");
     MLT_CUDA(cudaMemset(g_scr.state, 0, sizeof(SelectState)), "cudaMemset(select state)");
     MLT_CUDA(cudaMalloc(&g_scr.rerank_keys, sizeof(unsigned long long) * kMaxK), "cudaMalloc(rerank keys)");
@@ -1444,10 +1452,14 @@ int mlt_rerank(void* stream, const float* feats, int64_t n, const int64_t* cand,
   if (A.device != dev) return fail(MLT_EINVAL, "model A lives on device %d, current device is %d", A.device, dev);
   rc = ensure_scratch(0);
   if (rc != MLT_OK) return rc;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // a captured call keeps the two launches: its replays would share one number
+  const bool fused = rerank_fused(m) && !is_capturing(st);
+  if (fused) ++g_scr.rerank_calls;
   MLT_CUDA(launch_rerank(A.dm, feats, g_F, n, cand, m, n_final, out_score, out_final, g_scr.rerank_keys, g_scr.err,
-                         g_scr.err + 1, static_cast<cudaStream_t>(stream)),
+                         fused ? g_scr.rerank_arrivals : nullptr, g_scr.rerank_calls, st),
            "rerank launch");
-  g_launches += m > 0 && !rerank_fused(m) ? 2 : 1;
+  g_launches += m > 0 && !fused ? 2 : 1;
   return MLT_OK;
 }
 
@@ -1690,6 +1702,10 @@ int mlt_selftest_poison_state(int static_scratch, uint32_t value) {
   if (rc != MLT_OK) return rc;
   const unsigned int words[4] = {value, value, value, value};  // survivors, n_cand, ticket, v_ticket
   MLT_CUDA(cudaMemcpy(s.state, words, sizeof(words), cudaMemcpyHostToDevice), "state write");
+  if (!static_scratch) {  // the last rerank's number, `value` arrivals
+    const unsigned long long a = (g_scr.rerank_calls << kRerankCallShift) + (value & 0xFFFFu);
+    MLT_CUDA(cudaMemcpy(g_scr.rerank_arrivals, &a, sizeof(a), cudaMemcpyHostToDevice), "rerank arrivals write");
+  }
   return MLT_OK;
 }
 

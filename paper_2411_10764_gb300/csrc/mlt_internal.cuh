@@ -470,8 +470,9 @@ cudaError_t launch_wait_selftest(unsigned* err, unsigned long long limit_ns, cud
 // rerank.cu
 cudaError_t launch_rerank(const DeviceModel& A, const float* feats, int F, long long n,
                           const int64_t* cand, int m, int n_final, float* out_score,
-                          int64_t* out_final, unsigned long long* keys, unsigned* err, unsigned* ticket,
-                          cudaStream_t st);
-bool rerank_fused(int m);  // whether that is one launch
+                          int64_t* out_final, unsigned long long* keys, unsigned* err, unsigned long long* arrivals,
+                          unsigned long long call, cudaStream_t st);
+bool rerank_fused(int m);  // whether that is one launch where `arrivals` is given
+constexpr int kRerankCallShift = 16;  // the word `arrivals` points to: call number << 16 | CTAs done
 
 }  // namespace mlt

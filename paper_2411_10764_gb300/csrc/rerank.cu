@@ -10,8 +10,9 @@
 // the batch is small enough to spread over the GPU -- leaves parked in
 // shared memory and added by one thread in tree order (the same exact fp32
 // sequential sum as the screening walk).  The 64-bit keys (score, index) are
-// then ordered: up to 512 by the last walk CTA to finish (a ticket), each key
-// counting the better ones; more by a CTA of its own with a bitonic sort.
+// then ordered: up to 512 by the last walk CTA to finish, each key counting the
+// better ones; more, and those of a captured call, by a CTA of its own with a
+// bitonic sort.
 #include <algorithm>
 
 #include "mlt_internal.cuh"
@@ -78,8 +79,9 @@ struct RerankArgs {
   float* out_score;
   unsigned long long* keys;
   unsigned* err;
-  // fused selection (ticket null: k_rerank_select follows)
-  unsigned* ticket;  // zero before and after the call
+  // fused selection (arrivals null: k_rerank_select follows)
+  unsigned long long* arrivals;
+  unsigned long long call;  // what the word holds before the call's first arrival
   int n_final;
   int64_t* out_final;
 };
@@ -148,16 +150,20 @@ __global__ void __launch_bounds__(1024) k_rerank_walk(const __grid_constant__ Re
   __shared__ unsigned long long sk[kRerankFused];
   __shared__ unsigned last;
   pdl_wait();
+  // The word is the call's number << kRerankCallShift | CTAs done.  Numbers only
+  // grow, so whatever an earlier call left (one that overlapped another, or
+  // stopped part-way) is below `call` and the maximum replaces it: every call
+  // counts from a known value, with no clearing before or after it.
+  if (a.arrivals != nullptr && threadIdx.x == 0) atomicMax(a.arrivals, a.call);
   rerank_score(a, blockIdx.x, parked);  // one candidate per CTA
-  if (a.ticket == nullptr) return;
+  if (a.arrivals == nullptr) return;
   if (threadIdx.x == 0) {  // wrote this CTA's key
     __threadfence();
-    last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+    last = atomicAdd(a.arrivals, 1ull) == a.call + gridDim.x - 1;
   }
   __syncthreads();
   if (!last) return;
   __threadfence();
-  if (threadIdx.x == 0) *a.ticket = 0u;
   rank_keys(a.keys, a.m, a.n_final, a.out_final, sk);
 }
 
@@ -195,8 +201,8 @@ bool rerank_fused(int m) { return m > 0 && m <= kRerankFused; }
 
 cudaError_t launch_rerank(const DeviceModel& A, const float* feats, int F, long long n, const int64_t* cand, int m,
                           int n_final, float* out_score, int64_t* out_final, unsigned long long* keys,
-                          unsigned* err, unsigned* ticket, cudaStream_t st) {
-  const bool fused = rerank_fused(m);
+                          unsigned* err, unsigned long long* arrivals, unsigned long long call, cudaStream_t st) {
+  const bool fused = arrivals != nullptr && rerank_fused(m);
   if (m > 0) {
     RerankArgs a{};
     a.feats = feats;
@@ -212,7 +218,8 @@ cudaError_t launch_rerank(const DeviceModel& A, const float* feats, int F, long 
     a.out_score = out_score;
     a.keys = keys;
     a.err = err;
-    a.ticket = fused ? ticket : nullptr;
+    a.arrivals = fused ? arrivals : nullptr;
+    a.call = call << kRerankCallShift;
     a.n_final = n_final;
     a.out_final = out_final;
     // threads per candidate: one per tree (a multiple of 32, at most 1,024),
