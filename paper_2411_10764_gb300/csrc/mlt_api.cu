@@ -591,17 +591,19 @@ int pack_ensemble(const mlt_node* nodes, int n_trees, int depth, int F, std::vec
 constexpr long long kOrdMinN = 256;
 int g_ord_mode = 1;  // 0: never, 1: by the rule, 2: wherever a model has an ordinal form
 
+// Cycles a node visit of the fp32 walk takes an SM, for 32 candidates.
+double fp32_visit_cycles(const DeviceModel& m) {
+  const double warps = std::max(1.0, std::min(16.0, std::floor(190.0 * 1024 / (128.0 * g_F))));
+  return 3.6 + 16.0 / warps + (m.kind == kTableSplit ? 4.0 : 0.0) + (m.kind == kTableFull && m.depth > 9 ? 1.0 : 0.0);
+}
+
 bool ord_wanted(const DeviceModel& m, const ShapeOverride& ov, long long n, long long n_eff) {
   if (m.ord.table == nullptr || g_ord_mode == 0) return false;
   if (ov.threads || ov.chunk_trees || ov.nbuf || ov.lanes || ov.group) return false;  // a fixed shape of the fp32 walk
   if (g_ord_mode == 2) return n > 0;
   if (n < kOrdMinN) return false;
   const double F = g_F, visits = m.ord.visits;
-  const double warps = std::max(1.0, std::min(16.0, std::floor(190.0 * 1024 / (128.0 * F))));
-  double fp32 = 3.6 + 16.0 / warps;
-  if (m.kind == kTableSplit) fp32 += 4.0;
-  if (m.kind == kTableFull && m.depth > 9) fp32 += 1.0;
-  const double cycles = visits * (fp32 - 2.8) - 20.0 * F;
+  const double cycles = visits * (fp32_visit_cycles(m) - 2.8) - 20.0 * F;
   const double us = static_cast<double>(n_eff) / 32.0 * cycles / (sm_count() * 2070.0) + 0.006 * visits;
   return us > 7.0;
 }
@@ -830,13 +832,58 @@ int noalloc_scratch(int dev, Scratch* out) {
 // and every later batch's kernels cost a launch each to find out that the
 // target was reached.  V walks a group of consecutive batches at once; k_cut
 // finds the batch that reaches `target` and drops the survivors past it; P
-// walks the rest.  A group holds at least kStreamRows candidates (one batch if
-// that is larger) and each is twice the one before, so that V walks at most
-// about twice what is consumed and a long run needs few launches.  One top-k
-// then ranks all survivors kept.  The result equals screening the consumed
-// prefix of the candidates as a single batch.
-constexpr long long kStreamRows = 24576;
-constexpr long long kStreamMostRows = 196608;
+// walks the rest.  One top-k then ranks all survivors kept.  The result equals
+// screening the consumed prefix of the candidates as a single batch.
+//
+// A group is whole batches, at least one, of up to max(group_rows, a third of
+// what is consumed before it) candidates; a rest of less than half a group (an
+// eighth, beside the first) joins the last, for a group that is skipped costs
+// its launches too.  What V walks past the batch that reaches the target is
+// less than that, and nothing where one batch is as large as a group: it is
+// then screened by itself, without a cut.
+//
+// group_rows: where a group's candidates cost about what any group costs
+// whatever its size.  Up to four warps of candidates an SM cost little beside
+// the chain of one walk and the group's launches; then come the candidates that
+// take 12 us, after the first group 36 (a skipped group costs 5 to 15).
+// Measured, us a group of 256 / 19,456 / 58,368 candidates (V, P trees x depth,
+// features), and group_rows of the first group:
+//     50 x 6, 100 x 6, 32: 21 / 37 / 47; 59,000
+//     200 x 8, 400 x 8, 64: 38 / 66 / 104; 30,000
+//     1,000 x 8, 100 x 6, 64: 52 / 90 / 175; 24,000
+//     1,000 x 12, 300 x 12, unbalanced, 64: 214 / 216 / 589; 21,000
+// Groups of 24,576, rounded up and doubled, walked up to three times what was
+// consumed: three batches of 24,576 through the last models, target in the
+// second, 872 us against 643 (one batch at a time: 649).
+constexpr double kGroupFirstUs = 12.0, kGroupLaterUs = 36.0;
+constexpr long long kGroupMostRows = 1LL << 19;  // bounds the row and ordinal buffers
+
+// Cycles of a pass on an SM for 32 candidates.
+double pass_cycles(const DeviceModel& m) {
+  const bool ord = m.ord.table != nullptr && g_ord_mode != 0;
+  const double visits = m.ord.visits > 0 ? m.ord.visits : static_cast<double>(m.n_trees) * m.depth;
+  return ord ? visits * (m.ord.rounds > 0 ? 10.0 : 2.8) + 20.0 * g_F : visits * fp32_visit_cycles(m);
+}
+
+struct GroupRows {
+  long long first, later;
+};
+GroupRows group_rows(const DeviceModel& V, const DeviceModel& P, bool decoded) {
+  // about half the candidates survive; the row decoder takes 24 cycles a feature
+  const double cycles = pass_cycles(V) + 0.5 * pass_cycles(P) + (decoded ? 24.0 * g_F : 0.0);
+  const double per_us = 2070.0 * sm_count() * 32.0 / cycles;
+  const double base = 128.0 * sm_count();
+  return {static_cast<long long>(base + kGroupFirstUs * per_us), static_cast<long long>(base + kGroupLaterUs * per_us)};
+}
+
+// Candidates of the group that starts at candidate `at`.
+long long next_group(long long at, long long n_total, long long batch, const GroupRows& rows) {
+  const long long least = at > 0 ? rows.later : rows.first;
+  const long long most = std::min(std::max(least, at / 3), kGroupMostRows);
+  const long long rest = n_total - at;
+  if (rest <= most + most / (at > 0 ? 2 : 8)) return rest;
+  return std::min(rest, std::max(1LL, most / batch) * batch);
+}
 
 int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, long long n_total, long long batch,
                long long target, float thr, int k, float* out_pvalid, float* out_perf, int64_t* out_topk,
@@ -852,14 +899,11 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
   StreamState* ss = g_scr.stream;
   const DeviceModel& V = g_models[MLT_MODEL_V].dm;
   const DeviceModel& P = g_models[MLT_MODEL_P].dm;
-  // the groups: whole batches, but the last one of the call
-  std::vector<long long> groups;
-  long long per = 1;  // candidates of the largest
-  for (long long at = 0, least = kStreamRows; at < n_total; least = std::min(2 * least, kStreamMostRows)) {
-    const long long g = std::min((least + batch - 1) / batch * batch, n_total - at);
-    groups.push_back(g);
+  const GroupRows most_rows = group_rows(V, P, dec0 != nullptr);
+  long long per = 1;  // candidates of the largest group
+  for (long long at = 0, g; at < n_total; at += g) {
+    g = next_group(at, n_total, batch, most_rows);
     per = std::max(per, g);
-    at += g;
   }
   // decoded batches: each group's rows are written first, as in run_screen_with
   const bool rows = dec0 != nullptr && per > 0 && g_scr.feats.ensure(static_cast<size_t>(per) * g_F * sizeof(float), st);
@@ -886,8 +930,8 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
   a.decode = dec0 != nullptr && !rows;
   a.stream = ss;
   long long launches = 0;
-  long long b0 = 0;
-  for (const long long nb : groups) {
+  for (long long b0 = 0, nb; b0 < n_total; b0 += nb) {
+    nb = next_group(b0, n_total, batch, most_rows);
     plan_passes(V, P, nb, dec0 == nullptr || rows, st, &pv, &pp);
     const ScreenShape& sv = pv.shape;
     TraverseArgs ab = a;
@@ -905,26 +949,29 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
       MLT_CUDA(launch_decode_rows(d, nb, nullptr, static_cast<float*>(g_scr.feats.p), st, ss), "decoder launch");
       launches += 1;
     }
-    TraverseArgs av = ab;
+    const bool cut = nb > batch;  // one batch is consumed whole
+    TraverseArgs ap = ab;
+    ap.p_pass = 1;
+    ap.out_perf = out_perf ? out_perf + b0 : nullptr;
+    TraverseArgs av = cut ? ab : ap;
     av.p_pass = 0;
-    av.out_pvalid = out_pvalid ? group_pvalid : nullptr;
+    av.out_pvalid = !out_pvalid ? nullptr : cut ? group_pvalid : out_pvalid + b0;
     const long long tiles_v = (nb + sv.threads - 1) / sv.threads;
     MLT_CUDA(launch_pass(V, av, pv, walk_dec, nb, st, &launches), "V pass launch");
     MLT_CUDA(launch_compact(s, nb, sv.threads, tiles_v, ss, st), "compaction launch");
-    MLT_CUDA(launch_cut(ss, s.state, s.rows, nb, batch, tgt, st), "cut launch");
-    if (out_pvalid || out_perf) {
+    if (cut) {
+      MLT_CUDA(launch_cut(ss, s.state, s.rows, nb, batch, tgt, st), "cut launch");
+      launches += 1;
+    }
+    if (cut && (out_pvalid || out_perf)) {
       MLT_CUDA(launch_stream_out(ss, group_pvalid, s.masks, nb, out_pvalid ? out_pvalid + b0 : nullptr,
                                  out_perf ? out_perf + b0 : nullptr, st),
                "output launch");
       launches += 1;
     }
-    TraverseArgs ap = ab;
-    ap.p_pass = 1;
-    ap.out_perf = out_perf ? out_perf + b0 : nullptr;
     MLT_CUDA(launch_pass(P, ap, pp, walk_dec, nb, st, &launches), "P pass launch");
-    MLT_CUDA(launch_accumulate(ss, s.state, tgt, st), "accumulate launch");
-    launches += 3;
-    b0 += nb;
+    MLT_CUDA(launch_accumulate(ss, s.state, cut ? 0 : nb, tgt, st), "accumulate launch");
+    launches += 2;
   }
   MLT_CUDA(launch_topk(s, n_total, k, dec0 ? dec0->first_index : 0, out_topk, sm_count(), &ss->total, st),
            "top-k launch");

@@ -436,7 +436,8 @@ cudaError_t launch_cut(StreamState* ss, SelectState* st_, const uint32_t* rows, 
 // pvalid and the invalid candidates' perf of the group's consumed candidates
 cudaError_t launch_stream_out(const StreamState* ss, const float* pvalid, const uint32_t* masks, long long n,
                               float* out_pvalid, float* out_perf, cudaStream_t st);
-cudaError_t launch_accumulate(StreamState* ss, SelectState* st_, unsigned target, cudaStream_t st);
+cudaError_t launch_accumulate(StreamState* ss, SelectState* st_, long long one_batch, unsigned target,
+                              cudaStream_t st);
 cudaError_t launch_stream_stats(const StreamState* ss, int64_t* out_stats, cudaStream_t st);
 
 // sa.cu (explorer proposal step)

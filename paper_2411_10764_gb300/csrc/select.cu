@@ -279,14 +279,15 @@ __global__ void __launch_bounds__(256)
 }
 
 // After a group: add its survivors and candidates to the running counts and
-// raise `done` once the target is reached.
-__global__ void k_accumulate(StreamState* ss, SelectState* st, unsigned target) {
+// raise `done` once the target is reached.  one_batch: the group is a single
+// batch of that many candidates (0: k_cut has counted what it consumed).
+__global__ void k_accumulate(StreamState* ss, SelectState* st, long long one_batch, unsigned target) {
   pdl_wait();
   if (threadIdx.x != 0 || ss->done) return;
   ss->total += st->survivors;
-  ss->consumed += ss->cut_rows;
-  ss->batches += ss->cut_batches;
-  st->survivors = ss->last_survivors;  // what the last batch by itself had
+  ss->consumed += one_batch > 0 ? static_cast<unsigned long long>(one_batch) : ss->cut_rows;
+  ss->batches += one_batch > 0 ? 1u : ss->cut_batches;
+  if (one_batch == 0) st->survivors = ss->last_survivors;  // what the last batch by itself had
   if (ss->total >= target) ss->done = 1u;
 }
 
@@ -312,8 +313,9 @@ cudaError_t launch_stream_out(const StreamState* ss, const float* pvalid, const 
                     out_pvalid, out_perf);
 }
 
-cudaError_t launch_accumulate(StreamState* ss, SelectState* st_, unsigned target, cudaStream_t st) {
-  return launch_pdl(k_accumulate, dim3(1), dim3(32), 0, st, ss, st_, target);
+cudaError_t launch_accumulate(StreamState* ss, SelectState* st_, long long one_batch, unsigned target,
+                              cudaStream_t st) {
+  return launch_pdl(k_accumulate, dim3(1), dim3(32), 0, st, ss, st_, one_batch, target);
 }
 
 cudaError_t launch_stream_stats(const StreamState* ss, int64_t* out_stats, cudaStream_t st) {

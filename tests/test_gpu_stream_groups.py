@@ -1,6 +1,7 @@
-"""Batched accumulation screens groups of batches at once (24,576 candidates,
-then twice as many each): the batch that reaches the target must still be the
-last one consumed, wherever in a group it lies, and nothing past it written."""
+"""Batched accumulation screens groups of batches at once: the batch that
+reaches the target must still be the last one consumed, wherever in a group it
+lies, and nothing past it written; and where a batch alone keeps the GPU busy,
+no group holds a second one for V to walk in vain."""
 import numpy as np
 import pytest
 
@@ -10,7 +11,7 @@ from paper_2411_10764_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-N = 80000  # groups of 24,576, 49,152 and the rest, in whole batches
+N = 80000  # two groups of small batches
 
 
 @pytest.fixture(scope="module")
@@ -69,3 +70,44 @@ def test_no_outputs(problem):
     _, _, tk, stats = _run(w, 1000, target, 64, with_outputs=False)
     assert stats[0] <= 30000 and stats[1] >= target
     assert np.array_equal(tk, O.topk(opf[:stats[0]], valid[:stats[0]], 64)[0])
+
+
+def _launches(n, batch):
+    """Kernels of one accumulation call over the loaded models (zero rows)."""
+    import torch
+
+    x = torch.zeros((n, 64), device="cuda")
+    mlt.screen_until(x, batch, 1 << 30, 0.5, 16, with_outputs=False)  # buffers and plans
+    before = mlt.kernel_launches()
+    mlt.screen_until(x, batch, 1 << 30, 0.5, 16, with_outputs=False)
+    mlt.sync_status()
+    return mlt.kernel_launches() - before
+
+
+def _load(vt, vd, pt, pd):
+    mlt.set_num_features(64)
+    for m, trees, depth in ((mlt.MLT_MODEL_V, vt, vd), (mlt.MLT_MODEL_P, pt, pd)):
+        e = W.make_ensemble(W.ScreenConfig(2, "groups", 64, 64, vt, vd, pt, pd, 0.5, 16, 0.5), "V" if m == mlt.MLT_MODEL_V
+                            else "P", W._RangeThresholds([(0.0, 1.0)] * 64), 7, n_trees=trees, depth=depth)
+        mlt.load_ensemble(m, e.nodes, e.n_trees, e.depth)
+
+
+@pytest.mark.parametrize("vt,vd,pt,pd,batch,batches,groups,cuts", [
+    (1000, 12, 300, 12, 24576, 4, 4, 0),  # a batch fills the GPU: one a group
+    (1000, 8, 100, 6, 24576, 3, 3, 0),
+    (1000, 12, 300, 12, 8192, 3, 2, 1),   # two batches, then the third
+    (1000, 12, 300, 12, 8192, 5, 2, 2),   # two batches, then three
+    (50, 6, 100, 6, 24576, 2, 1, 1),      # cheap walks: both together
+    (50, 6, 100, 6, 500, 40, 1, 1),
+])
+def test_groups(vt, vd, pt, pd, batch, batches, groups, cuts):
+    """`cuts` groups hold several batches and take a cut each."""
+    _load(vt, vd, pt, pd)
+    mlt.tune_ordinal(0)  # one launch a walk whatever the group's size
+    try:
+        one = _launches(batch, batch)
+        # two batches as large as these are two groups whatever the models
+        per = _launches(1 << 21, 1 << 20) - _launches(1 << 20, 1 << 20)
+        assert _launches(batches * batch, batch) - one == (groups - 1) * per + cuts
+    finally:
+        mlt.tune_ordinal(1)
