@@ -376,6 +376,15 @@ int mlt_selftest_wait_timeout(void *stream, int64_t limit_ns);
  * No fault, trap or endless loop is involved.  Host-only bookkeeping. */
 int mlt_selftest_walk_timeout(int cta, int64_t limit_ns);
 
+/* The same inside the ordinal form (mlt_tune_ordinal): arms a one-shot so that
+ * CTA 0 of the next kernel that writes candidates' ordinals (model V's, or P's
+ * where V is walked in fp32 form) waits limit_ns (1e6 .. 2e9 ns) on a barrier
+ * that nothing completes.  Its share of the ordinals is then not written, so
+ * the walks of that call take no candidate as valid, or where P's ordinals
+ * failed give every valid candidate the score -inf; mlt_sync_status reports
+ * MLT_ETIMEOUT and the next call is unaffected.  Host-only bookkeeping. */
+int mlt_selftest_ordinal_timeout(int64_t limit_ns);
+
 /* Test support: writes `value` into the four counters (survivor count,
  * collected keys, two CTA tickets) of the selection state that the
  * allocating entry points (static_scratch = 0) or mlt_screen_noalloc

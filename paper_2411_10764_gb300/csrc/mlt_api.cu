@@ -196,6 +196,8 @@ long long g_jit_min_n = kDecodeJitMinN;
 long long g_jit_calls = 0;
 int g_stall_cta = -1;
 unsigned long long g_stall_ns = 0;
+// the same for the next kernel that writes ordinals (mlt_selftest_ordinal_timeout)
+unsigned long long g_ord_stall_ns = 0;
 
 size_t align16(size_t v) { return (v + 15) & ~static_cast<size_t>(15); }
 
@@ -666,6 +668,9 @@ cudaError_t launch_pass(const DeviceModel& m, TraverseArgs a, const Pass& p, con
   o.out = static_cast<uint32_t*>(g_scr.ord.p);
   o.nan_flags = static_cast<unsigned char*>(g_scr.ord.p) + ord_bytes(n);
   o.err = a.err;
+  o.failed = &a.state_rw->ord_failed;
+  o.stall_ns = g_ord_stall_ns;
+  g_ord_stall_ns = 0;
   cudaError_t e = launch_ordinals(m.ord, o, n, sm_count(), st);
   if (e != cudaSuccess) return e;
   a.table = m.ord.table;
@@ -1731,6 +1736,14 @@ int mlt_selftest_walk_timeout(int cta, int64_t limit_ns) {
   std::lock_guard<std::mutex> lk(g_mu);
   g_stall_cta = cta;
   g_stall_ns = static_cast<unsigned long long>(limit_ns);
+  return MLT_OK;
+}
+
+int mlt_selftest_ordinal_timeout(int64_t limit_ns) {
+  if (limit_ns < 1000000LL || limit_ns > static_cast<int64_t>(kWaitLimitNs))
+    return fail(MLT_EINVAL, "limit_ns must lie in [1e6, %llu]", kWaitLimitNs);
+  std::lock_guard<std::mutex> lk(g_mu);
+  g_ord_stall_ns = static_cast<unsigned long long>(limit_ns);
   return MLT_OK;
 }
 

@@ -228,6 +228,7 @@ struct SelectState {
   unsigned int ticket;     // CTAs of the top-k kernel that finished
   unsigned int v_ticket;   // CTAs of the V pass that finished
   unsigned int hist[kTopBins];  // 16-byte aligned
+  unsigned int ord_failed;      // a CTA gave up writing ordinals: none of the call's are walked
 };
 
 // Batched accumulation (mlt_screen_until): bookkeeping carried on the device

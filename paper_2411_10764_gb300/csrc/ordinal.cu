@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
   constexpr int kRows = VEC ? S / 2 : 1;  // blocks of 32 rows a warp takes together
   static_assert(VEC || S == 8, "unaligned rows: 8 slots of 4 rows");
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ __align__(8) unsigned long long bar;
+  __shared__ __align__(8) unsigned long long bar, never;  // never completed (self-test)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int gi = 0;
   for (int hi = a.n_groups; gi + 1 < hi;) {
@@ -138,6 +138,7 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
   const OrdGroup g = a.groups[gi];
   if (tid == 0) {
     mbar_init(smem_u32(&bar), 1);
+    mbar_init(smem_u32(&never), 1);
     fence_mbar_init();
   }
   __syncthreads();
@@ -157,10 +158,18 @@ __global__ void __launch_bounds__(kOrdThreads, 1) k_ordinals(const __grid_consta
   const uint32_t step = slabs * (blockDim.x >> 5);
   const uint32_t sm = smem_u32(smem);
   // every warp waits for the copy, also one without rows: it must land before
-  // the CTA's shared memory is released
-  if (g.bytes > 0 && !__all_sync(0xFFFFFFFFu, mbar_wait_bounded(smem_u32(&bar), 0u))) {
-    mbar_wait_bounded(smem_u32(&bar), 0u);
-    atomicOr(a.err, kErrWaitTimeout);
+  // the CTA's shared memory is released.  A CTA that gives up leaves the buffer's
+  // earlier contents in its share, so it marks the call's ordinals as failed: the
+  // walk then takes no candidate as valid.
+  const bool stall = a.stall_ns > 0 && blockIdx.x == 0;
+  const bool here = stall ? mbar_wait_bounded_ns(smem_u32(&never), 0u, a.stall_ns)
+                          : g.bytes == 0 || mbar_wait_bounded(smem_u32(&bar), 0u);
+  if (!__all_sync(0xFFFFFFFFu, here)) {
+    if (g.bytes > 0) mbar_wait_bounded(smem_u32(&bar), 0u);
+    if (lane == 0) {
+      atomicOr(a.failed, 1u);
+      atomicOr(a.err, kErrWaitTimeout);
+    }
     return;
   }
   for (uint32_t it = warp * slabs + slab; it < items; it += step) {
@@ -476,6 +485,7 @@ template <int D, int U, int DEEP = 0>
 __global__ void __launch_bounds__(kOrdMaxCta, 1) k_walk_ord(const __grid_constant__ TraverseArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int last_issued[4];  // latest chunk copied into each buffer
+  __shared__ unsigned ord_failed;
   constexpr bool kGroups = U > 0;
   const int Q = kGroups ? a.groups : 1, TC = blockDim.x / Q, tid = threadIdx.x, lane = tid & 31;
   const int cols = TC >> 5, q = (tid >> 5) / cols, col = (tid >> 5) - q * cols;  // warp-uniform
@@ -526,6 +536,9 @@ __global__ void __launch_bounds__(kOrdMaxCta, 1) k_walk_ord(const __grid_constan
     const uint32_t tile_bytes = static_cast<uint32_t>(live_cols) * static_cast<uint32_t>(F2) * 128u;
     mbar_expect_tx(smem_u32(&bars[4]), tile_bytes);
     bulk_copy_g2s(smem_u32(smem), a.ord + (tile0 >> 5) * F2 * 32, tile_bytes, smem_u32(&bars[4]));
+    // in shared memory, not a register: needed at the end only, read while the
+    // tile is on its way (a register held over the walk cost the deep kernel 5 %)
+    ord_failed = *reinterpret_cast<const volatile unsigned*>(&a.state->ord_failed);
   }
   if (a.p_pass && tid < rows_here) rowidx[tid] = a.rows[tile0 + tid];
   bool nan = false;
@@ -603,7 +616,7 @@ __global__ void __launch_bounds__(kOrdMaxCta, 1) k_walk_ord(const __grid_constan
       }
     }
   }
-  if (__syncthreads_or(timed_out)) {
+  if (__syncthreads_or(timed_out || (tid == 0 && ord_failed != 0u))) {
     if (tid == 0) {
       // every copy in flight lands before the CTA's shared memory is released
       // (bounded waits), then the timeout is reported

@@ -74,6 +74,8 @@ struct OrdArgs {
   uint32_t* out;           // [blocks][ceil(F/2)][32]
   unsigned char* nan_flags;  // [blocks][ceil(F/8)]: a missing value among 8 features
   unsigned* err;
+  unsigned* failed;        // SelectState::ord_failed
+  unsigned long long stall_ns;  // self-test: CTA 0 waits this long on a barrier nothing completes (0: no)
   int n_groups;
   unsigned short first_cta[kOrdMaxGroups + 1];  // CTAs [first_cta[g], first_cta[g + 1]) take group g
 };

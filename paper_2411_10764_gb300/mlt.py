@@ -61,6 +61,7 @@ def lib(build_if_missing: bool = True):
             "mlt_screen_host_batches": [P, i64, P, i64, f32, i32, P, P, P],
             "mlt_selftest_wait_timeout": [P, i64],
             "mlt_selftest_walk_timeout": [i32, i64],
+            "mlt_selftest_ordinal_timeout": [i64],
             "mlt_selftest_poison_state": [i32, C.c_uint32],
             "mlt_free_ensemble": [i32],
             "mlt_validity_cut": [f32, P],
@@ -379,6 +380,12 @@ def selftest_walk_timeout(cta: int, limit_ns: int) -> None:
     table) makes CTA `cta` give up waiting for its first tree chunk after
     limit_ns; the next sync_status raises MltError with MLT_ETIMEOUT."""
     _check(lib().mlt_selftest_walk_timeout(int(cta), int(limit_ns)))
+
+
+def selftest_ordinal_timeout(limit_ns: int) -> None:
+    """Arm a one-shot: CTA 0 of the next kernel that writes ordinals waits
+    limit_ns on a barrier nothing completes."""
+    _check(lib().mlt_selftest_ordinal_timeout(int(limit_ns)))
 
 
 def selftest_poison_state(value: int, static_scratch: bool = False) -> None:

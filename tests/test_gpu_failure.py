@@ -59,3 +59,42 @@ def test_poisoned_selection_state_does_not_reach_the_next_call(value):
     mlt.load_workload_models(w)
     mlt.selftest_poison_state(value)
     assert_parity(gpu_screen(w), o)
+
+
+@pytest.mark.parametrize("cid,n", [(2, 20000), (3, 9001), (5, 4097)])
+@pytest.mark.parametrize("which", ["v", "p"])
+def test_ordinal_timeout_leaves_no_stale_ordinals(cid, n, which):
+    """A CTA that writes ordinals gives up: its share of the buffer still holds
+    an earlier call's.  No result may come from them (V: no candidate is valid;
+    P: no valid candidate has a score), and the next call is exact."""
+    import numpy as np
+    import torch
+
+    w = W.make_workload(cid, seed=4, n=n)
+    mlt.load_workload_models(w)
+    x = torch.from_numpy(w.feats).cuda()
+    mlt.tune_ordinal(2)
+    if which == "p":  # a fixed shape keeps V in fp32 form
+        mlt.tune_walk(mlt.MLT_MODEL_V, candidates=64)
+    try:
+        mlt.screen(torch.flip(x, [0]).contiguous(), w.thr, w.k)  # other ordinals in the buffer
+        mlt.sync_status()
+        mlt.selftest_ordinal_timeout(20_000_000)  # 20 ms
+        pv, pf, tk = mlt.screen(x, w.thr, w.k)
+        with pytest.raises(mlt.MltError) as e:
+            mlt.sync_status()
+        assert e.value.code == -5  # MLT_ETIMEOUT
+        assert np.all(np.isneginf(pf.cpu().numpy()))
+        opv, opf, otk, os_ = oracle_screen(w)
+        if which == "v":
+            assert np.all(pv.cpu().numpy() == 0.0) and np.all(tk.cpu().numpy() == -1)
+            assert mlt.last_survivor_count() == 0
+        else:
+            assert mlt.last_survivor_count() == os_
+        pv, pf, tk = mlt.screen(x, w.thr, w.k)
+        mlt.sync_status()
+        assert_parity((pv.cpu().numpy(), pf.cpu().numpy(), tk.cpu().numpy(), mlt.last_survivor_count()),
+                      (opv, opf, otk, os_))
+    finally:
+        mlt.tune_ordinal(1)
+        mlt.tune_walk(mlt.MLT_MODEL_V)
