@@ -319,8 +319,9 @@ int mlt_decode_knobs(void *stream, const int32_t *radices, const float *option_v
  * are written once into a library-owned device buffer (n x F x 4 bytes, grown
  * as needed, given back when the feature count changes or a V or P model is
  * freed) and screened.  Where the buffer cannot be had (no memory, or it
- * would have to grow during a stream capture) the features are built on chip
- * inside the screening kernels instead (same results).
+ * would have to grow during a stream capture) or would hold more than 8 GB
+ * without the compiled program below, the features are built on chip inside
+ * the screening kernels instead (same results).
  * The program length must equal the current F.  out_topk holds candidate
  * indices (first_index + position).  Batches of at least the
  * mlt_tune_decode_jit threshold build their rows with the compiled feature

@@ -254,8 +254,10 @@ void free_model(Model& m) {
   m = Model();
 }
 
-// The ordinal buffer holds at most this; a larger batch walks the fp32 rows.
-constexpr size_t kOrdMaxBytes = 8ull << 30;
+// The ordinal buffer holds at most this, and so do rows that the library's own
+// decoder writes; a larger batch walks the fp32 rows, or decodes inside the
+// walks.  (The compiled program's rows are the batch's size.)
+constexpr size_t kBufferMaxBytes = 8ull << 30;
 
 void release_buffers() {
   g_scr.feats.release();
@@ -652,7 +654,7 @@ void plan_passes(const DeviceModel& V, const DeviceModel& P, long long n, bool s
     p[i]->ord = p[i]->ord && p[i]->shape.threads > 0;
     if (p[i]->ord) bytes = std::max(bytes, ord_bytes(n) + ord_flag_bytes(n));
   }
-  if (bytes > 0 && (bytes > kOrdMaxBytes || !g_scr.ord.ensure(bytes, st))) pv->ord = pp->ord = false;
+  if (bytes > 0 && (bytes > kBufferMaxBytes || !g_scr.ord.ensure(bytes, st))) pv->ord = pp->ord = false;
   for (int i = 0; i < 2; ++i)
     if (!p[i]->ord) p[i]->shape = plan_walk(*m[i], n_eff[i], g_shape[i], i == 0);
 }
@@ -716,12 +718,14 @@ int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec
   // a decoded batch: its rows are written once, by the compiled feature
   // program where the batch is large, and the walks read them like stored
   // features (the same bits as decoding inside the walks, which remains where
-  // the buffer cannot be had); top-k positions stay candidate indices
+  // the buffer cannot be had or would be too large); top-k positions stay candidate indices
   const long long topk_base = dec ? dec->first_index : 0;
   const DecodeParams* rows_dec = nullptr;
   JitDecoder jd{};
-  if (dec != nullptr && n > 0 && g_scr.feats.ensure(static_cast<size_t>(n) * g_F * sizeof(float), st)) {
-    if (g_jit_min_n > 0 && n >= g_jit_min_n) jd = jit_decoder_for(*dec, dev);
+  if (dec != nullptr && g_jit_min_n > 0 && n >= g_jit_min_n) jd = jit_decoder_for(*dec, dev);
+  const size_t row_bytes = static_cast<size_t>(n) * g_F * sizeof(float);
+  if (dec != nullptr && n > 0 && (jd.fn != nullptr || row_bytes <= kBufferMaxBytes) &&
+      g_scr.feats.ensure(row_bytes, st)) {
     rows_dec = dec;
     feats = static_cast<const float*>(g_scr.feats.p);
     dec = nullptr;
@@ -928,7 +932,8 @@ int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, lo
     per = std::max(per, g);
   }
   // decoded batches: each group's rows are written first, as in run_screen_with
-  const bool rows = dec0 != nullptr && per > 0 && g_scr.feats.ensure(static_cast<size_t>(per) * g_F * sizeof(float), st);
+  const size_t row_bytes = static_cast<size_t>(per) * g_F * sizeof(float);
+  const bool rows = dec0 != nullptr && row_bytes <= kBufferMaxBytes && g_scr.feats.ensure(row_bytes, st);
   Pass pv, pp;  // of the largest group: the buffers it needs, and that a shape exists
   plan_passes(V, P, per, dec0 == nullptr || rows, st, &pv, &pp);
   if (pv.shape.threads == 0 || pp.shape.threads == 0)

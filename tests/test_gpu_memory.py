@@ -1,5 +1,6 @@
-"""The row and ordinal buffers of a device that is short of memory: a buffer that
-cannot be had costs a call its faster form, not the time of asking for it."""
+"""The row and ordinal buffers: on a device that is short of memory one that cannot
+be had costs a call its faster form, not the time of asking for it; and rows
+stay within their bound."""
 import time
 
 import numpy as np
@@ -64,3 +65,45 @@ def test_a_full_device_does_not_slow_every_call():
         torch.cuda.empty_cache()
     assert all(torch.equal(a, b) for a, b in zip(want, outs))
     assert full < fp32 + 100.0, (full, fp32)  # asking takes 240
+
+
+def _held(call):
+    """Bytes of device memory that the call leaves taken."""
+    import torch
+
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    call()
+    torch.cuda.synchronize()
+    return before - torch.cuda.mem_get_info()[0]
+
+
+def test_interpreted_rows_are_bounded():
+    """16,777,216 rows of 144 features are 9.7 GB: they are decoded inside the
+    walks instead, with the results of two halves, whose rows fit."""
+    import torch
+
+    F, n, k = 144, 1 << 24, 64
+    d = W.conv2d_decoder(3, F)
+    cfg = W.ScreenConfig(4, "memory", n, F, 6, 5, 6, 5, 0.5, k, None, decoded=True)
+    th = W._RangeThresholds(d.ranges)
+    v, p = W.make_ensemble(cfg, "V", th, 3), W.make_ensemble(cfg, "P", th, 3)
+    mlt.set_num_features(F)
+    mlt.load_ensemble(mlt.MLT_MODEL_V, v.nodes, v.n_trees, v.depth)
+    mlt.load_ensemble(mlt.MLT_MODEL_P, p.nodes, p.n_trees, p.depth)
+    space = (d.radices, d.option_values, d.program)
+    whole = torch.empty(n, device="cuda"), torch.empty(n, device="cuda"), torch.empty(k, dtype=torch.int64, device="cuda")
+    mlt.tune_decode_jit(0)
+    try:
+        held = _held(lambda: mlt.screen_decoded(*space, 0, n, 0.5, k, out_pvalid=whole[0], out_perf=whole[1],
+                                                out_topk=whole[2]))
+        assert held < 2 << 30, held
+        held = _held(lambda: mlt.screen_until_decoded(*space, 0, n, n, 1, 0.5, k, with_outputs=False))
+        assert held < 1 << 30, held
+        for at in (0, n // 2):
+            pv, pf, _ = mlt.screen_decoded(*space, at, n // 2, 0.5, k)
+            assert torch.equal(pv, whole[0][at:at + n // 2]) and torch.equal(pf, whole[1][at:at + n // 2])
+        mlt.sync_status()
+    finally:
+        mlt.tune_decode_jit(1 << 20)
+        mlt.set_num_features(1)  # gives the buffers back
