@@ -478,9 +478,10 @@ int mlt_tune_fused_small(int max_n);
  *   mode  1 (default): where the library expects it to be faster; 2: wherever
  *         the model has the form; 0: never
  * Needs a library-owned device buffer of 2 bytes per feature and candidate
- * (at most 8 GB, grown as needed, given back like the decoded rows'); where it
- * cannot be had, and in mlt_screen_noalloc, the fp32 form is walked.
- * Host-only. */
+ * (at most 8 GB, grown as needed, given back like the decoded rows', and by
+ * mode 0 unless a captured graph refers to it); where it cannot be had, and in
+ * mlt_screen_noalloc, the fp32 form is walked.  Mode 0 may wait for the device
+ * to give the buffer back. */
 int mlt_tune_ordinal(int mode);
 
 /* Tuning: the table format of models V and P deeper than 10 levels, for

@@ -138,6 +138,8 @@ struct GrowBuf {
     captured = captured || capturing;
     return true;
   }
+  // no captured work refers to it
+  bool idle() const { return !captured && aside.empty(); }
   void release() {
     failed = 0;
     pause = 0;
@@ -1318,6 +1320,7 @@ int mlt_tune_ordinal(int mode) {
   if (mode < 0 || mode > 2) return fail(MLT_EINVAL, "mode must be 0, 1 or 2, got %d", mode);
   std::lock_guard<std::mutex> lk(g_mu);
   g_ord_mode = mode;
+  if (mode == 0 && g_scr.ord.idle()) g_scr.ord.release();
   return MLT_OK;
 }
 

@@ -1,6 +1,6 @@
 """The row and ordinal buffers: on a device that is short of memory one that cannot
-be had costs a call its faster form, not the time of asking for it; and rows
-stay within their bound."""
+be had costs a call its faster form, not the time of asking for it; they stay
+within their bound; and the ordinals' goes back when the form is turned off."""
 import time
 
 import numpy as np
@@ -107,3 +107,30 @@ def test_interpreted_rows_are_bounded():
     finally:
         mlt.tune_decode_jit(1 << 20)
         mlt.set_num_features(1)  # gives the buffers back
+
+
+def test_turning_the_form_off_gives_its_buffer_back():
+    import torch
+
+    F, n = 256, 1 << 20  # ordinals of 512 MiB
+    _load(F)
+    x = torch.rand((n, F), device="cuda")
+    mlt.tune_ordinal(2)
+    try:
+        mlt.screen(x, 0.5, 16)
+        assert _held(lambda: mlt.tune_ordinal(0)) <= -(500 << 20)
+        # a captured call's buffer stays
+        mlt.tune_ordinal(2)
+        outs = mlt.screen(x, 0.5, 16)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            mlt.screen(x, 0.5, 16, *outs)
+        assert _held(lambda: mlt.tune_ordinal(0)) == 0
+        want = [o.clone() for o in outs]
+        for o in outs:
+            o.zero_()
+        g.replay()
+        mlt.sync_status()
+        assert all(torch.equal(a, b) for a, b in zip(want, outs))
+    finally:
+        mlt.tune_ordinal(1)
