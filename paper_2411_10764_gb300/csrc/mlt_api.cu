@@ -14,8 +14,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "mlt.h"
@@ -476,9 +478,8 @@ int build_decoder(const int32_t* radices, const float* option_values, int n_knob
   return MLT_OK;
 }
 
-// Validate the heap-order ensemble and pack it for the device.
-int pack_ensemble(const mlt_node* nodes, int n_trees, int depth, int F, std::vector<unsigned char>& out,
-                  DeviceModel& dm) {
+// Refuse an ensemble that is no heap of finite splits and leaves.
+int validate_ensemble(const mlt_node* nodes, int n_trees, int depth, int F) {
   const int slots = (2 << depth) - 1;
   std::vector<unsigned char> reach(slots);
   std::vector<int> depth_of(slots);
@@ -507,7 +508,13 @@ int pack_ensemble(const mlt_node* nodes, int n_trees, int depth, int F, std::vec
     leaf_bound += maxabs;
   }
   if (leaf_bound >= 1e37L) return fail(MLT_EINVAL, "leaf magnitudes could overflow the fp32 sum");
+  return MLT_OK;
+}
 
+// Pack a validated ensemble for the device.
+int pack_ensemble(const mlt_node* nodes, int n_trees, int depth, std::vector<unsigned char>& out, DeviceModel& dm) {
+  const int slots = (2 << depth) - 1;
+  std::vector<unsigned char> reach(slots);
   dm.n_trees = n_trees;
   dm.depth = depth;
   if (depth <= kMaxFullDepth) {
@@ -1030,18 +1037,12 @@ int run_screen(cudaStream_t st, const float* feats, const DecodeParams* dec, lon
   return run_screen_with(st, feats, dec, n, thr, k, out_pvalid, out_perf, out_topk, g_scr.s, false);
 }
 
-// Split table (kTableSplit, deep models V and P): validate like
-// pack_ensemble, then store each tree's first H levels and its level-H exits
-// as a head block and everything below level H as breadth-first compact
-// records in one tail array (layout in mlt_internal.cuh).
-int pack_split(const mlt_node* nodes, int n_trees, int depth, int F, int H, std::vector<unsigned char>& out,
+// Split table (kTableSplit, deep models V and P) of a validated ensemble: each
+// tree's first H levels and its level-H exits as a head block and everything
+// below level H as breadth-first compact records in one tail array (layout in
+// mlt_internal.cuh).
+int pack_split(const mlt_node* nodes, int n_trees, int depth, int H, std::vector<unsigned char>& out,
                DeviceModel& dm) {
-  {
-    std::vector<unsigned char> scratch;
-    DeviceModel probe;
-    const int rc = pack_ensemble(nodes, n_trees, depth, F, scratch, probe);  // validation
-    if (rc != MLT_OK) return rc;
-  }
   const int slots = (2 << depth) - 1;
   const uint32_t hb = split_head_bytes(H);
   const int n_head = (1 << H) - 1;         // slots of levels 0 .. H-1
@@ -1163,16 +1164,10 @@ int pack_split(const mlt_node* nodes, int n_trees, int depth, int F, int H, std:
   return MLT_OK;
 }
 
-// Half table (kTableHalf): validate like pack_ensemble, then store the
-// complete heap with binary16 thresholds and leaves (round to nearest even).
-int pack_ensemble_half(const mlt_node* nodes, int n_trees, int depth, int F, std::vector<unsigned char>& out,
+// Half table (kTableHalf) of a validated ensemble: the complete heap with
+// binary16 thresholds and leaves (round to nearest even).
+int pack_ensemble_half(const mlt_node* nodes, int n_trees, int depth, std::vector<unsigned char>& out,
                        DeviceModel& dm) {
-  {
-    std::vector<unsigned char> scratch;
-    DeviceModel probe;
-    const int rc = pack_ensemble(nodes, n_trees, depth, F, scratch, probe);  // validation
-    if (rc != MLT_OK) return rc;
-  }
   const int slots = (2 << depth) - 1;
   const HalfLayout lay = half_layout(depth);
   const size_t tb = lay.bytes;
@@ -1227,19 +1222,52 @@ int pack_ensemble_half(const mlt_node* nodes, int n_trees, int depth, int F, std
   return MLT_OK;
 }
 
-// Upload a packed table into model slot `model_id` (lock held).
-// `base` bytes of it are the model; the rest is its ordinal form, left out
-// where the device has no room for both.
-int install_model(int model_id, const std::vector<unsigned char>& packed, size_t base, DeviceModel dm) {
+// Packs the ordinal form of a validated ensemble on a thread of its own, beside
+// the caller, who packs the table meanwhile; small ensembles (where the start of
+// a thread shows) when it is asked for, and so where there is no thread to be had.
+class OrdinalBeside {
+ public:
+  OrdinalBeside(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half)
+      : work_([=] { pack_ordinal(nodes, n_trees, depth, F, round_half, form, table); }) {
+    if (static_cast<size_t>(n_trees) * ((2u << depth) - 1) < 16384) return;
+    try {
+      thread_ = std::thread(work_);
+      started_ = true;
+    } catch (...) {
+    }
+  }
+  ~OrdinalBeside() {
+    if (thread_.joinable()) thread_.join();
+  }
+  void finish() {
+    if (started_)
+      thread_.join();
+    else
+      work_();
+  }
+  std::vector<unsigned char> form;
+  OrdTable table;
+
+ private:
+  std::function<void()> work_;
+  std::thread thread_;
+  bool started_ = false;
+};
+
+// Upload a packed table into model slot `model_id` (lock held), and its ordinal
+// form (may be empty) after it, left out where the device has no room for both.
+int install_model(int model_id, const std::vector<unsigned char>& packed, const std::vector<unsigned char>& ordinal,
+                  DeviceModel dm) {
   int dev = 0;
   int rc = current_device(&dev);
   if (rc != MLT_OK) return rc;
   unsigned char* d = nullptr;
-  size_t bytes = packed.size();
+  const size_t ord_at = (packed.size() + 127) & ~static_cast<size_t>(127);
+  size_t bytes = ordinal.empty() ? packed.size() : ord_at + ordinal.size();
   cudaError_t e = cudaMalloc(&d, bytes);
-  if (e != cudaSuccess && bytes > base) {
+  if (e != cudaSuccess && !ordinal.empty()) {
     cudaGetLastError();
-    bytes = base;
+    bytes = packed.size();
     dm.ord = OrdTable();
     e = cudaMalloc(&d, bytes);
   }
@@ -1247,7 +1275,9 @@ int install_model(int model_id, const std::vector<unsigned char>& packed, size_t
     cudaGetLastError();
     return fail(MLT_ENOMEM, "cannot allocate %zu bytes for the ensemble", bytes);
   }
-  e = cudaMemcpy(d, packed.data(), bytes, cudaMemcpyHostToDevice);
+  e = cudaMemcpy(d, packed.data(), packed.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && dm.ord.n_trees > 0)
+    e = cudaMemcpy(d + ord_at, ordinal.data(), ordinal.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(d);
     return cuda_fail(e, "ensemble upload");
@@ -1260,15 +1290,15 @@ int install_model(int model_id, const std::vector<unsigned char>& packed, size_t
   m.owned = d;
   m.dm = dm;
   m.dm.table = d;
-  m.dm.bytes = base;
   if (dm.kind == kTableSplit) m.dm.tail = d + dm.tail_off;
   OrdTable& o = m.dm.ord;
   if (o.n_trees > 0) {
-    o.table = d + o.off_table;
-    o.tail = reinterpret_cast<const uint4*>(d + o.off_tail);
-    o.image = d + o.off_image;
-    o.features = reinterpret_cast<const OrdFeature*>(d + o.off_features);
-    o.groups = reinterpret_cast<const OrdGroup*>(d + o.off_groups);
+    const unsigned char* at = d + ord_at;
+    o.table = at + o.off_table;
+    o.tail = reinterpret_cast<const uint4*>(at + o.off_tail);
+    o.image = at + o.off_image;
+    o.features = reinterpret_cast<const OrdFeature*>(at + o.off_features);
+    o.groups = reinterpret_cast<const OrdGroup*>(at + o.off_groups);
   }
   return MLT_OK;
 }
@@ -1300,13 +1330,22 @@ int mlt_load_ensemble(int model_id, const mlt_node* nodes, int n_trees, int dept
   // models V and P deeper than a full table: split tables (model A keeps
   // the compact table its rerank walks)
   const bool split = depth > kMaxFullDepth && model_id != MLT_MODEL_A && g_head_levels > 0;
-  int rc = split ? pack_split(nodes, n_trees, depth, g_F, g_head_levels, packed, dm)
-                 : pack_ensemble(nodes, n_trees, depth, g_F, packed, dm);
+  int rc = validate_ensemble(nodes, n_trees, depth, g_F);
   if (rc != MLT_OK) return rc;
-  const size_t base = packed.size();
-  if ((dm.kind == kTableFull || dm.kind == kTableSplit) && model_id != MLT_MODEL_A)
-    pack_ordinal(nodes, n_trees, depth, g_F, false, packed, dm.ord);
-  return install_model(model_id, packed, base, dm);
+  auto pack = [&] {
+    return split ? pack_split(nodes, n_trees, depth, g_head_levels, packed, dm)
+                 : pack_ensemble(nodes, n_trees, depth, packed, dm);
+  };
+  if (model_id == MLT_MODEL_A || (depth > kMaxFullDepth && !split)) {  // no ordinal form
+    rc = pack();
+    return rc != MLT_OK ? rc : install_model(model_id, packed, {}, dm);
+  }
+  OrdinalBeside ord(nodes, n_trees, depth, g_F, false);
+  rc = pack();
+  if (rc != MLT_OK) return rc;
+  ord.finish();
+  dm.ord = ord.table;
+  return install_model(model_id, packed, ord.form, dm);
 }
 
 int mlt_tune_decode_jit(int64_t min_n) {
@@ -1361,11 +1400,14 @@ int mlt_load_ensemble_f16(int model_id, const mlt_node* nodes, int n_trees, int 
   if (g_F > static_cast<int>(kHalfFeatureMask) + 1) return fail(MLT_EINVAL, "half tables need F <= 1024");
   std::vector<unsigned char> packed;
   DeviceModel dm;
-  int rc = pack_ensemble_half(nodes, n_trees, depth, g_F, packed, dm);
+  int rc = validate_ensemble(nodes, n_trees, depth, g_F);
   if (rc != MLT_OK) return rc;
-  const size_t base = packed.size();
-  pack_ordinal(nodes, n_trees, depth, g_F, true, packed, dm.ord);
-  return install_model(model_id, packed, base, dm);
+  OrdinalBeside ord(nodes, n_trees, depth, g_F, true);
+  rc = pack_ensemble_half(nodes, n_trees, depth, packed, dm);
+  if (rc != MLT_OK) return rc;
+  ord.finish();
+  dm.ord = ord.table;
+  return install_model(model_id, packed, ord.form, dm);
 }
 
 int mlt_free_ensemble(int model_id) {

@@ -174,7 +174,7 @@ struct OrdTable {
   const uint4* tail = nullptr;  // deep models: blocks below the heads
   float visits = 0;  // node tests a candidate is expected to meet
   int rounds = 0;    // deep models: most blocks on a path (0: a full table)
-  size_t off_tail = 0, off_table = 0, off_image = 0, off_features = 0, off_groups = 0;  // in the model's allocation
+  size_t off_tail = 0, off_table = 0, off_image = 0, off_features = 0, off_groups = 0;  // from its start
   int n_trees = 0;         // padded
   int n_groups = 0;
   uint32_t max_bytes = 0;  // of a group's image
@@ -184,7 +184,6 @@ struct OrdTable {
 
 struct DeviceModel {
   const unsigned char* table = nullptr;
-  size_t bytes = 0;
   int kind = kTableFull;
   int n_trees = 0;
   int depth = 0;

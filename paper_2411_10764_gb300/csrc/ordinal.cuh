@@ -80,9 +80,9 @@ struct OrdArgs {
   unsigned short first_cta[kOrdMaxGroups + 1];  // CTAs [first_cta[g], first_cta[g + 1]) take group g
 };
 
-// ordinal_pack.cu: appends the ordinal form of a validated ensemble to `out` and describes it in t (offsets into `out`).
-// round_half: thresholds, leaves and features rounded to binary16.  False
-// when a feature has too many distinct thresholds (or one of -inf).
+// ordinal_pack.cu: the ordinal form of a validated ensemble, described by t
+// (offsets into `out`; multiples of 128).  round_half: thresholds, leaves and
+// features rounded to binary16.  False (and `out` empty) when a feature has too many distinct thresholds (or one of -inf).
 bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
                   std::vector<unsigned char>& out, OrdTable& t);
 // ordinal.cu

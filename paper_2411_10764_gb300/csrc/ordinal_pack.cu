@@ -1,10 +1,14 @@
-// Builds the ordinal form of a full-table model on the host (layout:
-// ordinal.cuh).  Host code only.
+// Builds the ordinal form of a model on the host (layout: ordinal.cuh).  Host
+// code only.  Every load of a V or P model pays for it: 600 trees of depth 10
+// over 96 features take 3.3 ms on 8 threads, 2,000 of depth 12 over 256 features
+// 29 ms (aarch64).
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <limits>
+#include <memory>
 #include <thread>
 #include <vector>
 
@@ -45,72 +49,158 @@ uint32_t bits_of(float v) {
 struct Buckets {
   float lo = 0.0f, add = 0.0f;
   uint32_t base = 0, shift = 0, count = 1, most = 0;
-  uint32_t at(float t) const { return (bits_of(std::fmax(t, lo) + add) - base) >> shift; }
+  uint32_t at(float t) const { return (bits_of((t > lo ? t : lo) + add) - base) >> shift; }
 };
-void fill(Buckets* b, const std::vector<float>& t) {
-  b->count = b->at(t.back()) + 1;
-  b->most = 0;
-  uint32_t run = 0, last = 0xFFFFFFFFu;
-  for (float v : t) {
-    const uint32_t at = b->at(v);
-    run = at == last ? run + 1 : 1;
-    last = at;
-    b->most = std::max(b->most, run);
-  }
-}
-// The most buckets allowed for offset c.
-Buckets buckets_for(const std::vector<float>& t, float c) {
-  Buckets b;
-  b.lo = t.front();
-  b.add = c - b.lo;
-  b.base = bits_of(b.lo + b.add);
-  while (b.at(t.back()) >= static_cast<uint32_t>(kOrdMaxBuckets)) ++b.shift;
-  fill(&b, t);
-  return b;
-}
 // Steps of a search among m thresholds.
 uint32_t steps_for(uint32_t m) {
   uint32_t s = 0;
   while ((1u << s) <= m) ++s;
   return s;
 }
+// Thresholds of the fullest bucket, bucket ids (ascending) shifted right by
+// `shift`; looked no further once there are `enough`.
+uint32_t fullest(const std::vector<uint32_t>& ids, uint32_t shift, uint32_t enough) {
+  uint32_t most = 0, run = 0, last = 0xFFFFFFFFu;
+  for (uint32_t id : ids) {
+    const uint32_t at = id >> shift;
+    run = at == last ? run + 1 : 1;
+    last = at;
+    if (run > most && (most = run) >= enough) break;
+  }
+  return most;
+}
+// The lookup table of ascending thresholds t: over the offsets c, the most
+// buckets allowed that leave the fewest steps; then the fewest buckets that
+// leave as few.  `ids` is working memory.
+Buckets choose_buckets(const std::vector<float>& t, std::vector<uint32_t>& ids) {
+  const double range = std::min(3.0e38, std::max(1e-30, static_cast<double>(t.back()) - t.front()));
+  const size_t m = t.size();
+  ids.resize(m);
+  Buckets best;
+  for (int q = 0; q < 26; q += 2) {
+    const float c = std::max(1e-30f, static_cast<float>(std::ldexp(range, 1 - q)));
+    Buckets b;
+    b.lo = t.front();
+    b.add = c - b.lo;
+    b.base = bits_of(b.lo + b.add);
+    while (b.at(t.back()) >= static_cast<uint32_t>(kOrdMaxBuckets)) ++b.shift;
+    for (size_t i = 0; i < m; ++i) ids[i] = b.at(t[i]);
+    // fewer steps than the best offset's: fewer than half of 2^steps thresholds
+    const uint32_t enough = q == 0 ? 0xFFFFFFFFu : (1u << steps_for(best.most)) / 2;
+    b.most = fullest(ids, 0, enough);
+    if (q == 0 || b.most < enough) best = b;
+  }
+  best.count = best.at(t.back()) + 1;
+  for (size_t i = 0; i < m; ++i) ids[i] = best.at(t[i]);
+  uint32_t shift = 0;
+  const uint32_t enough = 1u << steps_for(best.most);
+  while ((ids[m - 1] >> shift) > 0 && fullest(ids, shift + 1, enough) < enough) ++shift;
+  best.shift += shift;
+  best.count = (ids[m - 1] >> shift) + 1;
+  return best;
+}
 
-// Threads for n items that hold `nodes` nodes in all. Below 4096 nodes a thread
-// the start of the threads shows: a V and a P model of 50 and 100 trees of depth 6 loaded
-// in 1.3 ms with eight, 0.8 ms with this rule (aarch64 host, 16 cores).
+// Ascending order of the high words (a radix sort by 11 bits at a time; a
+// comparison sort of the 6,400 splits of a feature took six times as long).
+void sort_by_key(uint64_t* v, size_t n, std::vector<uint64_t>& other) {
+  if (n < 512) {
+    std::sort(v, v + n);
+    return;
+  }
+  other.resize(n);
+  uint64_t *from = v, *to = other.data();
+  uint32_t at[3][2048] = {};
+  for (size_t i = 0; i < n; ++i)
+    for (int d = 0; d < 3; ++d) ++at[d][(v[i] >> (32 + 11 * d)) & 2047u];
+  for (int d = 0; d < 3; ++d) {
+    uint32_t sum = 0;
+    for (uint32_t& a : at[d]) {
+      const uint32_t count = a;
+      a = sum;
+      sum += count;
+    }
+    for (size_t i = 0; i < n; ++i) to[at[d][(from[i] >> (32 + 11 * d)) & 2047u]++] = from[i];
+    std::swap(from, to);
+  }
+  std::memcpy(v, from, n * sizeof(uint64_t));  // three passes end in `other`
+}
+
+// Threads for n items that hold `nodes` nodes in all.  Below 4,096 nodes a
+// thread the start of the threads shows: a V and a P model of 50 and 100 trees of
+// depth 6 loaded in 1.3 ms with eight, 0.7 ms with this rule (aarch64 host, 16
+// cores).
 int worker_count(int n, size_t nodes) {
   const size_t most = std::min<size_t>(std::min(8u, std::thread::hardware_concurrency()), nodes / 4096);
   return std::max(1, std::min<int>(static_cast<int>(most), n / 8));
 }
-// body(i) for i in [0, n) on `workers` threads; false if one could not finish
-// (no exception leaves a thread, and a thread that cannot be had is done
-// without).
-template <typename F>
-bool spread(int n, int workers, F&& body) {
-  std::atomic<bool> ok{true};
-  auto share = [&](int w) {
+
+// Threads that share the steps of one packing.  run(n, body) calls body(i, w)
+// for i in [0, n), item i on worker i % workers(), and returns false if one could
+// not finish: no exception leaves a thread, and a thread that cannot be had is
+// done without.  Started once, for starting seven takes 0.2 ms and there are five
+// steps; between them the threads yield, later sleep.
+class Crew {
+ public:
+  explicit Crew(int workers) {
     try {
-      for (int f = w; f < n; f += workers) body(f);
+      threads_.reserve(workers);
+      while (static_cast<int>(threads_.size()) + 1 < workers)
+        threads_.emplace_back([this, w = static_cast<int>(threads_.size()) + 1] { serve(w); });
     } catch (...) {
-      ok = false;
     }
-  };
-  std::vector<std::thread> pool;
-  pool.reserve(workers);
-  int started = 1;
-  try {
-    for (; started < workers; ++started) pool.emplace_back(share, started);
-  } catch (...) {
+    workers_ = static_cast<int>(threads_.size()) + 1;
   }
-  share(0);
-  for (int w = started; w < workers; ++w) share(w);
-  for (std::thread& t : pool) t.join();
-  return ok;
-}
+  ~Crew() {
+    job_ = nullptr;
+    step_.fetch_add(1, std::memory_order_release);
+    for (std::thread& t : threads_) t.join();
+  }
+  int workers() const { return workers_; }
+  template <typename F>
+  bool run(int n, F&& body) {
+    struct Job {
+      F& body;
+      int n, workers;
+      std::atomic<bool> ok{true};
+    } job{body, n, workers_};
+    arg_ = &job;
+    job_ = [](void* p, int w) {
+      Job& j = *static_cast<Job*>(p);
+      try {
+        for (int i = w; i < j.n; i += j.workers) j.body(i, w);
+      } catch (...) {
+        j.ok = false;
+      }
+    };
+    busy_.store(static_cast<int>(threads_.size()), std::memory_order_relaxed);
+    step_.fetch_add(1, std::memory_order_release);
+    job_(arg_, 0);
+    while (busy_.load(std::memory_order_acquire) > 0) std::this_thread::yield();
+    return job.ok;
+  }
 
-}  // namespace
+ private:
+  void serve(int w) {
+    for (unsigned seen = 0;; ++seen) {
+      for (int tries = 0; step_.load(std::memory_order_acquire) == seen; ++tries) {
+        if (tries < 1000)
+          std::this_thread::yield();
+        else
+          std::this_thread::sleep_for(std::chrono::microseconds(20));
+      }
+      if (job_ == nullptr) return;
+      job_(arg_, w);
+      busy_.fetch_sub(1, std::memory_order_release);
+    }
+  }
+  std::vector<std::thread> threads_;
+  int workers_ = 1;
+  void (*job_)(void*, int) = nullptr;
+  void* arg_ = nullptr;
+  std::atomic<unsigned> step_{0};
+  std::atomic<int> busy_{0};
+};
 
-namespace {
 bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half, std::vector<unsigned char>& out,
           OrdTable& t) {
   const int slots = (2 << depth) - 1;
@@ -122,10 +212,25 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
   auto value = [&](const mlt_node& nd) {
     return round_half ? __half2float(__float2half_rn(nd.value)) : nd.value;
   };
-  std::vector<uint32_t> words(static_cast<size_t>(padded) * tree_words, 0u);
+  // the most that the lookup tables and what describes them can take (checked
+  // below), so that `out` is allocated once
+  const int F8 = (F + 7) / 8 * 8;
+  const size_t other_bytes = static_cast<size_t>(F8 / 8) * (kGroupMaxBytes + sizeof(OrdGroup)) + F8 * sizeof(OrdFeature) + 512;
+  const size_t tail_word = static_cast<size_t>(padded) * tree_words;  // a deep model's blocks follow the heads
+  if (tail_word >= 0x7FFFFFFFull) return false;
+  std::vector<uint32_t> heads;  // deep: until the tail's size is known
+  if (deep) {
+    heads.resize(tail_word, 0u);
+  } else {
+    out.reserve(tail_word * 4 + other_bytes);
+    out.resize(tail_word * 4, 0);
+  }
+  uint32_t* words = deep ? heads.data() : reinterpret_cast<uint32_t*>(out.data());
 
   // the tables with every word but the ordinals, and the split nodes as
-  // (feature, threshold's order key, word index); full tables on a few threads
+  // (feature, threshold's order key, word index), on a few threads that take
+  // consecutive trees; a deep model's blocks are numbered within a thread's share
+  // until all are counted
   struct Split {
     uint32_t feature;
     uint32_t key;
@@ -141,16 +246,19 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
     std::vector<unsigned char> reach;
     std::vector<float> inherit;
     std::vector<Root> queue;
+    std::vector<uint32_t> blocks;  // deep: the tail
+    size_t first_block = 0;        // of this share in the whole tail
+    std::vector<uint64_t> other;   // working memory of the features' step
+    std::vector<uint32_t> ids;
+    std::vector<size_t> at;        // where this share's next split of a feature goes
+    int first = 0, last = 0;       // its trees
     bool usable = true;
     double visits = 0.0;
   };
-  std::vector<uint32_t> blocks;  // deep: the tail
-  if (words.size() >= 0x7FFFFFFFull) return false;
   std::vector<float> reached(slots);  // share of the candidates that a random path brings to a slot
   for (int j = 0; j < slots; ++j) reached[j] = j == 0 ? 1.0f : 0.5f * reached[(j - 1) / 2];
   const int levels = deep ? kOrdHead : depth;  // of the complete heap
   const int inner = (1 << levels) - 1;
-  const size_t tail_word = words.size();  // the tail follows the heads
   auto put_split = [&](Worker& k, const mlt_node& nd, int j, size_t word, uint32_t* at) {
     const float v = value(nd);
     k.usable = k.usable && v != -INFINITY;  // every number is >= it: no ordinal stands for that
@@ -163,6 +271,7 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
     std::vector<unsigned char>& reach = k.reach;
     std::vector<float>& inherit = k.inherit;
     std::vector<Root>& queue = k.queue;
+    std::vector<uint32_t>& blocks = k.blocks;
     const mlt_node* nd = nodes + static_cast<size_t>(tr) * slots;
     const size_t base = static_cast<size_t>(tr) * tree_words;
     std::fill(reach.begin(), reach.end(), 0);
@@ -232,30 +341,56 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
     }
     k.usable = k.usable && blocks.size() / 8 < (1u << kOrdBlockBits);
   };
-  const int workers = deep ? 1 : worker_count(n_trees, total_nodes);  // the tail is one array
+  Crew crew(worker_count(n_trees, total_nodes));
+  const int workers = crew.workers();
   std::vector<Worker> made(workers);
-  const bool built = spread(workers, workers, [&](int w) {
+  const bool built = crew.run(workers, [&](int w, int) {
     Worker& k = made[w];
     k.per_feature.assign(F + 1, 0u);
     k.reach.resize(slots);
     k.inherit.resize(slots);
-    const int first = static_cast<int>(static_cast<long long>(n_trees) * w / workers);
-    const int last = static_cast<int>(static_cast<long long>(n_trees) * (w + 1) / workers);
-    if (!deep) k.splits.reserve(static_cast<size_t>(last - first) * inner);
-    for (int tr = first; tr < last && k.usable; ++tr) put_tree(k, tr);
+    k.first = static_cast<int>(static_cast<long long>(n_trees) * w / workers);
+    k.last = static_cast<int>(static_cast<long long>(n_trees) * (w + 1) / workers);
+    if (!deep) k.splits.reserve(static_cast<size_t>(k.last - k.first) * inner);
+    for (int tr = k.first; tr < k.last && k.usable; ++tr) put_tree(k, tr);
   });
   if (!built) return false;
   double visits = 0.0;
-  for (const Worker& k : made) {
+  size_t n_blocks = 0;
+  for (Worker& k : made) {
     if (!k.usable) return false;
     visits += k.visits;
+    k.first_block = n_blocks;
+    n_blocks += k.blocks.size() / 8;
   }
-  if (blocks.empty()) blocks.resize(8, 0u);  // finished walkers read block 0
+  if (n_blocks >= (1u << kOrdBlockBits) || tail_word + 8 * n_blocks >= 0x7FFFFFFFull) return false;
   if (deep)  // the padding trees' exits are leaves of +0
     for (int tr = n_trees; tr < padded; ++tr)
       for (uint32_t e = 0; e < (1u << levels); ++e)
         words[static_cast<size_t>(tr) * tree_words + (1u << levels) + 2 * e + 1] = kOrdExitLeaf;
-  words.insert(words.end(), blocks.begin(), blocks.end());
+  size_t n_words = tail_word;
+  if (deep) {
+    n_words += 8 * std::max<size_t>(n_blocks, 1);  // finished walkers read block 0
+    out.reserve(n_words * 4 + other_bytes);
+    out.resize(n_words * 4, 0);
+    words = reinterpret_cast<uint32_t*>(out.data());
+    std::memcpy(words, heads.data(), tail_word * 4);
+    crew.run(workers, [&](int w, int) {  // no allocation in it: nothing to fail
+      Worker& k = made[w];
+      const uint32_t base = static_cast<uint32_t>(k.first_block), mask = (1u << kOrdBlockBits) - 1u;
+      for (int tr = k.first; tr < k.last; ++tr)
+        for (uint32_t e = 0; e < (1u << levels); ++e) {
+          uint32_t& exit = words[static_cast<size_t>(tr) * tree_words + (1u << levels) + 2 * e + 1];
+          if (exit != kOrdExitLeaf) exit += base;
+        }
+      for (size_t i = 0; i < k.blocks.size(); i += 8)
+        if (k.blocks[i] & mask) k.blocks[i] += base;  // a root's children come after it, never at 0
+      if (!k.blocks.empty())
+        std::memcpy(&words[tail_word + 8 * k.first_block], k.blocks.data(), k.blocks.size() * 4);
+      for (Split& s : k.splits)
+        if (s.word >= tail_word) s.word += 8 * base;
+    });
+  }
 
   // thresholds of every feature in order, and each node's place among them
   std::vector<size_t> start(F + 1, 0);
@@ -263,21 +398,29 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
     start[f + 1] = start[f];
     for (const Worker& k : made) start[f + 1] += k.per_feature[f];
   }
-  std::vector<uint64_t> sorted(start[F]);
+  const std::unique_ptr<uint64_t[]> sorted(new uint64_t[start[F]]);  // written before it is read
   {
     std::vector<size_t> at(start.begin(), start.end() - 1);
-    for (const Worker& k : made)
-      for (const Split& s : k.splits) sorted[at[s.feature]++] = (static_cast<uint64_t>(s.key) << 32) | s.word;
+    for (Worker& k : made) {
+      k.at = at;
+      for (int f = 0; f < F; ++f) at[f] += k.per_feature[f];
+    }
   }
+  crew.run(workers, [&](int w, int) {  // no allocation in it
+    Worker& k = made[w];
+    for (const Split& s : k.splits) sorted[k.at[s.feature]++] = (static_cast<uint64_t>(s.key) << 32) | s.word;
+  });
   std::vector<std::vector<float>> keys(F);  // distinct thresholds, ascending
   std::vector<Buckets> buckets(F);
   std::vector<unsigned char> fits(F, 1);
-  if (!spread(F, worker_count(F, total_nodes), [&](int f) {
-    auto b = sorted.begin() + start[f], e = sorted.begin() + start[f + 1];
-    std::sort(b, e);
+  if (!crew.run(F, [&](int f, int w) {
+    std::vector<uint64_t>& other = made[w].other;
+    std::vector<uint32_t>& ids = made[w].ids;
+    uint64_t *b = sorted.get() + start[f], *e = sorted.get() + start[f + 1];
+    sort_by_key(b, static_cast<size_t>(e - b), other);
     std::vector<float>& k = keys[f];
     uint32_t before = 0;
-    for (auto it = b; it != e; ++it) {
+    for (const uint64_t* it = b; it != e; ++it) {
       const uint32_t key = static_cast<uint32_t>(*it >> 32);
       if (k.empty() || before != key) k.push_back(order_value(key));
       before = key;
@@ -287,29 +430,12 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
       }
       words[static_cast<uint32_t>(*it)] |= static_cast<uint32_t>(k.size() - 1) << 16;
     }
-    if (k.empty()) return;
-    // the offset that leaves the fewest steps; then the fewest buckets that
-    // leave as few
-    const double range = std::min(3.0e38, std::max(1e-30, static_cast<double>(k.back()) - k.front()));
-    Buckets best;
-    for (int q = 0; q < 26; q += 2) {
-      const Buckets b2 = buckets_for(k, std::max(1e-30f, static_cast<float>(std::ldexp(range, 1 - q))));
-      if (q == 0 || steps_for(b2.most) < steps_for(best.most)) best = b2;
-    }
-    while (best.count > 1) {
-      Buckets less = best;
-      ++less.shift;
-      fill(&less, k);
-      if (steps_for(less.most) > steps_for(best.most)) break;
-      best = less;
-    }
-    buckets[f] = best;
+    if (!k.empty()) buckets[f] = choose_buckets(k, ids);
       }))
     return false;
   if (std::find(fits.begin(), fits.end(), 0) != fits.end()) return false;
   // the table is padded to a multiple of 8 features; one without thresholds
   // has a bucket of its own and nothing but padding (ordinal 0)
-  const int F8 = (F + 7) / 8 * 8;
   keys.resize(F8);
   buckets.resize(F8);
   std::vector<OrdFeature> feat(F8, OrdFeature{});
@@ -351,13 +477,19 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
     total += eight;
     t.max_bytes = std::max(t.max_bytes, g.bytes);
   }
-  std::vector<unsigned char> image(total);
+  auto room = [&](size_t bytes) {  // in `out`, on a 128-byte boundary
+    const size_t at = (out.size() + 127) & ~static_cast<size_t>(127);
+    out.resize(at + bytes, 0);
+    return at;
+  };
+  t.off_image = room(total);
+  unsigned char* const image = out.data() + t.off_image;
   std::vector<uint32_t> image_at(F8);
   for (const OrdGroup& g : groups)
     for (uint32_t q = g.first; q < (g.first + g.count + 7) / 8 * 8; ++q) image_at[q] = g.off;
-  const bool filled = spread(F8, worker_count(F8, total_nodes), [&](int q) {
-    float* thr = reinterpret_cast<float*>(image.data() + image_at[q] + feat[q].thr);
-    uint16_t* lut = reinterpret_cast<uint16_t*>(image.data() + image_at[q] + feat[q].lut);
+  const bool filled = crew.run(F8, [&](int q, int) {
+    float* thr = reinterpret_cast<float*>(image + image_at[q] + feat[q].thr);
+    uint16_t* lut = reinterpret_cast<uint16_t*>(image + image_at[q] + feat[q].lut);
     for (uint32_t i = 0; i < (feat[q].lut - feat[q].thr) / 4; ++i)
       thr[i] = i < keys[q].size() ? keys[q][i] : std::numeric_limits<float>::quiet_NaN();
     uint32_t b = 0;  // lut[b] = thresholds in the buckets below b
@@ -370,16 +502,14 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
   if (!filled) return false;
 
   auto append = [&](const void* p, size_t bytes) {
-    const size_t at = (out.size() + 127) & ~static_cast<size_t>(127);
-    out.resize(at + bytes);
-    if (bytes) std::memcpy(out.data() + at, p, bytes);
+    const size_t at = room(bytes);
+    std::memcpy(out.data() + at, p, bytes);
     return at;
   };
-  t.off_table = append(words.data(), words.size() * 4);
+  t.off_table = 0;
   t.off_tail = t.off_table + tail_word * 4;
   t.visits = deep ? static_cast<float>(visits) : static_cast<float>(n_trees) * depth;  // a full walk has no early end
   t.rounds = deep ? (depth - kOrdHead + 2) / 3 : 0;
-  t.off_image = append(image.data(), image.size());
   t.off_features = append(feat.data(), feat.size() * sizeof(OrdFeature));
   t.off_groups = append(groups.data(), groups.size() * sizeof(OrdGroup));
   t.n_trees = padded;
@@ -391,14 +521,14 @@ bool pack(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
 
 bool pack_ordinal(const mlt_node* nodes, int n_trees, int depth, int F, bool round_half,
                   std::vector<unsigned char>& out, OrdTable& t) {
-  const size_t before = out.size();
   bool ok = false;
+  out.clear();
   try {
     ok = pack(nodes, n_trees, depth, F, round_half, out, t);
   } catch (const std::exception&) {  // no memory: the model does without
   }
   if (!ok) {
-    out.resize(before);
+    out.clear();
     t = OrdTable();
   }
   return ok;

@@ -231,3 +231,21 @@ def test_rule(F, n, trees, depth, launches):
     mlt.screen(torch.zeros((n, F), device="cuda"), 0.5, 10)
     mlt.sync_status()
     assert mlt.kernel_launches() - before == launches
+
+
+def test_the_form_is_packed_beside_the_table():
+    """Loading a V model costs little more than loading the same trees as model
+    A, which has no ordinal form."""
+    import time
+
+    cfg = W.ScreenConfig(4, "load", 64, 96, 300, 10, 300, 10, 0.5, 16, None)
+    e = W.make_ensemble(cfg, "V", W._RangeThresholds([(0.0, 1.0)] * 96), 3)
+    mlt.set_num_features(96)
+    best = {}
+    for _ in range(7):
+        for m in (mlt.MLT_MODEL_V, mlt.MLT_MODEL_A):
+            t = time.perf_counter()
+            mlt.load_ensemble(m, e.nodes, e.n_trees, e.depth)
+            best[m] = min(best.get(m, 1e9), time.perf_counter() - t)
+    mlt.free_ensemble(mlt.MLT_MODEL_A)
+    assert best[mlt.MLT_MODEL_V] < 2.0 * best[mlt.MLT_MODEL_A], best
