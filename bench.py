@@ -594,7 +594,10 @@ def measure_workload(ctx, w, args, headline: bool):
         "gpu_launches": int(launches), "clocks": clocks,
         "wall_ms_per_step_incl_flush": wall * 1e3 / steps,
     }
-    rec["walk_shapes"] = {"v": mlt.walk_shape(mlt.MLT_MODEL_V, w.n), "p": mlt.walk_shape(mlt.MLT_MODEL_P, w.n, True),
+    def walk_shape(model, p_pass):
+        return mlt.ordinal_shape(model, w.n, p_pass) or mlt.walk_shape(model, w.n, p_pass)
+
+    rec["walk_shapes"] = {"v": walk_shape(mlt.MLT_MODEL_V, False), "p": walk_shape(mlt.MLT_MODEL_P, True),
                           "note": "planned shape of each pass's walk (a step of one launch uses the single-launch "
                                   "kernel instead)" if launches == steps else "planned shape of each pass's walk"}
     if w.decoder is not None:

@@ -449,18 +449,24 @@ int mlt_phase_times(float *out_ms, int n_phases, int64_t *n_calls_out);
  * choice.  Results never depend on the shape.  Host-only. */
 int mlt_tune_walk(int model_id, int candidates, int splits, int group, int chunk_trees, int nbuf);
 
-/* Measurement: the launch shape the tree walk over model `model_id`'s
- * trees (V or P, loaded on the current device) would use for a screening
- * call of n candidates -- the V pass (p_pass = 0) walks n, the P pass
+/* Measurement: the launch shape the fp32 (or binary16) tree walk over model
+ * `model_id`'s trees (V or P, loaded on the current device) would use for a
+ * screening call of n candidates -- the V pass (p_pass = 0) walks n, the P pass
  * (p_pass != 0) is planned for about half of them -- including any shape
  * fixed by mlt_tune_walk.  out[7]: candidates per CTA, splits (tree groups
  * or lanes per candidate), trees in flight per thread, trees per chunk,
  * chunk buffers, CTAs resident per SM, table kind (0 full, 1 compact,
  * 2 half, 3 split).  Batches that mlt_screen screens in one launch
- * (mlt_tune_fused_small) do not use this shape, nor do large batches of
- * stored rows that are walked in ordinal form (integers in place of the
- * thresholds and features, same results).  Host-only. */
+ * (mlt_tune_fused_small) do not use this shape, nor do passes over rows that
+ * are walked in ordinal form (mlt_ordinal_shape).  Host-only. */
 int mlt_walk_shape(int model_id, int64_t n, int p_pass, int32_t *out);
+
+/* The same for the walk in ordinal form (mlt_tune_ordinal).  out[6]: candidates
+ * per CTA, tree groups, trees in flight per thread, trees per chunk, chunk
+ * buffers, CTAs resident per SM; all 0 where such a pass over rows would be
+ * walked in fp32 form (it also is where the ordinal buffer cannot be had).
+ * Host-only. */
+int mlt_ordinal_shape(int model_id, int64_t n, int p_pass, int32_t *out);
 
 /* Tuning: batches of up to max_n candidates (0 .. 8,192; the default is
  * 8,192) with stored features, whose V and P are full tables (depth <= 10)

@@ -644,9 +644,20 @@ size_t ord_flag_bytes(long long n) { return align16(static_cast<size_t>((n + 31)
 
 // One walk pass (V over all candidates or P over the survivors).
 struct Pass {
-  ScreenShape shape;
+  ScreenShape shape{};
   bool ord = false;  // the ordinal walk (shape is then plan_ord's)
 };
+
+// Whether a pass over n candidates, n_eff of which it is expected to walk, takes
+// the ordinal form, and its shape.
+Pass plan_ordinal_pass(const DeviceModel& m, const ShapeOverride& ov, long long n, long long n_eff) {
+  Pass p;
+  if (ord_wanted(m, ov, n, n_eff)) {
+    p.shape = plan_ordinal(m, n_eff);
+    p.ord = p.shape.threads > 0;
+  }
+  return p;
+}
 
 // Plans of both passes over n candidates.  stored: the rows are in memory and
 // the ordinal buffer may be allocated.
@@ -658,9 +669,7 @@ void plan_passes(const DeviceModel& V, const DeviceModel& P, long long n, bool s
   const long long n_eff[2] = {n, (n + 1) / 2};
   size_t bytes = 0;
   for (int i = 0; i < 2; ++i) {
-    p[i]->ord = stored && ord_wanted(*m[i], g_shape[i], n, n_eff[i]);
-    if (p[i]->ord) p[i]->shape = plan_ordinal(*m[i], n_eff[i]);
-    p[i]->ord = p[i]->ord && p[i]->shape.threads > 0;
+    *p[i] = stored ? plan_ordinal_pass(*m[i], g_shape[i], n, n_eff[i]) : Pass();
     if (p[i]->ord) bytes = std::max(bytes, ord_bytes(n) + ord_flag_bytes(n));
   }
   if (bytes > 0 && (bytes > kBufferMaxBytes || !g_scr.ord.ensure(bytes, st))) pv->ord = pp->ord = false;
@@ -1253,6 +1262,21 @@ class OrdinalBeside {
   std::thread thread_;
   bool started_ = false;
 };
+
+// Arguments of the shape queries (lock held).
+int check_shape_args(int model_id, int64_t n, const int32_t* out) {
+  if (model_id != MLT_MODEL_V && model_id != MLT_MODEL_P)
+    return fail(MLT_EINVAL, "model id must be V (0) or P (1), got %d", model_id);
+  if (out == nullptr) return fail(MLT_EINVAL, "out must be non-NULL");
+  if (n < 1) return fail(MLT_EINVAL, "n must be >= 1, got %lld", static_cast<long long>(n));
+  int dev = 0;
+  const int rc = current_device(&dev);
+  if (rc != MLT_OK) return rc;
+  const Model& m = g_models[model_id];
+  if (!m.loaded) return fail(MLT_ENOMODEL, "model %d is not loaded", model_id);
+  if (m.device != dev) return fail(MLT_EINVAL, "model %d lives on device %d, current device is %d", model_id, m.device, dev);
+  return MLT_OK;
+}
 
 // Upload a packed table into model slot `model_id` (lock held), and its ordinal
 // form (may be empty) after it, left out where the device has no room for both.
@@ -1930,17 +1954,10 @@ int mlt_walk_peak(void* stream, int model_id, const float* feats, int64_t n, int
 }
 
 int mlt_walk_shape(int model_id, int64_t n, int p_pass, int32_t* out) {
-  if (model_id != MLT_MODEL_V && model_id != MLT_MODEL_P)
-    return fail(MLT_EINVAL, "model id must be V (0) or P (1), got %d", model_id);
-  if (out == nullptr) return fail(MLT_EINVAL, "out must be non-NULL");
-  if (n < 1) return fail(MLT_EINVAL, "n must be >= 1, got %lld", static_cast<long long>(n));
   std::lock_guard<std::mutex> lk(g_mu);
-  int dev = 0;
-  int rc = current_device(&dev);
+  const int rc = check_shape_args(model_id, n, out);
   if (rc != MLT_OK) return rc;
   const Model& m = g_models[model_id];
-  if (!m.loaded) return fail(MLT_ENOMODEL, "model %d is not loaded", model_id);
-  if (m.device != dev) return fail(MLT_EINVAL, "model %d lives on device %d, current device is %d", model_id, m.device, dev);
   // the P pass is planned for about half the batch, as the screening does
   const ScreenShape sh = plan_for(m.dm, g_F, p_pass ? (n + 1) / 2 : n, g_shape[model_id], !p_pass);
   if (sh.threads == 0) return fail(MLT_EINVAL, "F=%d leaves no room for a shared-memory tile", g_F);
@@ -1951,6 +1968,19 @@ int mlt_walk_shape(int model_id, int64_t n, int p_pass, int32_t* out) {
   out[4] = sh.nbuf;
   out[5] = sh.resident;
   out[6] = m.dm.kind;
+  return MLT_OK;
+}
+
+int mlt_ordinal_shape(int model_id, int64_t n, int p_pass, int32_t* out) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  const int rc = check_shape_args(model_id, n, out);
+  if (rc != MLT_OK) return rc;
+  const Model& m = g_models[model_id];
+  const Pass p = plan_ordinal_pass(m.dm, g_shape[model_id], n, p_pass ? (n + 1) / 2 : n);
+  const bool ord = p.ord && ord_bytes(n) + ord_flag_bytes(n) <= kBufferMaxBytes;
+  const int32_t shape[6] = {p.shape.threads, p.shape.lanes, p.shape.group, p.shape.chunk_trees, p.shape.nbuf,
+                            p.shape.resident};
+  for (int i = 0; i < 6; ++i) out[i] = ord ? shape[i] : 0;
   return MLT_OK;
 }
 

@@ -75,6 +75,7 @@ def lib(build_if_missing: bool = True):
             "mlt_phase_times": [P, i32, P],
             "mlt_tune_walk": [i32, i32, i32, i32, i32, i32],
             "mlt_walk_shape": [i32, i64, i32, P],
+            "mlt_ordinal_shape": [i32, i64, i32, P],
             "mlt_tune_head_levels": [i32],
             "mlt_tune_fused_small": [i32],
             "mlt_tune_decode_jit": [i64],
@@ -449,13 +450,25 @@ def tune_fused_small(max_n: int) -> None:
 
 
 def walk_shape(model_id: int, n: int, p_pass: bool = False) -> dict:
-    """The launch shape the walk over model_id's trees would use for a
-    screening call of n candidates (P pass: planned for about n/2)."""
+    """The launch shape the fp32 (or binary16) walk over model_id's trees would
+    use for a screening call of n candidates (P pass: planned for about n/2)
+    that is not walked in ordinal form."""
     out = np.zeros(7, dtype=np.int32)
     _check(lib().mlt_walk_shape(int(model_id), int(n), 1 if p_pass else 0, out.ctypes.data))
     kinds = {0: "full", 1: "compact", 2: "half", 3: "split"}
     return {"candidates": int(out[0]), "splits": int(out[1]), "group": int(out[2]), "chunk_trees": int(out[3]),
             "nbuf": int(out[4]), "resident": int(out[5]), "table": kinds.get(int(out[6]), str(int(out[6])))}
+
+
+def ordinal_shape(model_id: int, n: int, p_pass: bool = False) -> dict | None:
+    """The same for the walk in ordinal form; None where such a pass would be
+    walked in fp32 form."""
+    out = np.zeros(6, dtype=np.int32)
+    _check(lib().mlt_ordinal_shape(int(model_id), int(n), 1 if p_pass else 0, out.ctypes.data))
+    if out[0] == 0:
+        return None
+    names = ("candidates", "splits", "group", "chunk_trees", "nbuf", "resident")
+    return dict({k: int(v) for k, v in zip(names, out)}, table="ordinal")
 
 
 def tune_decode_jit(min_n: int) -> None:

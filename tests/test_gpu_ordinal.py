@@ -249,3 +249,30 @@ def test_the_form_is_packed_beside_the_table():
             best[m] = min(best.get(m, 1e9), time.perf_counter() - t)
     mlt.free_ensemble(mlt.MLT_MODEL_A)
     assert best[mlt.MLT_MODEL_V] < 2.0 * best[mlt.MLT_MODEL_A], best
+
+
+@pytest.mark.parametrize("F,n,v,p", [(20, 13397, (500, 5), (500, 5)), (64, 65536, (200, 8), (20, 4)),
+                                     (47, 20011, (20, 5), (300, 14)), (30, 200, (900, 8), (900, 8))])
+def test_shape_query_agrees_with_the_launches(F, n, v, p):
+    """A pass has an ordinal shape exactly where it takes one more launch."""
+    import torch
+
+    mlt.tune_ordinal(1)
+    rng = np.random.default_rng(2)
+    mlt.set_num_features(F)
+    for m, (trees, depth) in ((mlt.MLT_MODEL_V, v), (mlt.MLT_MODEL_P, p)):
+        e = _trees(rng, F, trees, depth, _pool(rng, 500), split=0.75 if depth > 10 else 1.0)
+        mlt.load_ensemble(m, e.nodes, e.n_trees, e.depth)
+    mlt.tune_fused_small(0)
+    try:
+        before = mlt.kernel_launches()
+        mlt.screen(torch.zeros((n, F), device="cuda"), 0.5, 10)
+        mlt.sync_status()
+        launches = mlt.kernel_launches() - before
+    finally:
+        mlt.tune_fused_small(8192)
+    shapes = [mlt.ordinal_shape(mlt.MLT_MODEL_V, n), mlt.ordinal_shape(mlt.MLT_MODEL_P, n, True)]
+    assert launches == 4 + sum(s is not None for s in shapes), shapes
+    assert all(s is None or s["candidates"] * s["splits"] <= 1024 for s in shapes), shapes
+    mlt.tune_ordinal(0)
+    assert mlt.ordinal_shape(mlt.MLT_MODEL_P, n, True) is None
