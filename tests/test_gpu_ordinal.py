@@ -276,3 +276,28 @@ def test_shape_query_agrees_with_the_launches(F, n, v, p):
     assert all(s is None or s["candidates"] * s["splits"] <= 1024 for s in shapes), shapes
     mlt.tune_ordinal(0)
     assert mlt.ordinal_shape(mlt.MLT_MODEL_P, n, True) is None
+
+
+@pytest.mark.parametrize("n", [20001, 20033, 20127])
+@pytest.mark.parametrize("half", [False, True])
+@pytest.mark.parametrize("nan", [0.0, 0.05])
+def test_wide_items(n, half, nan):
+    """Aligned batches large enough for 128 rows an item (the others here take
+    64), ending inside one."""
+    import torch
+
+    F = 256
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert n // 128 * (F // 8) >= sms * 32  # the rule of launch_ordinals
+    rng = np.random.default_rng(n)
+    pool = _pool(rng, 150)
+    x = _rows(rng, n, F, pool, nan=nan)
+    _check(x, _trees(rng, F, 60, 7, pool), _trees(rng, F, 60, 7, pool), 0.5, 64, half=half)
+
+
+@pytest.mark.parametrize("F", [4, 12, 40])
+def test_half_tables_of_aligned_rows(F):
+    rng = np.random.default_rng(F)
+    pool = _pool(rng, 200)
+    x = _rows(rng, N0 + 61, F, pool, nan=0.05)
+    _check(x, _trees(rng, F, 30, 7, pool), _trees(rng, F, 30, 7, pool), 0.5, 64, half=True)
