@@ -5,7 +5,7 @@ One step = one screening call over one batch of a workload (ML^2Tuner's
 explorer step, Sec. 2; tree ensembles as in Table 3).  The headline line is
 the largest single-GPU workload, the exhaustive conv2d knob space: all
 16,777,216 candidate indices of 8 knobs x 8 options are decoded on the
-device into 96 fp32 features inside the walk kernels, V = 300 trees of depth
+device into rows of 96 fp32 features, once a step, V = 300 trees of depth
 10, P = 600 trees of depth 10, validity threshold 0.5, top-1,024.  The same
 line carries a `per_config` record for every workload (1 tiny, 2 gemm,
 3 sa-batch, 4 conv2d decoded, 5 skewed-nan).  Inputs sit in HBM before the
@@ -362,7 +362,7 @@ def screen_step(ctx, w):
         if d is None:
             mlt.screen(x, thr, k, pv, pf, tk, stream=ctx.stream)
         else:
-            # knob indices decoded and featurised inside the walk kernels
+            # knob indices decoded into rows of features, then screened
             mlt.screen_decoded(d.radices, d.option_values, d.program, w.first_index, n, thr, k,
                                out_pvalid=pv, out_perf=pf, out_topk=tk, stream=ctx.stream)
 

@@ -24,8 +24,9 @@
  *     mlt_sync_status() on that stream.
  *   - Library state (loaded ensembles, feature count, scratch buffers) is
  *     process-wide and guarded by a lock; scratch buffers are shared, so
- *     screening calls must be ordered on one stream (or the caller must
- *     synchronize between streams).
+ *     calls that screen, accumulate, propose, decode to screen or rerank must
+ *     be ordered on one stream (or the caller must synchronize between
+ *     streams).
  *   - Candidate counts are limited to n < 2^31; top-k to 1 <= k <= 16384.
  */
 #ifndef MLT_H
@@ -469,9 +470,8 @@ int mlt_walk_shape(int model_id, int64_t n, int p_pass, int32_t *out);
 int mlt_ordinal_shape(int model_id, int64_t n, int p_pass, int32_t *out);
 
 /* Tuning: batches of up to max_n candidates (0 .. 8,192; the default is
- * 8,192) with stored features, whose V and P are full tables (depth <= 10)
- * of the same depth small enough to share a CTA's shared memory, are
- * screened by one kernel launch (V walk, validity, P walk, keys and the
+ * 8,192), whose V and P are full tables (depth <= 10) of the same depth small
+ * enough to share a CTA's shared memory, are screened by one kernel launch (V walk, validity, P walk, keys and the
  * top-k selection by its last CTA) instead of four; 0 turns that path off.
  * Results never depend on the path.  Host-only. */
 int mlt_tune_fused_small(int max_n);

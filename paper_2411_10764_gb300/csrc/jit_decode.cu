@@ -2,14 +2,14 @@
 //
 // ML^2Tuner's explorer (Sec. 2) enumerates the knob space; each candidate's
 // features come from its knob values through the feature program (derived
-// features after Table 5).  Inside the walk kernels the program is data,
-// interpreted one operation at a time (about 67 instructions each).  For a
-// large batch the library instead turns the program into CUDA C -- one
+// features after Table 5).  To the library's own decoder (and inside the walk
+// kernels, where the row buffer cannot be had) the program is data, interpreted
+// one operation at a time (about 45 instructions each).  For a large batch the library instead turns the program into CUDA C -- one
 // straight-line statement per feature, the same rounded intrinsic per
 // operation as the interpreter, constants as exact bit patterns -- compiles
 // it once per program and device with NVRTC, and runs the result as a
 // decode kernel that writes the batch's rows to a device buffer; the
-// screening then stages those rows like caller-supplied features.  Every
+// screening then reads those rows like caller-supplied features.  Every
 // feature is bit-identical to the interpreter's.
 //
 // NVRTC and the driver entry points are resolved with dlopen at first use,

@@ -206,15 +206,15 @@ ScratchOwner g_scr;
 int g_optin = -1;
 int g_sms = -1;
 ShapeOverride g_shape[3];
-// failure-detection self-test, armed by mlt_selftest_walk_timeout: the next
-// full-table V pass makes CTA g_stall_cta wait on a barrier phase that
-// nothing completes, for g_stall_ns (one shot)
 int g_head_levels = kSplitHeadDefault;  // split tables for deep V and P models (0: compact tables)
 long long g_small_max = kSmallMaxN;     // batches up to this size screen in one launch when eligible
 // decoded batches of at least this many candidates use the compiled feature
 // program (0: never); the count of calls that did
 long long g_jit_min_n = kDecodeJitMinN;
 long long g_jit_calls = 0;
+// failure-detection self-test, armed by mlt_selftest_walk_timeout: the next V
+// pass (not over compact tables) makes CTA g_stall_cta wait on a barrier phase
+// that nothing completes, for g_stall_ns (one shot)
 int g_stall_cta = -1;
 unsigned long long g_stall_ns = 0;
 // the same for the next kernel that writes ordinals (mlt_selftest_ordinal_timeout)
@@ -606,7 +606,7 @@ int pack_ensemble(const mlt_node* nodes, int n_trees, int depth, std::vector<uns
   return MLT_OK;
 }
 
-// Ordinal walk of a pass over stored rows: taken where it is expected to save
+// Ordinal walk of a pass over rows: taken where it is expected to save
 // time.  With n_eff candidates to walk it saves, per 32 candidates on an SM, a
 // visit's cycles beyond the ordinal walk's 2.8 (the fp32 walk needs 3.6 and 16
 // shared by the warps whose rows fit beside the tree chunks, one more where a
@@ -799,8 +799,8 @@ int run_screen_with(cudaStream_t st, const float* feats, const DecodeParams* dec
     }
     g_launches += 1;
   }
-  // a small batch of stored features: the whole step in one launch (its
-  // time is recorded as the V phase)
+  // a small batch of rows: the whole step in one launch (its time is recorded as the
+  // V phase)
   if (dec == nullptr && n <= g_small_max) {
     const SmallPlan pl = plan_small(g_F, n, V, P, sm_count(), smem_optin());
     if (pl.threads > 0) {

@@ -137,7 +137,7 @@ constexpr uint32_t kCompactFeatureMask = 0x3FFu;  // bits 0..9
 constexpr uint32_t kCompactChildShift = 10;       // bits 10..29
 constexpr uint32_t kCompactChildMask = 0xFFFFFu;
 
-// Ordinal form of a full or half table (ordinal.cuh has the layout).
+// Ordinal form of a full, half or split table (ordinal.cuh has the layout).
 constexpr int kOrdHead = 6;             // levels of a deep model's tree in shared memory
 constexpr uint32_t kOrdExitLeaf = 0x80000000u;
 constexpr int kOrdBlockBits = 25;       // block index in a tail block's word 0
@@ -191,7 +191,7 @@ struct DeviceModel {
   int head_levels = 0;      // split tables: H
   const unsigned char* tail = nullptr;  // split tables: the tail records
   size_t tail_off = 0;                  // split tables: byte offset of the tail records
-  OrdTable ord;                         // full and half tables: the ordinal form, when there is one
+  OrdTable ord;                         // full, half and split tables: the ordinal form, when there is one
 };
 
 // ---------------------------------------------------------------------------

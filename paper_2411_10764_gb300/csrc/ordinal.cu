@@ -1,6 +1,7 @@
 // Feature ordinals and the ordinal walk (layout and exactness: ordinal.cuh).
-// XGBoost gbtree prediction (Sec. 3, Table 3) for large batches of stored
-// rows: k_ordinals turns the rows into ordinals, k_walk_ord walks them.
+// XGBoost gbtree prediction (Sec. 3, Table 3) over rows, the caller's or those a
+// decoded batch was written to: k_ordinals turns them into ordinals, k_walk_ord
+// walks these.
 #include <algorithm>
 #include <cmath>
 
@@ -473,9 +474,10 @@ __device__ __forceinline__ uint32_t mbar_arrive_pending(uint32_t bar) {
 // ordinals arrive in one bulk copy, the trees in chunks through nbuf buffers
 // (a warp arrives on the buffer's second barrier when it is done with it, and
 // the last one to arrive refills it).  The groups take units of U trees in
-// turn (U = 0: one group, the sum stays in its register).  With Q > 1 a candidate's sum goes from group to group: a warp walks
-// its unit, waits for the sum of the trees before it, adds its leaves in tree
-// order and hands the sum on -- the same sequential fp32 sum as one walker.
+// turn (U = 0: one group, the sum stays in its register).  With Q > 1 a
+// candidate's sum goes from group to group: a warp walks its unit, waits for the
+// sum of the trees before it, adds its leaves in tree order and hands the sum on
+// -- the same sequential fp32 sum as one walker.
 // A warp issues an instruction every other cycle at best, so the groups
 // multiply the warps where a tile's candidates alone leave an SM too few.
 // Bound: shared-memory wavefronts (one per ordinal gather, one to 3.4 per node

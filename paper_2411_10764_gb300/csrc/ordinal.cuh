@@ -1,6 +1,6 @@
-// Ordinal form of a full-table model: every threshold replaced by its place
-// among the model's distinct thresholds of that feature, and every candidate
-// feature by the number of those thresholds it is not below.
+// Ordinal form of a model: every threshold replaced by its place among the
+// model's distinct thresholds of that feature, and every candidate feature by
+// the number of those thresholds it is not below.
 //
 // x >= t_i  <=>  #{distinct t <= x} > i, so a comparison of two small
 // integers decides exactly what the fp32 comparison decides: the walk takes

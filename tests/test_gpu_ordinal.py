@@ -1,6 +1,5 @@
-"""The ordinal walk (large batches of stored rows) against the oracle, bit for
-bit, where it can go wrong: block and tile edges, every depth, odd and even
-feature counts, aligned and unaligned rows, missing values on both default
+"""The ordinal walk against the oracle, bit for bit, where it can go wrong:
+block and tile edges, every depth, odd and even feature counts, aligned and unaligned rows, missing values on both default
 sides, values on and beside the thresholds, infinities, one threshold, a full
 search tree, and the models it must refuse."""
 import numpy as np
