@@ -879,19 +879,21 @@ int noalloc_scratch(int dev, Scratch* out) {
 // walks the rest.  One top-k then ranks all survivors kept.  The result equals
 // screening the consumed prefix of the candidates as a single batch.
 //
-// A group is whole batches, at least one, of up to max(group_rows, a third of
-// what is consumed before it) candidates; a rest of less than half a group (an
-// eighth, beside the first) joins the last, for a group that is skipped costs
-// its launches too.  What V walks past the batch that reaches the target is
-// less than that, and nothing where one batch is as large as a group: it is
-// then screened by itself, without a cut.
+// A group is whole batches, at least one: the first of up to group_rows.first
+// candidates, later ones of about group_rows.later or up to half of what is
+// consumed before them, whichever is more.  A rest of less than half a group (an
+// eighth, beside the first) joins the last, for a group that is skipped costs its
+// launches too.  What V walks past the batch that reaches the target is less than
+// that, and nothing where one batch is as large as a group: it is then screened
+// by itself, without a cut.
 //
 // group_rows: where a group's candidates cost about what any group costs
 // whatever its size.  Up to four warps of candidates an SM cost little beside
 // the chain of one walk and the group's launches; then come the candidates that
-// take 12 us, after the first group 36 (a skipped group costs 5 to 15).
+// take 12 us, after the first group 60 (a group costs about 35 beside its
+// candidates, a skipped one 5 to 15).
 // Measured, us a group of 256 / 19,456 / 58,368 candidates (V, P trees x depth,
-// features), and group_rows of the first group:
+// features), and group_rows.first:
 //     50 x 6, 100 x 6, 32: 21 / 37 / 47; 59,000
 //     200 x 8, 400 x 8, 64: 38 / 66 / 104; 30,000
 //     1,000 x 8, 100 x 6, 64: 52 / 90 / 175; 24,000
@@ -899,7 +901,7 @@ int noalloc_scratch(int dev, Scratch* out) {
 // Groups of 24,576, rounded up and doubled, walked up to three times what was
 // consumed: three batches of 24,576 through the last models, target in the
 // second, 872 us against 643 (one batch at a time: 649).
-constexpr double kGroupFirstUs = 12.0, kGroupLaterUs = 36.0;
+constexpr double kGroupFirstUs = 12.0, kGroupLaterUs = 60.0;
 constexpr long long kGroupMostRows = 1LL << 19;  // bounds the row and ordinal buffers
 
 // Cycles of a pass on an SM for 32 candidates.
@@ -922,11 +924,12 @@ GroupRows group_rows(const DeviceModel& V, const DeviceModel& P, bool decoded) {
 
 // Candidates of the group that starts at candidate `at`.
 long long next_group(long long at, long long n_total, long long batch, const GroupRows& rows) {
-  const long long least = at > 0 ? rows.later : rows.first;
-  const long long most = std::min(std::max(least, at / 3), kGroupMostRows);
+  const long long most = std::min(at > 0 ? std::max(rows.later, at / 2) : rows.first, kGroupMostRows);
   const long long rest = n_total - at;
   if (rest <= most + most / (at > 0 ? 2 : 8)) return rest;
-  return std::min(rest, std::max(1LL, most / batch) * batch);
+  // to the nearest whole batch of rows.later, down from the others
+  const long long room = at > 0 ? std::max(std::min(rows.later + batch / 2, kGroupMostRows), most) : most;
+  return std::min(rest, std::max(1LL, room / batch) * batch);
 }
 
 int run_stream(cudaStream_t st, const float* feats, const DecodeParams* dec0, long long n_total, long long batch,

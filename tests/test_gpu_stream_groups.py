@@ -94,7 +94,7 @@ def _load(vt, vd, pt, pd):
 
 @pytest.mark.parametrize("vt,vd,pt,pd,batch,batches,groups,cuts", [
     (1000, 12, 300, 12, 24576, 4, 4, 0),  # a batch fills the GPU: one a group
-    (1000, 8, 100, 6, 24576, 3, 3, 0),
+    (1000, 8, 100, 6, 32768, 3, 3, 0),
     (1000, 12, 300, 12, 8192, 3, 2, 1),   # two batches, then the third
     (1000, 12, 300, 12, 8192, 5, 2, 2),   # two batches, then three
     (50, 6, 100, 6, 24576, 2, 1, 1),      # cheap walks: both together
