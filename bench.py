@@ -237,8 +237,9 @@ def walk_source_hash() -> str:
 
 
 def dram_traffic(workload: int, phase: str):
-    """DRAM bytes per launch of the phase's walk kernel from the committed
-    ncu capture, or None if there is none or the walk sources changed since."""
+    """DRAM bytes of the phase's kernels (ordinals, walk, and the decoder in a
+    decoded V pass) from the committed ncu capture, or None if there is none
+    or their sources changed since."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as f:
@@ -248,7 +249,7 @@ def dram_traffic(workload: int, phase: str):
     if tr.get("walk_source_hash") != walk_source_hash():
         return None
     ent = tr.get(f"workload{workload}:{phase}")
-    return ent.get("dram_bytes_per_launch") if ent else None
+    return ent.get("dram_bytes") if ent else None
 
 
 def mean_path(ens, x):
