@@ -96,7 +96,7 @@ bool is_capturing(cudaStream_t st) {
 // feature count changes or a V or P model is freed.  A stream capture never
 // grows it (an allocation would end the capture), and a buffer that captured
 // work refers to is set aside instead of freed when a larger one replaces it.
-// An allocation that fails takes the driver 0.24 ms (1,048,576 x 256, whole call
+// An allocation that fails takes CUDA 0.24 ms (1,048,576 x 256, whole call
 // beside a full device: 0.97 -> 1.21 ms), more than a small batch, and a program
 // that keeps the device full would meet it on every call: as large a one is
 // next tried after 16 calls, then 32, at last every 1,024.
