@@ -111,3 +111,23 @@ def test_groups(vt, vd, pt, pd, batch, batches, groups, cuts):
         assert _launches(batches * batch, batch) - one == (groups - 1) * per + cuts
     finally:
         mlt.tune_ordinal(1)
+
+
+@pytest.mark.parametrize("vt,vd,batch", [(400, 12, 24583), (400, 12, 4000), (1500, 8, 24576)])
+@pytest.mark.parametrize("hit", [1, 2, 4])
+def test_deep_models_equal_screening_of_the_prefix(vt, vd, batch, hit):
+    """Groups of one batch and of several, V and P in ordinal form."""
+    import torch
+
+    _load(vt, vd, 60, 12)
+    n = 4 * batch + 11
+    x = torch.rand((n, 64), device="cuda", generator=torch.Generator(device="cuda").manual_seed(batch))
+    _, pf, _ = mlt.screen(x, 0.5, 16)
+    counts = torch.cumsum(torch.isfinite(pf).long(), 0)
+    target = int(counts[hit * batch - 1]) if hit > 1 else 1
+    used = int((counts >= target).nonzero()[0]) // batch * batch + batch
+    pv, pf, tk, stats = mlt.screen_until(x, batch, target, 0.5, 100)
+    wv, wf, wk = mlt.screen(x[:used].contiguous(), 0.5, 100)
+    mlt.sync_status()
+    assert stats.cpu().tolist() == [used, int(counts[used - 1]), used // batch]
+    assert torch.equal(pv[:used], wv) and torch.equal(pf[:used], wf) and torch.equal(tk, wk)
